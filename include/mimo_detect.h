@@ -37,7 +37,13 @@
  *                                              leaves re-scored in FP64, and the
  *                                              algorithmic FP32 flops of the search,
  *                                              sum over branched nodes at row i of
- *                                              2 (n-1-i) + 4 P; may be NULL
+ *                                              2 (n-1-i) + 4 P; may be NULL.
+ *                                              Counts are of the tree in the natural
+ *                                              antenna order; detect_sd without stats, a
+ *                                              node budget or MDX_SEQUENTIAL_SEARCH /
+ *                                              MDX_NO_RESCORE may search the antennas of a
+ *                                              vector in another order, with the same
+ *                                              symbols, metrics and status
  *
  * Streams.  `stream` is a cudaStream_t passed as void* (NULL = the legacy
  * default stream).  Device-pointer calls only enqueue work and return; a
@@ -155,7 +161,7 @@ size_t mdx_workspace_bytes(const mdx_ctx* ctx);
  * ybar = Q^H y, both returned in the real interleaved form of size n = 2 n_tx.
  *   R_out    double [batch][n][n], row-major, zero below the diagonal
  *   ybar_out double [batch][n]
- * Computed in FP64 (complex Householder reflections). */
+ * Complex Householder reflections, to FP64 accuracy or better. */
 mdx_status mdx_qr(mdx_ctx* ctx, int batch, int n_rx, int n_tx, const double* H, const double* y,
                   double* R_out, double* ybar_out, int flags, void* stream);
 

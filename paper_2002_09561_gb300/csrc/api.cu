@@ -31,6 +31,8 @@ struct mdx_ctx {
   unsigned char* sd_vstate = nullptr;
   int* sd_order = nullptr;
   unsigned long long sd_epoch = 0;
+  // sorted antenna order of detect_sd: [sorted x B | perm x B n_tx | place x B n_tx]
+  uint8_t* sd_sorted = nullptr;
   // learned radius model (mdx_mlp_init), null until created
   mdx::MlpState* mlp = nullptr;
   // staging for MDX_HOST_BUFFERS
@@ -146,7 +148,7 @@ void free_all(mdx_ctx* c) {
       if (c->prof_ev[i][k]) cudaEventDestroy(c->prof_ev[i][k]);
   void* ptrs[] = {c->R64, c->yb64, c->R32,  c->yb32, c->singular, c->counter,  c->counts,
                   c->sH,  c->sy,   c->snv,  c->ssym, c->ssym2,    c->smet,     c->svst,
-                  c->sstats, c->sd_shared, c->sd_queue, c->sd_vstate, c->sd_order};
+                  c->sstats, c->sd_shared, c->sd_queue, c->sd_vstate, c->sd_order, c->sd_sorted};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->mx_graph) cudaGraphExecDestroy(c->mx_graph);
@@ -163,6 +165,12 @@ enum Algo { ALGO_SD = 0, ALGO_KBEST = 1, ALGO_HYBRID = 2, ALGO_LINEAR = 3 };
 
 // Task-queue slots of the sphere decoder (tasks exist only while warps are idle).
 constexpr unsigned int kSdQueueSlots = 1u << 16;
+
+// Whether choosing antenna orders can pay (sd_reorder.cu chooses vector by
+// vector): a handful of vectors leaves the GPU idle, and the order's extra QR
+// takes longer than it saves (one 16x16 vector at 18 dB: 119 us a call
+// without, 155 with); trees of fewer than four antennas are small.
+bool reorder_pays(int batch, int n_tx) { return n_tx >= 4 && n_tx <= kReorderMaxTx && batch >= 32; }
 
 mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, const double* H,
                       const double* y, const double* nv, uint8_t* sym, double* met, int32_t* vst,
@@ -339,7 +347,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
   a.metric_out = dmet;
   a.vstatus = dvst;
   a.stats = dstats;
-  e = cudaMemsetAsync(c->counter, 0, sizeof(unsigned int), s);
+  e = cudaMemsetAsync(c->counter, 0, 3 * sizeof(unsigned int), s);
   if (e != cudaSuccess) return cuda_fail(c, e, "work counter reset");
   if (algo == ALGO_SD && (complex_tree || natural)) {
     // complex-tree or natural-order SD: the persistent warp-per-vector kernel on a uniform batch
@@ -394,7 +402,20 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
     e = launch_mixed(m, c->mx_W, 0, c->num_sms, s);
   } else if (algo == ALGO_SD) {
     if (ev) cudaEventRecord(ev[1], s);
-    SdWorkspace w{c->sd_shared, c->sd_queue, kSdQueueSlots, c->sd_vstate, ++c->sd_epoch, c->sd_order};
+    // The antenna order is the search's own business where nothing that the
+    // call returns depends on it (the statistics count the natural tree's nodes)
+    if (!a.stats && a.budget == 0 && !(p->flags & (MDX_SEQUENTIAL_SEARCH | MDX_NO_RESCORE)) &&
+        reorder_pays(batch, M)) {
+      ReorderArgs r{a, c->sd_sorted, c->sd_sorted + batch, c->sd_sorted + (size_t)batch * (1 + M),
+                    c->sd_order, c->counter + 1};
+      e = launch_reorder_select(r, s);
+      if (e == cudaSuccess) e = launch_qr_reorder(r, s);
+      if (e != cudaSuccess) return cuda_fail(c, e, "antenna order");
+      a.sorted = r.sorted;
+      a.place = r.place;
+    }
+    SdWorkspace w{c->sd_shared, c->sd_queue, kSdQueueSlots, c->sd_vstate, ++c->sd_epoch, c->sd_order,
+                  a.sorted != nullptr};
     e = launch_sd(a, w, c->num_sms, s);
   }
   else if (algo == ALGO_KBEST) {
@@ -953,6 +974,7 @@ mdx_status mdx_create(mdx_ctx** out, int device, int max_batch, int max_n_rx, in
   chk(alloc(c, reinterpret_cast<unsigned char**>(&c->sd_queue), sd_task_bytes() * kSdQueueSlots));
   chk(alloc(c, &c->sd_vstate, B * sd_vec_state_bytes(n)));
   chk(alloc(c, &c->sd_order, sd_order_ints(max_batch)));
+  chk(alloc(c, &c->sd_sorted, B * (1 + 2 * (size_t)std::min(max_n_tx, kReorderMaxTx))));
   chk(cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
   chk(cudaEventCreateWithFlags(&c->ev_free, cudaEventDisableTiming));
   for (cudaEvent_t& ev : c->ev_chunk) chk(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));

@@ -65,7 +65,26 @@ struct SearchArgs {
   double* metric_out;
   int32_t* vstatus;
   int64_t* stats;
+  // antenna order of the search (sd_reorder.cu), null: natural.  sorted[v] != 0:
+  // R32 / yb32 of vector v are those of its sorted channel, and antenna j is
+  // column place[v n_tx + j] of it; R64 / yb64 are always the natural ones.
+  const uint8_t* sorted;
+  const uint8_t* place;
 };
+
+// Sorted antenna order of exact sphere decoding: see sd_reorder.cu.
+constexpr int kReorderMaxTx = 32;
+struct ReorderArgs {
+  SearchArgs a;         // the call's R, ybar (overwritten in FP32 for the vectors chosen), radius, sizes
+  uint8_t* sorted;      // [batch]
+  uint8_t* perm;        // [batch][n_tx]: natural column at each place
+  uint8_t* place;       // [batch][n_tx]: place of each natural column
+  int* list;            // [batch]: the vectors chosen, then (from the back) the others
+  unsigned int* count;  // [2], zero on entry: how many of each
+};
+cudaError_t launch_reorder_select(const ReorderArgs& r, cudaStream_t s);
+// QR of the chosen vectors' R with permuted columns (qr.cu).
+cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s);
 
 cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out,
                       cudaStream_t s);
@@ -136,6 +155,7 @@ struct SdWorkspace {
   unsigned char* vstate; // batch x sd_vec_state_bytes(n)
   unsigned long long epoch;  // distinct per launch on this workspace
   int* order;            // batch ints + sd_order_scratch_ints(): the fresh-vector order
+  bool ordered;          // order holds one already
 };
 size_t sd_order_ints(int max_batch);
 size_t sd_shared_bytes();
@@ -203,6 +223,70 @@ constexpr float kU32 = 5.9604645e-8f;
 __device__ __forceinline__ float prune_bound(float r2, float E, int n) {
   if (!(r2 < INFINITY)) return INFINITY;
   return r2 + 4.0f * sqrtf(r2) * E + 4.0f * (float)n * kU32 * r2;
+}
+
+// Initial r^2 of vector v (not a positive number: no radius).
+__device__ __forceinline__ float initial_r2(const SearchArgs& a, int v) {
+  float r2;
+  if (a.radius_mode == RADIUS_NONE) r2 = INFINITY;
+  else if (a.radius_mode == RADIUS_PAPER) r2 = (float)((double)a.n_rx * a.n_tx * a.noise_var[v]);
+  else if (a.radius_mode == RADIUS_PER_VECTOR) r2 = a.r2_vec[v];
+  else r2 = (float)a.radius_value;
+  return r2 > 0.0f ? r2 : INFINITY;
+}
+
+// Path index of natural real row j (place: the vector's antenna places, or null).
+__device__ __forceinline__ int path_at(const uint8_t* place, int j) {
+  return place ? 2 * place[j >> 1] + (j & 1) : j;
+}
+
+// Whether the natural-order search's first sphere (initial r^2 = r0) holds
+// none of the leaves px[0 .. np - 1] (sorted path indices, kept when within
+// FP32 error of the best, whose metric is best): the leaves' FP32 partial
+// distances on the natural R by that search's own FMA chains against its own
+// pruning bound, so that the vector's status does not depend on the antenna
+// order.  By G lanes (gl: lane of the group, gmask: its mask).
+template <int G, typename Path>
+__device__ bool first_sphere_empty(const SearchArgs& a, int v, const uint8_t* place, double best, int np, Path path,
+                                   int gl, unsigned gmask) {
+  const float r0 = initial_r2(a, v);
+  if (!(r0 < INFINITY) || best < 0.999 * (double)r0) return false;
+  const int n = a.n, P = a.P;
+  const double* R64 = a.R64 + (size_t)v * tri_stride64(n);
+  const double* y64 = a.yb64 + (size_t)v * vec_stride64(n);
+  const float alpha = a.alpha, amax = alpha * (float)(P - 1);
+  float e2 = 0.0f;
+  for (int r = gl; r < n; r += G) {
+    float T = fabsf((float)y64[r]);
+    for (int j = r; j < n; ++j) T += amax * fabsf((float)R64[col_off(j) + r]);
+    const float w = (float)(n - r + 1) * T;
+    e2 += w * w;
+  }
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) e2 += __shfl_xor_sync(gmask, e2, o, G);
+  const float bnd = prune_bound(r0, sqrtf(e2) * kU32, n);
+  for (int q = 0; q < np; ++q) {
+    float ped = 0.0f;
+    for (int r0w = (n - 1) / G * G; r0w >= 0; r0w -= G) {
+      const int r = r0w + gl;
+      float d = 0.0f;
+      if (r < n) {
+        float z = (float)y64[r];
+        for (int j = n - 1; j >= r; --j) {
+          const int k = path(q, path_at(place, j));
+          if (k < 0) break;
+          z = fmaf(-(float)R64[col_off(j) + r], fmaf((float)k, 2.0f, -((float)P - 1.0f)) * alpha, z);
+        }
+        d = z;
+      }
+      for (int t = G - 1; t >= 0; --t) {
+        const float dt = __shfl_sync(gmask, d, t, G);
+        if (r0w + t < n) ped = fmaf(dt, dt, ped);
+      }
+    }
+    if (path(q, 0) >= 0 && ped < bnd) return false;
+  }
+  return true;
 }
 
 // Warp-wide minimum of 64-bit keys (every lane gets it): the high words are

@@ -17,6 +17,7 @@
 // 2.15 ms, 4,000 100x100 31.5 -> 10.5 ms; error of R against 64 bits 2.5e-15
 // -> 1.9e-15 (64x64, of which the reference's own is most).
 #include <algorithm>
+#include <type_traits>
 
 #include "fx64.cuh"
 #include "mdx_internal.cuh"
@@ -40,6 +41,9 @@ struct QrDst {
   double* Rdense;
   double* ybdense;
   int* singular;
+  // a re-factored R (SrcR): only R32 and yb32 are written, and where the
+  // matrix needs the FP64 form the natural ones are restored and *sorted cleared
+  uint8_t* sorted = nullptr;
 };
 
 // Phase fix and output of a factorised [R | ybar]: row k of R and ybar_k are
@@ -412,6 +416,32 @@ struct QsSweep<L, SL, SL> {
                                              int, bool, int, const QrDst&) {}
 };
 
+// The matrix [H | y] to factor: entry (row r, column j), y being column M.
+struct SrcH {  // row-major channel and received vector
+  const longlong2* H;
+  const longlong2* y;
+  int M;
+  __device__ __forceinline__ longlong2 operator()(int r, int j) const {
+    return j < M ? H[(size_t)r * M + j] : y[r];
+  }
+};
+struct SrcR {  // a factored R (real interleaved, column-packed) with its antennas permuted, and ybar
+  const i64* R;
+  const i64* y;
+  const uint8_t* perm;
+  int M;
+  __device__ __forceinline__ longlong2 operator()(int r, int j) const {
+    if (j == M) return make_longlong2(y[2 * r], y[2 * r + 1]);
+    const int c = perm[j];
+    const i64* at = R + col_off(2 * c) + 2 * r;
+    return make_longlong2(r <= c ? at[0] : 0, r < c ? at[1] : 0);
+  }
+  __device__ void restore(const QrDst& out, int t0, int step) const {
+    for (int t = t0; t < tri(2 * M); t += step) out.R32[t] = f32_of((u64)R[t]);
+    for (int t = t0; t < 2 * M; t += step) out.yb32[t] = f32_of((u64)y[t]);
+  }
+};
+
 // A matrix left to the FP64 form is marked by -1 in its singular flag or,
 // without one (mdx_qr), in the entry of the dense R below its first diagonal
 // entry (zero in every finished R).
@@ -426,13 +456,11 @@ __device__ __forceinline__ bool is_redo(const QrDst& out, int n) {
   return out.singular ? *out.singular == -1 : reinterpret_cast<const i64*>(out.Rdense)[n] == kRedo;
 }
 
-// Factorises the [H | y] of this lane group (act: the group has a matrix), or
-// marks it for the FP64 form.  Hb:
-// row-major N x M complex, yv: N complex.  Every lane of the warp calls this
+// Factorises the matrix of this lane group (act: the group has one), or marks
+// it for the FP64 form.  Every lane of the warp calls this
 // with the same N, M (shuffles inside).
-template <int L, int SL>
-__device__ void qr_small_pair(int N, int M, bool act, const longlong2* __restrict__ Hb,
-                              const longlong2* __restrict__ yv, const QrDst& out, int4* U) {
+template <int L, int SL, typename Src>
+__device__ void qr_small_pair(int N, int M, bool act, const Src& src, const QrDst& out, int4* U) {
   constexpr int mats = 32 / L;
   const int lane = threadIdx.x & 31, m = lane / L, h = lane % L;
   const int n = 2 * M;
@@ -448,7 +476,7 @@ __device__ void qr_small_pair(int N, int M, bool act, const longlong2* __restric
     for (int q = 0; q < SL; ++q) {
       const int r = L * q + h;
       longlong2 z = make_longlong2(0, 0);
-      if (act && r < N) z = (j < M) ? Hb[(size_t)r * M + j] : yv[r];
+      if (act && r < N) z = src(r, j);
       ar[q] = z.x;
       ai[q] = z.y;
       ex = max(ex, max(ex_of((u64)z.x), ex_of((u64)z.y)));
@@ -514,7 +542,14 @@ __device__ void qr_small_pair(int N, int M, bool act, const longlong2* __restric
         if (t / n > t % n) out.Rdense[t] = 0.0;
   }
   __syncwarp();
-  if (act && h == 0) mark_redo(out, n, bad);
+  if (act && out.sorted) {
+    if constexpr (std::is_same<Src, SrcR>::value) {
+      if (bad) src.restore(out, h, L);
+    }
+    if (bad && h == 0) *out.sorted = 0;
+  } else if (act && h == 0) {
+    mark_redo(out, n, bad);
+  }
 }
 
 // Outputs of matrix b of a uniform batch (stride the library's per-vector layout).
@@ -560,8 +595,31 @@ __global__ void __launch_bounds__(32) qr_small_kernel(QrBatch g) {
   const bool act = i < g.count;
   const double *Hb, *yb;
   const QrDst d = g.get(act ? i : 0, Hb, yb);
-  qr_small_pair<L, SL>(g.N, g.M, act, reinterpret_cast<const longlong2*>(Hb),
-                       reinterpret_cast<const longlong2*>(yb), d, reinterpret_cast<int4*>(smem_raw));
+  const SrcH src{reinterpret_cast<const longlong2*>(Hb), reinterpret_cast<const longlong2*>(yb), g.M};
+  qr_small_pair<L, SL>(g.N, g.M, act, src, d, reinterpret_cast<int4*>(smem_raw));
+}
+
+// The chosen vectors' R with their antennas in search order (see sd_reorder.cu).
+__device__ __forceinline__ QrDst reorder_at(const ReorderArgs& g, int i, SrcR& src) {
+  const int v = g.list[i], n = g.a.n, M = g.a.n_tx;
+  src = SrcR{reinterpret_cast<const i64*>(g.a.R64 + (size_t)v * tri_stride64(n)),
+             reinterpret_cast<const i64*>(g.a.yb64 + (size_t)v * vec_stride64(n)), g.perm + (size_t)v * M, M};
+  QrDst d{};
+  d.R32 = const_cast<float*>(g.a.R32) + (size_t)v * tri_stride32(n);
+  d.yb32 = const_cast<float*>(g.a.yb32) + (size_t)v * vec_stride32(n);
+  d.sorted = g.sorted + v;
+  return d;
+}
+template <int L, int SL>
+__global__ void __launch_bounds__(32) qr_reorder_small_kernel(ReorderArgs g, int few) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int count = (int)*g.count, i0 = blockIdx.x * (32 / L);
+  if (count <= few || i0 >= count) return;
+  const int i = i0 + (threadIdx.x & 31) / L;
+  const bool act = i < count;
+  SrcR src;
+  const QrDst d = reorder_at(g, act ? i : i0, src);
+  qr_small_pair<L, SL>(g.a.n_tx, g.a.n_tx, act, src, d, reinterpret_cast<int4*>(smem_raw));
 }
 
 // The matrices that qr_small_kernel left, in FP64.
@@ -649,8 +707,8 @@ __device__ __forceinline__ void qc_update(longlong2* col, const int4* u, int k, 
   }
 }
 
-__device__ void qr_cta_one(int N, int M, const double* __restrict__ Hd, const double* __restrict__ yd,
-                           const QrDst& out) {
+template <typename Src>
+__device__ void qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   QrCtaLayout L;
   L.init(N, M);
@@ -662,11 +720,9 @@ __device__ void qr_cta_one(int N, int M, const double* __restrict__ Hd, const do
   int* es = reinterpret_cast<int*>(smem_raw + L.off_e);
   volatile int* flag = reinterpret_cast<volatile int*>(smem_raw + L.off_flag);
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
-  const longlong2* Hb = reinterpret_cast<const longlong2*>(Hd);
-  const longlong2* yb = reinterpret_cast<const longlong2*>(yd);
   if (tid == 0) *flag = 0;
-  for (int t = tid; t < N * M; t += nthr) A[(size_t)(t % M) * N + t / M] = Hb[t];
-  for (int r = tid; r < N; r += nthr) A[(size_t)M * N + r] = yb[r];
+  for (int t = tid; t < N * M; t += nthr) A[(size_t)(t % M) * N + t / M] = src(t / M, t % M);
+  for (int r = tid; r < N; r += nthr) A[(size_t)M * N + r] = src(r, M);
   __syncthreads();
   // the columns' scales, a warp per column
   for (int c = warp; c <= M; c += nw) {
@@ -741,7 +797,12 @@ __device__ void qr_cta_one(int N, int M, const double* __restrict__ Hd, const do
   const bool redo = *flag != 0;
   __syncthreads();  // every thread has read the flag that qr_one's data overwrites
   if (redo) {
-    qr_one<32>(N, M, reinterpret_cast<const double2*>(Hd), reinterpret_cast<const double2*>(yd), out);
+    if constexpr (std::is_same<Src, SrcH>::value) {
+      qr_one<32>(N, M, reinterpret_cast<const double2*>(src.H), reinterpret_cast<const double2*>(src.y), out);
+    } else {
+      if (tid == 0) *out.sorted = 0;
+      src.restore(out, tid, nthr);
+    }
     return;
   }
   const int n = 2 * M, nb = M * (M + 1) / 2;  // complex entries (a, c) with a <= c
@@ -775,7 +836,15 @@ template <int T, int B>
 __global__ void __launch_bounds__(T, B) qr_cta_kernel(QrBatch g) {
   const double *Hb, *yb;
   const QrDst d = g.get(blockIdx.x, Hb, yb);
-  qr_cta_one(g.N, g.M, Hb, yb, d);
+  const SrcH src{reinterpret_cast<const longlong2*>(Hb), reinterpret_cast<const longlong2*>(yb), g.M};
+  qr_cta_one(g.N, g.M, src, d);
+}
+__global__ void __launch_bounds__(256, 3) qr_reorder_cta_kernel(ReorderArgs g, int few) {
+  const int count = (int)*g.count;
+  if (count > few || (int)blockIdx.x >= count) return;
+  SrcR src;
+  const QrDst d = reorder_at(g, blockIdx.x, src);
+  qr_cta_one(g.a.n_tx, g.a.n_tx, src, d);
 }
 
 size_t qr_smem(int n_rx, int n_tx) {
@@ -827,6 +896,14 @@ int qr_form(int count, int n_rx) {
   return 8;
 }
 
+template <int L, int SL>
+cudaError_t launch_rs(const ReorderArgs& r, int few, cudaStream_t s) {
+  const size_t sm = qs_smem(r.a.n_tx, r.a.n_tx, L);
+  cudaFuncSetAttribute(qr_reorder_small_kernel<L, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_reorder_small_kernel<L, SL><<<(r.a.batch + 32 / L - 1) / (32 / L), 32, sm, s>>>(r, few);
+  return cudaGetLastError();
+}
+
 cudaError_t launch(const QrBatch& g, cudaStream_t s) {
   if (g.count <= 0) return cudaSuccess;
   const int N = g.N;
@@ -860,6 +937,22 @@ cudaError_t launch(const QrBatch& g, cudaStream_t s) {
 }
 
 }  // namespace
+
+// The number of vectors chosen is on the device: the CTA form's grid is for
+// up to `few` of them (as in qr_form), the other's for the whole batch, and
+// the one that does not apply returns at once.
+cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s) {
+  const int M = r.a.n_tx, few = M <= 16 ? 1216 : 1824;
+  const size_t sm = qr_cta_smem(M, M);
+  cudaFuncSetAttribute(qr_reorder_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_reorder_cta_kernel<<<std::min(r.a.batch, few), 32 * std::max(2, std::min(1 + (M + 3) / 4, 5)), sm, s>>>(r, few);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || r.a.batch <= few) return e;
+  if (M <= 8) return launch_rs<4, 2>(r, few, s);
+  if (M <= 16) return launch_rs<8, 2>(r, few, s);
+  if (M <= 24) return launch_rs<4, 6>(r, few, s);
+  return launch_rs<8, 4>(r, few, s);
+}
 
 cudaError_t launch_qr_gather(int count, int n_rx, int n_tx, const int* ids, const MixedReq* reqs,
                              const double* H, const double* y, QrOut out, cudaStream_t s) {

@@ -191,12 +191,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
       }
       __syncwarp();
       const float E0 = error_scale_warp(n, P, alpha, Rc, yb, lane);
-      float r2;
-      if (a.radius_mode == RADIUS_NONE) r2 = INFINITY;
-      else if (a.radius_mode == RADIUS_PAPER) r2 = (float)((double)a.n_rx * a.n_tx * a.noise_var[v]);
-      else if (a.radius_mode == RADIUS_PER_VECTOR) r2 = a.r2_vec[v];
-      else r2 = (float)a.radius_value;
-      if (!(r2 > 0.0f)) r2 = INFINITY;
+      const float r2 = initial_r2(a, v);
       if (lane == 0) {
         vs->r2bits = __float_as_uint(r2);
         vs->pending = 1;
@@ -605,6 +600,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
       const double* y64 = a.yb64 + (size_t)v * vec_stride64(n);
       // candidates are read through L2 (other warps wrote them) into this
       // warp's path buffer; the winner's indices are kept in registers
+      const uint8_t* place = a.sorted && a.sorted[v] ? a.place + (size_t)v * a.n_tx : nullptr;
       int win = -1;
       double win_m = INFINITY;
       long long rescored = 0;
@@ -613,7 +609,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
         if (!(vv->cand_ped[q] <= keep)) continue;
         const uint8_t* cx = cand_path(vs, q, n);
         __syncwarp();
-        for (int r = lane; r < n; r += 32) xs[r] = __ldcg(cx + r);
+        for (int r = lane; r < n; r += 32) xs[r] = __ldcg(cx + path_at(place, r));  // natural order
         __syncwarp();
         double m;
         if (a.flags & MDX_NO_RESCORE) {
@@ -627,7 +623,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
           // tie: lexicographically smaller index vector, top row first
           const uint8_t* wx = cand_path(vs, win, n);
           for (int j = n - 1; j >= 0; --j) {
-            const uint8_t w1 = xs[j], w2 = __ldcg(wx + j);
+            const uint8_t w1 = xs[j], w2 = __ldcg(wx + path_at(place, j));
             if (w1 != w2) {
               better = w1 < w2;
               break;
@@ -653,9 +649,17 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
         if (j < a.n_tx)
           a.sym_out[(size_t)v * a.n_tx + j] = win >= 0 ? (uint8_t)(wsym[2 * t] * P + wsym[2 * t + 1]) : 0;
       }
+      bool empty = rs > 0;
+      if (place && win >= 0) {
+        // the status of the natural order's first sphere
+        auto path = [&](int q, int at) {
+          return vv->cand_ped[q] <= keep ? (int)__ldcg(cand_path(vs, q, n) + at) : -1;
+        };
+        empty = first_sphere_empty<32>(a, v, place, win_m, nc, path, lane, 0xffffffffu);
+      }
       if (lane == 0) {
         a.metric_out[v] = (win >= 0) ? win_m : (double)INFINITY;
-        a.vstatus[v] = bh ? MDX_V_BUDGET_EXCEEDED : (vv->restarts > 0 ? MDX_V_EMPTY_RETRIED : MDX_V_OK);
+        a.vstatus[v] = bh ? MDX_V_BUDGET_EXCEEDED : (empty ? MDX_V_EMPTY_RETRIED : MDX_V_OK);
         if (a.stats) {
           a.stats[(size_t)v * kStats + 0] = (long long)vv->nodes;
           a.stats[(size_t)v * kStats + 1] = (long long)vv->peds;
@@ -755,7 +759,9 @@ cudaError_t launch_sd(const SearchArgs& a, const SdWorkspace& w, int num_sms, cu
   g.order = nullptr;
   cudaError_t e = cudaMemsetAsync(w.shared, 0, sizeof(SdShared), s);
   if (e != cudaSuccess) return e;
-  if (a.noise_var && w.order && a.batch > 1) {
+  if (w.ordered) {
+    g.order = w.order;
+  } else if (a.noise_var && w.order && a.batch > 1) {
     int* order = w.order;
     unsigned int* cnt = reinterpret_cast<unsigned int*>(order + a.batch);
     e = cudaMemsetAsync(cnt, 0, sizeof(unsigned int) * kOrderBuckets, s);

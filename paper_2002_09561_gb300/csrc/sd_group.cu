@@ -161,12 +161,13 @@ __host__ __device__ constexpr size_t group_cta_bytes() {
   return (size_t)group_warps<G>() * WarpLayout<G>::WORDS * 4 + 8 * sizeof(double);
 }
 
-// FP64 ||ybar - R x||^2 of path x (n <= 32) by the G lanes of a group: lane
+// FP64 ||ybar - R x||^2 of path x (n <= 32; place: its antennas' places, or
+// null) by the G lanes of a group: lane
 // g accumulates rows g, g + G, ...; the PAM levels come from a table.
 template <int G>
 __device__ __forceinline__ double rescore_fp64_group(int n, const double* lev64, const double* __restrict__ R64,
                                                      const double* __restrict__ y64, const uint8_t* x, bool x_global,
-                                                     int gl, unsigned gmask) {
+                                                     const uint8_t* place, int gl, unsigned gmask) {
   constexpr int RPL = kGroupN / G;
   double rr[RPL];
 #pragma unroll
@@ -175,7 +176,8 @@ __device__ __forceinline__ double rescore_fp64_group(int n, const double* lev64,
     rr[t] = (r < n) ? y64[r] : 0.0;
   }
   for (int j = 0; j < n; ++j) {
-    const int k = x_global ? (int)__ldcg(x + j) : (int)x[j];
+    const int at = path_at(place, j);
+    const int k = x_global ? (int)__ldcg(x + at) : (int)x[at];
     const double xj = lev64[k];
     const double* col = R64 + col_off(j);
 #pragma unroll
@@ -627,6 +629,7 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
           const float keep = prune_bound(best, E, n);
           const double* R64 = a.R64 + (size_t)v * tri_stride64(n);
           const double* y64 = a.yb64 + (size_t)v * vec_stride64(n);
+          const uint8_t* place = a.sorted && a.sorted[v] ? a.place + (size_t)v * a.n_tx : nullptr;
           int win = -1;
           double win_m = INFINITY;
           long long rescored = 0;
@@ -638,7 +641,7 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
             if (a.flags & MDX_NO_RESCORE) {
               m = (double)cp;
             } else {
-              m = rescore_fp64_group<G>(n, lev64, R64, y64, px, use_global, gl, gmask);
+              m = rescore_fp64_group<G>(n, lev64, R64, y64, px, use_global, place, gl, gmask);
               ++rescored;
             }
             bool better = m < win_m;
@@ -646,8 +649,9 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
               // tie: lexicographically smaller index vector, top row first
               const uint8_t* wx = use_global ? cand_path(vs, win, n) : cx + win * kGroupN;
               for (int j = n - 1; j >= 0; --j) {
-                const uint8_t w1 = use_global ? __ldcg(px + j) : px[j];
-                const uint8_t w2 = use_global ? __ldcg(wx + j) : wx[j];
+                const int at = path_at(place, j);
+                const uint8_t w1 = use_global ? __ldcg(px + at) : px[at];
+                const uint8_t w2 = use_global ? __ldcg(wx + at) : wx[at];
                 if (w1 != w2) {
                   better = w1 < w2;
                   break;
@@ -663,15 +667,25 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
           for (int j = gl; j < a.n_tx; j += G) {
             uint8_t q = 0;
             if (wx) {
-              const int kre = use_global ? __ldcg(wx + 2 * j) : wx[2 * j];
-              const int kim = use_global ? __ldcg(wx + 2 * j + 1) : wx[2 * j + 1];
+              const int at = path_at(place, 2 * j);
+              const int kre = use_global ? __ldcg(wx + at) : wx[at];
+              const int kim = use_global ? __ldcg(wx + at + 1) : wx[at + 1];
               q = (uint8_t)(kre * P + kim);
             }
             a.sym_out[(size_t)v * a.n_tx + j] = q;
           }
+          int rs = use_global ? vv->restarts : restarts;
+          if (place && win >= 0) {
+            // the status of the natural order's first sphere
+            auto path = [&](int q, int at) {
+              const float cp = use_global ? vv->cand_ped[q] : cped[q];
+              if (!(cp <= keep)) return -1;
+              return use_global ? (int)__ldcg(cand_path(vs, q, n) + at) : (int)cx[q * kGroupN + at];
+            };
+            rs = first_sphere_empty<G>(a, v, place, win_m, nc, path, gl, gmask) ? 1 : 0;
+          }
           if (gl == 0) {
             a.metric_out[v] = (win >= 0) ? win_m : (double)INFINITY;
-            const int rs = use_global ? vv->restarts : restarts;
             a.vstatus[v] = budget_hit ? MDX_V_BUDGET_EXCEEDED : (rs > 0 ? MDX_V_EMPTY_RETRIED : MDX_V_OK);
             if (a.stats) {
               // vs holds the counts committed under a node budget and those of
@@ -800,12 +814,7 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
 #pragma unroll
             for (int o = G / 2; o > 0; o >>= 1) e2 += __shfl_xor_sync(gmask, e2, o, G);
             E = sqrtf(e2) * kU32;
-            float rr;
-            if (a.radius_mode == RADIUS_NONE) rr = INFINITY;
-            else if (a.radius_mode == RADIUS_PAPER) rr = (float)((double)a.n_rx * a.n_tx * a.noise_var[v]);
-            else if (a.radius_mode == RADIUS_PER_VECTOR) rr = a.r2_vec[v];
-            else rr = (float)a.radius_value;
-            if (!(rr > 0.0f)) rr = INFINITY;
+            const float rr = initial_r2(a, v);
             r2 = rr;
             r2_start = rr;
             restarts = 0;
