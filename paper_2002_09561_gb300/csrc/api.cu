@@ -423,7 +423,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
     e = launch_kbest(a, c->num_sms, s);
   } else if (algo == ALGO_LINEAR) {
     if (ev) cudaEventRecord(ev[1], s);
-    e = launch_linear(a, mmse, c->num_sms, s);
+    e = launch_linear(AugArgs{a, c->sd_vstate, sd_vec_state_bytes(n), c->sd_order}, mmse, c->num_sms, s);
   } else {
     if (ev) cudaEventRecord(ev[1], s);
     e = launch_hybrid(a, c->num_sms, s);

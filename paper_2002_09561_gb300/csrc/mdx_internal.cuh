@@ -86,6 +86,24 @@ cudaError_t launch_reorder_select(const ReorderArgs& r, cudaStream_t s);
 // QR of the chosen vectors' R with permuted columns (qr.cu).
 cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s);
 
+// MMSE's augmented systems [R; sigma I] x = [ybar; 0], factored into the space
+// of the FP32 R (the triangle as complex FP64 numbers: above the diagonal, then
+// the diagonal, 8 n_tx^2 bytes of 8 n_tx^2 + 4 n_tx) and of the sphere
+// decoder's per-vector state (Q^H y).
+constexpr int kAugMaxTx = 32;
+struct AugArgs {
+  SearchArgs a;
+  unsigned char* space;  // per-vector state, stride bytes each (at least 16 n_tx)
+  size_t stride;
+  int* bad;              // [batch]: 1 where the general form has to solve the vector
+  __host__ __device__ double* R(int v) const {
+    return reinterpret_cast<double*>(const_cast<float*>(a.R32) + (size_t)v * tri_stride32(a.n));
+  }
+  __host__ __device__ double* diag(int v) const { return R(v) + (size_t)a.n_tx * (a.n_tx - 1); }
+  __host__ __device__ double* y(int v) const { return reinterpret_cast<double*>(space + (size_t)v * stride); }
+};
+cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s);
+
 cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out,
                       cudaStream_t s);
 
@@ -170,7 +188,7 @@ size_t kbest_smem_bytes(int n, int K, int P, bool complex_tree);
 cudaError_t launch_hybrid(const SearchArgs& a, int num_sms, cudaStream_t s);
 // Linear detectors (linear.cu): ZF or MMSE on the QR workspace.
 size_t linear_smem_bytes(int n, bool mmse);
-cudaError_t launch_linear(const SearchArgs& a, bool mmse, int num_sms, cudaStream_t s);
+cudaError_t launch_linear(const AugArgs& g, bool mmse, int num_sms, cudaStream_t s);
 // Shared memory the hybrid needs for (n, K, P, depth), or (size_t)-1 if it does not fit.
 size_t hybrid_smem_bytes(int n, int K, int P, int depth);
 // Learned radius model (mlp.cu).  Systems with n_tx <= kFullFeaturesMaxTx use

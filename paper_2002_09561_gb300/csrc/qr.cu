@@ -44,6 +44,12 @@ struct QrDst {
   // a re-factored R (SrcR): only R32 and yb32 are written, and where the
   // matrix needs the FP64 form the natural ones are restored and *sorted cleared
   uint8_t* sorted = nullptr;
+  // the augmented system of MMSE (SrcAug): R above the diagonal as complex
+  // numbers, column c at c (c - 1) / 2, its diagonal, Q^H y, and the mark
+  longlong2* pk = nullptr;
+  i64* pk_diag = nullptr;
+  longlong2* pk_y = nullptr;
+  int* pk_bad = nullptr;
 };
 
 // Phase fix and output of a factorised [R | ybar]: row k of R and ybar_k are
@@ -225,6 +231,13 @@ __device__ __forceinline__ float f32_of(u64 bits) {
   return (float)__longlong_as_double((i64)bits);
 }
 __device__ __forceinline__ void put_r(const QrDst& out, int n, int k, int c, u64 re, u64 im) {
+  if (out.pk) {
+    if (k == c)
+      out.pk_diag[c] = (i64)re;
+    else
+      out.pk[c * (c - 1) / 2 + k] = make_longlong2((i64)re, (i64)im);
+    return;
+  }
   const int o0 = col_off(2 * c) + 2 * k, o1 = col_off(2 * c + 1) + 2 * k;
   const bool diag = k == c;  // the block's entry below the diagonal is not stored
   const u64 nim = im ? im ^ kSignBit : im;
@@ -251,6 +264,10 @@ __device__ __forceinline__ void put_r(const QrDst& out, int n, int k, int c, u64
   }
 }
 __device__ __forceinline__ void put_y(const QrDst& out, int k, u64 re, u64 im) {
+  if (out.pk) {
+    out.pk_y[k] = make_longlong2((i64)re, (i64)im);
+    return;
+  }
   if (out.yb64) {
     reinterpret_cast<i64*>(out.yb64)[2 * k] = (i64)re;
     reinterpret_cast<i64*>(out.yb64)[2 * k + 1] = (i64)im;
@@ -442,6 +459,19 @@ struct SrcR {  // a factored R (real interleaved, column-packed) with its antenn
   }
 };
 
+struct SrcAug {  // [R; sigma I] and [ybar; 0] of a factored R: the regularised least squares of MMSE
+  const i64* R;
+  const i64* y;
+  i64 sigma;
+  int M;
+  __device__ __forceinline__ longlong2 operator()(int r, int j) const {
+    if (r >= M) return make_longlong2(r - M == j ? sigma : 0, 0);
+    if (j == M) return make_longlong2(y[2 * r], y[2 * r + 1]);
+    const i64* at = R + col_off(2 * j) + 2 * r;
+    return make_longlong2(r <= j ? at[0] : 0, r < j ? at[1] : 0);
+  }
+};
+
 // A matrix left to the FP64 form is marked by -1 in its singular flag or,
 // without one (mdx_qr), in the entry of the dense R below its first diagonal
 // entry (zero in every finished R).
@@ -542,7 +572,9 @@ __device__ void qr_small_pair(int N, int M, bool act, const Src& src, const QrDs
         if (t / n > t % n) out.Rdense[t] = 0.0;
   }
   __syncwarp();
-  if (act && out.sorted) {
+  if (act && out.pk) {
+    if (h == 0) *out.pk_bad = bad ? 1 : 0;
+  } else if (act && out.sorted) {
     if constexpr (std::is_same<Src, SrcR>::value) {
       if (bad) src.restore(out, h, L);
     }
@@ -799,12 +831,15 @@ __device__ void qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
   if (redo) {
     if constexpr (std::is_same<Src, SrcH>::value) {
       qr_one<32>(N, M, reinterpret_cast<const double2*>(src.H), reinterpret_cast<const double2*>(src.y), out);
-    } else {
+    } else if constexpr (std::is_same<Src, SrcR>::value) {
       if (tid == 0) *out.sorted = 0;
       src.restore(out, tid, nthr);
+    } else {
+      if (tid == 0) *out.pk_bad = 1;
     }
     return;
   }
+  if (tid == 0 && out.pk) *out.pk_bad = 0;
   const int n = 2 * M, nb = M * (M + 1) / 2;  // complex entries (a, c) with a <= c
   for (int t = tid; t < nb; t += nthr) {
     int c = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // exact after the corrections below
@@ -845,6 +880,34 @@ __global__ void __launch_bounds__(256, 3) qr_reorder_cta_kernel(ReorderArgs g, i
   SrcR src;
   const QrDst d = reorder_at(g, blockIdx.x, src);
   qr_cta_one(g.a.n_tx, g.a.n_tx, src, d);
+}
+
+// The augmented systems of a batch (2 M x M, see linear.cu).
+__device__ __forceinline__ QrDst aug_at(const AugArgs& g, int v, SrcAug& src) {
+  const int n = g.a.n, M = g.a.n_tx;
+  src = SrcAug{reinterpret_cast<const i64*>(g.a.R64 + (size_t)v * tri_stride64(n)),
+               reinterpret_cast<const i64*>(g.a.yb64 + (size_t)v * vec_stride64(n)),
+               __double_as_longlong(sqrt(g.a.noise_var[v])), M};
+  QrDst d{};
+  d.pk = reinterpret_cast<longlong2*>(g.R(v));
+  d.pk_diag = reinterpret_cast<i64*>(g.diag(v));
+  d.pk_y = reinterpret_cast<longlong2*>(g.y(v));
+  d.pk_bad = g.bad + v;
+  return d;
+}
+template <int L, int SL>
+__global__ void __launch_bounds__(32) qr_aug_small_kernel(AugArgs g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int i = blockIdx.x * (32 / L) + (threadIdx.x & 31) / L;
+  const bool act = i < g.a.batch;
+  SrcAug src;
+  const QrDst d = aug_at(g, act ? i : 0, src);
+  qr_small_pair<L, SL>(2 * g.a.n_tx, g.a.n_tx, act, src, d, reinterpret_cast<int4*>(smem_raw));
+}
+__global__ void __launch_bounds__(256, 3) qr_aug_cta_kernel(AugArgs g) {
+  SrcAug src;
+  const QrDst d = aug_at(g, blockIdx.x, src);
+  qr_cta_one(2 * g.a.n_tx, g.a.n_tx, src, d);
 }
 
 size_t qr_smem(int n_rx, int n_tx) {
@@ -894,6 +957,14 @@ int qr_form(int count, int n_rx) {
   if (n_rx <= 12) return count <= 9728 ? 8 : 4;
   if (n_rx > 16 && n_rx <= 24) return count <= 4864 ? 8 : 4;
   return 8;
+}
+
+template <int L, int SL>
+cudaError_t launch_as(const AugArgs& g, cudaStream_t s) {
+  const size_t sm = qs_smem(2 * g.a.n_tx, g.a.n_tx, L);
+  cudaFuncSetAttribute(qr_aug_small_kernel<L, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_aug_small_kernel<L, SL><<<(g.a.batch + 32 / L - 1) / (32 / L), 32, sm, s>>>(g);
+  return cudaGetLastError();
 }
 
 template <int L, int SL>
@@ -952,6 +1023,28 @@ cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s) {
   if (M <= 16) return launch_rs<8, 2>(r, few, s);
   if (M <= 24) return launch_rs<4, 6>(r, few, s);
   return launch_rs<8, 4>(r, few, s);
+}
+
+cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s) {
+  const int M = g.a.n_tx;
+  switch (qr_form(g.a.batch, 2 * M)) {
+    case 0: {
+      const size_t sm = qr_cta_smem(2 * M, M);
+      cudaFuncSetAttribute(qr_aug_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      qr_aug_cta_kernel<<<g.a.batch, 32 * std::max(2, std::min(1 + (M + 3) / 4, g.a.batch > 608 ? 5 : 8)), sm, s>>>(g);
+      return cudaGetLastError();
+    }
+    case 2:
+      if (M <= 2) return launch_as<2, 2>(g, s);
+      return launch_as<2, 4>(g, s);
+    case 4:
+      if (M <= 4) return launch_as<4, 2>(g, s);
+      if (M <= 8) return launch_as<4, 4>(g, s);
+      return launch_as<4, 6>(g, s);
+    default:
+      if (M <= 8) return launch_as<8, 2>(g, s);
+      return launch_as<8, 4>(g, s);
+  }
 }
 
 cudaError_t launch_qr_gather(int count, int n_rx, int n_tx, const int* ids, const MixedReq* reqs,
