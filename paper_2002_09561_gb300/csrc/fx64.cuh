@@ -11,11 +11,12 @@
 // dropped).  A real multiply-add costs 7.5 cycles instead of 77, at a rounding
 // error of about 2^-58 of the column's norm against 2^-53 in FP64.
 //
-// A number x in [-2, 2] is the integer x 2^58 = h 2^29 + l with 0 <= l < 2^29
-// (|h| <= 2^30).  A sum of products is kept as two 64-bit accumulators,
+// A number x in [-2, 2] is the integer x 2^58 = h 2^29 + l with -2^28 <= l <
+// 2^28 (|h| <= 2^30; signed low limbs, so that the dropped products average to
+// zero and 0 stays exactly 0).  A sum of products is kept as two 64-bit accumulators,
 // hh = sum h h' (units) and md = sum h l' + l h' (units 2^-29): for vectors u
 // of norm sqrt(2) and a of norm 1 with m real entries, |md| is below
-// sqrt(m) 2^60 (Cauchy-Schwarz on the high limbs), so up to 64 entries per
+// sqrt(m) 2^59 (Cauchy-Schwarz on the high limbs), so up to 256 entries per
 // accumulator cannot overflow.
 #pragma once
 
@@ -30,14 +31,13 @@ typedef unsigned long long u64;
 
 constexpr int kFxBits = 58;   // fraction bits
 constexpr int kFxLimb = 29;   // bits of the low limb
-constexpr int kFxMask = (1 << kFxLimb) - 1;
 constexpr i64 kFxHalf = 1ll << (kFxLimb - 1);  // rounds md to the nearest unit
 
-__host__ __device__ __forceinline__ int fx_hi(i64 a) { return (int)(a >> kFxLimb); }
-__host__ __device__ __forceinline__ int fx_lo(i64 a) { return (int)a & kFxMask; }
-// a b and c + a b as one wide multiply(-add).  (Written out: from the C
-// expression the compiler widens the low limbs, known not to be negative, with
-// zeros and then multiplies in 64 bits, three instructions for one.)
+__host__ __device__ __forceinline__ int fx_lo(i64 a) { return (int)((unsigned)a << (32 - kFxLimb)) >> (32 - kFxLimb); }
+__host__ __device__ __forceinline__ int fx_hi(i64 a) { return (int)(a >> kFxLimb) + (int)((unsigned)fx_lo(a) >> 31); }
+// a b and c + a b as one wide multiply(-add).  (Written out: where the
+// compiler can tell a limb's sign it may widen it with zeros and multiply in 64
+// bits, three instructions for one.)
 __host__ __device__ __forceinline__ i64 wide(int a, int b) {
 #ifdef __CUDA_ARCH__
   i64 r;

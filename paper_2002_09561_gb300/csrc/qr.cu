@@ -8,7 +8,7 @@
 // (qr_cta_kernel).  The few matrices that a fixed scale per column does not
 // suit (a residual column below 2^-26 of its norm: singular or nearly so;
 // infinities, NaN and exponents near the ends of the range) are factored by
-// the FP64 form (qr_one).  The complex R is written out in the real
+// the FP64 forms (qr64_one).  The complex R is written out in the real
 // interleaved form (entry r_ab -> [[Re,-Im],[Im,Re]]) that the tree search
 // uses.
 //
@@ -282,18 +282,204 @@ __device__ __forceinline__ void put_y(const QrDst& out, int k, u64 re, u64 im) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// The FP64 form of a small system (n_rx <= 32): one matrix by one warp, column
+// by column in the left-looking order, lane h < L holding rows L q + h of the
+// current column (the other lanes run along on zeros).  V, Tau: qs_vo(M, N)
+// reflector entries and M scalars of shared memory.
+__host__ __device__ inline int qs_vo(int k, int N) { return k * N - k * (k - 1) / 2; }  // first entry of v_k
+// Conversions between a positive normal double in [1e-30, 1e30] and a float
+// estimate of it, done on the integer pipe (rebias the exponent, keep the top
+// 23 fraction bits): an FP64 conversion would occupy the FP64 unit.
+__device__ __forceinline__ float f32_estimate(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = ((hi >> 20) & 0x7ffu) - 1023u + 127u;
+  return __uint_as_float((e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double f64_of(float f) {
+  const unsigned b = __float_as_uint(f);
+  const unsigned e = ((b >> 23) & 0xffu) - 127u + 1023u;
+  return __hiloint2double((int)((e << 20) | ((b & 0x7fffffu) >> 3)), (int)((b & 7u) << 29));
+}
+
+// 1 / sqrt(x) for a positive x: a single-precision estimate y0 (relative
+// error below 2^-21) refined by one third-order step of the binomial series
+// (1 - e)^(-1/2) = 1 + e/2 + 3e^2/8 + O(e^3), e = 1 - x y0^2 (error below
+// 2^-60 before rounding).
+__device__ __forceinline__ double rsqrt64(double x) {
+  if (!(x > 1e-30 && x < 1e30)) return 1.0 / sqrt(x);
+  const double y = f64_of(rsqrtf(f32_estimate(x)));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y, e * fma(0.375, e, 0.5), y);
+}
+// 1 / d for a positive d: single-precision estimate refined by one
+// third-order step of 1 / (1 - e) = 1 + e + e^2 + O(e^3), e = 1 - d y0.
+__device__ __forceinline__ double rcp64(double d) {
+  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
+  const double y = f64_of(__frcp_rn(f32_estimate(d)));
+  const double e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+template <int L>
+__device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, const double2* __restrict__ yv,
+                               const QrDst& out, double2* V, double* Tau) {
+  constexpr int kQsSlots = 8;  // rows per lane (N <= 8 L)
+  const int lane = threadIdx.x & 31, h = lane % L;
+  const bool act = lane < L;
+  const int n = 2 * M;
+  double2 a[kQsSlots], ph[kQsSlots];
+#pragma unroll
+  for (int q = 0; q < kQsSlots; ++q) ph[q] = make_double2(1.0, 0.0);
+  int sing = 0;
+  for (int j = 0; j <= M; ++j) {
+#pragma unroll
+    for (int q = 0; q < kQsSlots; ++q) {
+      const int r = L * q + h;
+      a[q] = make_double2(0.0, 0.0);
+      if (act && r < N) a[q] = (j < M) ? Hb[(size_t)r * M + j] : yv[r];
+    }
+    // reflectors 0 .. j-1: a <- a - v_k tau_k (v_k^H a) over rows k..N-1
+    const int kend = j < M ? j : M;
+    for (int k = 0; k < kend; ++k) {
+      const double2* vk = V + (size_t)(qs_vo(k, N) - k);  // entry r at vk[r]
+      double wr = 0.0, wi = 0.0;
+#pragma unroll
+      for (int q = 0; q < kQsSlots; ++q) {
+        const int r = L * q + h;
+        if (L * q + L - 1 < k || L * q >= N) continue;  // no lane of the group has this row
+        if (r >= k && r < N) {
+          const double2 v = vk[r];
+          wr = fma(v.x, a[q].x, fma(v.y, a[q].y, wr));
+          wi = fma(v.x, a[q].y, fma(-v.y, a[q].x, wi));
+        }
+      }
+#pragma unroll
+      for (int o = 1; o < L; o <<= 1) {
+        wr += __shfl_xor_sync(0xffffffffu, wr, o);
+        wi += __shfl_xor_sync(0xffffffffu, wi, o);
+      }
+      const double tk = Tau[k];
+      wr *= tk;
+      wi *= tk;
+#pragma unroll
+      for (int q = 0; q < kQsSlots; ++q) {
+        const int r = L * q + h;
+        if (L * q + L - 1 < k || L * q >= N) continue;
+        if (r >= k && r < N) {
+          const double2 v = vk[r];
+          a[q].x = fma(-v.x, wr, fma(v.y, wi, a[q].x));
+          a[q].y = fma(-v.x, wi, fma(-v.y, wr, a[q].y));
+        }
+      }
+    }
+    if (j < M) {
+      // column j of R above the diagonal: rows k < j, final now, phase-fixed
+#pragma unroll
+      for (int q = 0; q < kQsSlots; ++q) {
+        const int r = L * q + h;
+        if (act && r < j) {
+          const double re = a[q].x * ph[q].x + a[q].y * ph[q].y, im = a[q].y * ph[q].x - a[q].x * ph[q].y;
+          put_r(out, n, r, j, (u64)__double_as_longlong(re), (u64)__double_as_longlong(im));
+        }
+      }
+      // reflector j from rows j..N-1
+      double s = 0.0;
+      double2 x0 = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int q = 0; q < kQsSlots; ++q) {
+        const int r = L * q + h;
+        if (r >= j && r < N) s = fma(a[q].x, a[q].x, fma(a[q].y, a[q].y, s));
+        if (r == j) x0 = a[q];
+      }
+#pragma unroll
+      for (int o = 1; o < L; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const int h0 = j % L;
+      x0.x = __shfl_sync(0xffffffffu, x0.x, (lane & ~(L - 1)) | h0);
+      x0.y = __shfl_sync(0xffffffffu, x0.y, (lane & ~(L - 1)) | h0);
+      double sigma = 0.0, tj = 0.0;
+      double2 phr = make_double2(1.0, 0.0), al = make_double2(0.0, 0.0);
+      if (s > 0.0) {
+        const double rs = rsqrt64(s);
+        sigma = s * rs;
+        const double qq = fma(x0.x, x0.x, x0.y * x0.y);
+        double ax0 = 0.0;
+        double2 p0 = make_double2(1.0, 0.0);
+        if (qq > 0.0) {
+          const double rq = rsqrt64(qq);
+          ax0 = qq * rq;
+          p0 = make_double2(x0.x * rq, x0.y * rq);
+        }
+        // alpha = -e^{i arg x0} sigma keeps v_j = x0 - alpha free of cancellation
+        al = make_double2(-p0.x * sigma, -p0.y * sigma);
+        phr = make_double2(-p0.x, -p0.y);
+        tj = rcp64(sigma * (sigma + ax0));
+      } else {
+        sing = 1;
+      }
+      double2* vj = V + (size_t)(qs_vo(j, N) - j);
+#pragma unroll
+      for (int q = 0; q < kQsSlots; ++q) {
+        const int r = L * q + h;
+        if (act && r >= j && r < N) vj[r] = (r == j) ? make_double2(x0.x - al.x, x0.y - al.y) : a[q];
+        if (r == j) ph[q] = phr;
+      }
+      if (lane == 0) Tau[j] = tj;
+      if (act && h == h0) put_r(out, n, j, j, (u64)__double_as_longlong(sigma), 0);
+    } else {
+      // ybar = Q^H y: rows k < M of the y column, phase-fixed
+#pragma unroll
+      for (int q = 0; q < kQsSlots; ++q) {
+        const int r = L * q + h;
+        if (act && r < M) {
+          const double re = a[q].x * ph[q].x + a[q].y * ph[q].y, im = a[q].y * ph[q].x - a[q].x * ph[q].y;
+          put_y(out, r, (u64)__double_as_longlong(re), (u64)__double_as_longlong(im));
+        }
+      }
+    }
+    __syncwarp();
+  }
+  if (act) {
+    if (out.Rdense)
+      for (int t = h; t < n * n; t += L)
+        if (t / n > t % n) out.Rdense[t] = 0.0;
+    if (h == 0 && out.singular) *out.singular = sing;
+  }
+}
+
+
+__host__ __device__ inline size_t qr64_smem(int N, int M) {
+  return N <= 32 ? sizeof(double2) * (size_t)qs_vo(M, N) + sizeof(double) * (size_t)M
+                 : sizeof(double2) * ((size_t)(M + 1) * N + M) + sizeof(double) * M + sizeof(int) * 4;
+}
+// Factorises one [H | y] in FP64 with the calling CTA.
+__device__ __noinline__ void qr64_one(int N, int M, const double* Hb, const double* yb, const QrDst& out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const double2* H2 = reinterpret_cast<const double2*>(Hb);
+  const double2* y2 = reinterpret_cast<const double2*>(yb);
+  if (N > 32) {
+    qr_one<32>(N, M, H2, y2, out);
+  } else if (threadIdx.x < 32) {
+    double2* V = reinterpret_cast<double2*>(smem_raw);
+    double* Tau = reinterpret_cast<double*>(V + qs_vo(M, N));
+    if (N <= 16)
+      qr_small64_one<2>(N, M, H2, y2, out, V, Tau);
+    else
+      qr_small64_one<4>(N, M, H2, y2, out, V, Tau);
+  }
+}
+
 // a conj(p) of a fixed-point entry and a phase p (limbs), as double bits.
 __device__ __forceinline__ void fx_unphase(i64 ar, i64 ai, int4 p, int e, u64& re, u64& im) {
   const int4 a = fx_split(ar, ai);
   const i64 mr = wide_add(a.x, p.y, wide_add(a.y, p.x, wide_add(a.z, p.w, wide(a.w, p.z))));
   const i64 mi = wide_add(a.z, p.y, wide(a.w, p.x)) - wide_add(a.x, p.w, wide(a.y, p.z));
-  re = fx_to_bits(wide(a.x, p.x) + wide(a.z, p.z) + ((mr + 2 * kFxHalf) >> kFxLimb), e);
+  re = fx_to_bits(wide(a.x, p.x) + wide(a.z, p.z) + ((mr + kFxHalf) >> kFxLimb), e);
   im = fx_to_bits(wide(a.z, p.x) - wide(a.x, p.z) + ((mi + kFxHalf) >> kFxLimb), e);
 }
 
-// u^H a summed over a lane's rows, one entry at a time.  The low limbs'
-// products (a quarter of a unit each on average) are left out: their mean,
-// half a unit per row of the real part, is added back by bias().
+// u^H a summed over a lane's rows, one entry at a time (the low limbs'
+// products, below a quarter of a unit each, are left out).
 struct FxDot {
   i64 rh = 0, rm = 0, rn = 0, ph = 0, pm = 0, qh = 0, qm = 0;
   __device__ __forceinline__ void add(int4 u, i64 ar, i64 ai) {
@@ -313,13 +499,10 @@ struct FxDot {
   }
   __device__ __forceinline__ i64 re() const { return rh + ((rm + rn + kFxHalf) >> kFxLimb); }
   __device__ __forceinline__ i64 im() const { return (ph - qh) + ((pm - qm + kFxHalf) >> kFxLimb); }
-  static __device__ __forceinline__ i64 bias(int rows) { return (i64)(rows >> 1); }
 };
-// a - u w (w limbs, nw the limbs of -w).  Two low-limb products are dropped
-// per part; with the rounding half this adds one unit to the middle sum (0
-// for a masked row, u = 0, which must not move).
-__device__ __forceinline__ void fx_axpy(int4 u, int4 w, int4 nw, i64& ar, i64& ai, i64 round = 2 * kFxHalf) {
-  i64 mr = round, mi = round;
+// a - u w (w limbs, nw the limbs of -w).
+__device__ __forceinline__ void fx_axpy(int4 u, int4 w, int4 nw, i64& ar, i64& ai) {
+  i64 mr = kFxHalf, mi = kFxHalf;
   mr = wide_add(u.x, nw.y, mr);
   mr = wide_add(u.y, nw.x, mr);
   mr = wide_add(u.z, w.w, mr);
@@ -380,7 +563,6 @@ __device__ __forceinline__ i64 lanes_sum(i64 v) {
 // warp's matrices innermost (consecutive lanes read consecutive 16-byte
 // entries); the phases of R's rows stay in the registers of the lanes owning
 // them.
-__host__ __device__ inline int qs_vo(int k, int N) { return k * N - k * (k - 1) / 2; }  // first entry of u_k
 __host__ __device__ inline size_t qs_smem(int N, int M, int lanes) {
   return sizeof(int4) * (32 / lanes) * (size_t)qs_vo(M, N);
 }
@@ -397,11 +579,10 @@ __device__ __forceinline__ void qs_apply(i64 (&ar)[SL], i64 (&ai)[SL], const int
     uu[q] = in ? u[r * stride] : make_int4(0, 0, 0, 0);
     d.add(uu[q], ar[q], ai[q]);
   }
-  const i64 wr = lanes_sum<L>(d.re()) + FxDot::bias(N - k), wi = lanes_sum<L>(d.im());
+  const i64 wr = lanes_sum<L>(d.re()), wi = lanes_sum<L>(d.im());
   const int4 w = fx_split(wr, wi), nw = fx_split(-wr, -wi);
 #pragma unroll
-  for (int q = Q0; q < SL; ++q)
-    fx_axpy(uu[q], w, nw, ar[q], ai[q], q > Q0 || L * Q0 + h >= k ? 2 * kFxHalf : 0);
+  for (int q = Q0; q < SL; ++q) fx_axpy(uu[q], w, nw, ar[q], ai[q]);
 }
 
 // Reflectors L Q0 .. kend - 1 on column j (kend = j, or M for the y column
@@ -666,7 +847,7 @@ __global__ void qr_redo_kernel(QrBatch g) {
       const QrDst d = g.get(t, Hb, yb);
       if (!is_redo(d, n)) continue;
       __syncthreads();  // every thread has read the mark that qr_one overwrites
-      qr_one<32>(g.N, g.M, reinterpret_cast<const double2*>(Hb), reinterpret_cast<const double2*>(yb), d);
+      qr64_one(g.N, g.M, Hb, yb, d);
       __syncthreads();
     }
   }
@@ -720,7 +901,7 @@ __device__ __forceinline__ void qc_update(longlong2* col, const int4* u, int k, 
     const longlong2 a0 = col[r];
     d.add(u[r], a0.x, a0.y);
   }
-  const i64 wr = lanes_sum<L>(d.re()) + FxDot::bias(N - k), wi = lanes_sum<L>(d.im());
+  const i64 wr = lanes_sum<L>(d.re()), wi = lanes_sum<L>(d.im());
   const int4 w = fx_split(wr, wi), nw = fx_split(-wr, -wi);
   for (r = k + h; r + L < end; r += 2 * L) {
     longlong2 a0 = col[r], a1 = col[r + L];
@@ -830,7 +1011,7 @@ __device__ void qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
   __syncthreads();  // every thread has read the flag that qr_one's data overwrites
   if (redo) {
     if constexpr (std::is_same<Src, SrcH>::value) {
-      qr_one<32>(N, M, reinterpret_cast<const double2*>(src.H), reinterpret_cast<const double2*>(src.y), out);
+      qr64_one(N, M, reinterpret_cast<const double*>(src.H), reinterpret_cast<const double*>(src.y), out);
     } else if constexpr (std::is_same<Src, SrcR>::value) {
       if (tid == 0) *out.sorted = 0;
       src.restore(out, tid, nthr);
@@ -910,13 +1091,10 @@ __global__ void __launch_bounds__(256, 3) qr_aug_cta_kernel(AugArgs g) {
   qr_cta_one(2 * g.a.n_tx, g.a.n_tx, src, d);
 }
 
-size_t qr_smem(int n_rx, int n_tx) {
-  return sizeof(double2) * ((size_t)(n_tx + 1) * n_rx + n_tx) + sizeof(double) * n_tx + sizeof(int) * 4;
-}
 size_t qr_cta_smem(int n_rx, int n_tx) {
   QrCtaLayout L;
   L.init(n_rx, n_tx);
-  return std::max(L.bytes, qr_smem(n_rx, n_tx));
+  return std::max(L.bytes, qr64_smem(n_rx, n_tx));
 }
 
 template <int L, int SL>
@@ -924,7 +1102,7 @@ cudaError_t launch_qs(const QrBatch& g, cudaStream_t s) {
   const size_t sm = qs_smem(g.N, g.M, L);
   cudaFuncSetAttribute(qr_small_kernel<L, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   qr_small_kernel<L, SL><<<(g.count + 32 / L - 1) / (32 / L), 32, sm, s>>>(g);
-  const size_t redo = qr_smem(g.N, g.M);
+  const size_t redo = qr64_smem(g.N, g.M);
   cudaFuncSetAttribute(qr_redo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)redo);
   qr_redo_kernel<<<std::min((g.count + 127) / 128, 304), 128, redo, s>>>(g);
   return cudaGetLastError();

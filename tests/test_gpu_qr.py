@@ -82,3 +82,19 @@ def test_uneven_batch_uses_the_same_forms():
     reqs = mdx.make_requests(np.full(B, n), n, qam, mdx.MDX_ALGO_KBEST, K=16)
     sym, met, _, _ = mdx.detect_mixed(ctx, reqs, H.reshape(-1), y.reshape(-1), nv)
     assert torch.equal(sym.view(B, n), uniform[0]) and torch.equal(met, uniform[1])
+
+
+@pytest.mark.parametrize("N,M,B", [(8, 8, 1300), (16, 16, 1300), (20, 17, 2000), (16, 16, 4), (64, 50, 4)])
+def test_zeros_stay_exactly_zero(N, M, B):
+    """y = 0 gives ybar = 0 and a diagonal channel a diagonal R, exactly (ties between leaves are then
+    exact ties), and the identity gives the identity."""
+    w = wl.generate(8400 + N, B, N, M, 16, 10.0)
+    H, y = w["H"].copy(), w["y"].copy()
+    y[0] = 0.0
+    H[1:3] = 0.0
+    H[1, np.arange(M), np.arange(M), 0] = 1.0
+    H[2, np.arange(M), np.arange(M), 0] = 1.0 + np.arange(M) / 7.0
+    R, yb = _run(H, y)
+    assert np.all(yb[0] == 0.0)
+    assert np.array_equal(R[1], np.eye(2 * M))
+    assert np.array_equal(R[2], np.diag(np.repeat(1.0 + np.arange(M) / 7.0, 2)))
