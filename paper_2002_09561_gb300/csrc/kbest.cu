@@ -30,6 +30,8 @@
 //
 // Both kernels keep the final leaves within FP32 error of the best and
 // re-score them in FP64 against the FP64 R and ybar.
+#include <algorithm>
+
 #include "mdx_internal.cuh"
 #include "warp_kbest.cuh"
 
@@ -666,7 +668,7 @@ __device__ void finish_vector(const SearchArgs& a, int v, const uint8_t* cx, con
 }
 
 __device__ bool singular_vector(const SearchArgs& a, int v) {
-  if (!(a.singular && a.singular[v])) return false;
+  if (!(a.singular && a.singular[v] == 1)) return false;
   for (int j = threadIdx.x; j < a.n_tx; j += blockDim.x) a.sym_out[(size_t)v * a.n_tx + j] = 0;
   if (threadIdx.x == 0) {
     a.metric_out[v] = 0.0;
@@ -677,7 +679,8 @@ __device__ bool singular_vector(const SearchArgs& a, int v) {
   return true;
 }
 
-__global__ void __launch_bounds__(1024) kbest_kernel(SearchArgs a, KbLayout L) {
+// redo: only the vectors that the warp kernel marked (kKbestRedo).
+__global__ void __launch_bounds__(1024) kbest_kernel(SearchArgs a, KbLayout L, int redo) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, T = blockDim.x;
   const int n = a.n, P = a.P;
@@ -687,11 +690,27 @@ __global__ void __launch_bounds__(1024) kbest_kernel(SearchArgs a, KbLayout L) {
   KbCtx c{n, P, a.K, L.pp, tid, T, a.alpha, reinterpret_cast<float*>(smem + L.off_R),
           reinterpret_cast<float*>(smem + L.off_yb), keys, misc, reinterpret_cast<float*>(smem + L.off_cc)};
 
+  // redo: chunks of T vectors, the marks of one read together
+  int chunk = ((int)blockIdx.x - (int)gridDim.x) * T, at = T;
+  auto next_marked = [&]() {
+    for (;;) {
+      for (; at < T; ++at)
+        if (chunk + at < a.batch && a.singular[chunk + at] == kKbestRedo) return chunk + at++;
+      chunk += gridDim.x * T;
+      if (chunk >= a.batch) return a.batch;
+      at = __syncthreads_or(chunk + tid < a.batch && a.singular[chunk + tid] == kKbestRedo) ? 0 : T;
+    }
+  };
   for (;;) {
-    if (tid == 0) misc[1] = (int)atomicAdd(a.work_counter, 1u);
-    __syncthreads();
-    const int v = misc[1];
-    __syncthreads();
+    int v;
+    if (redo) {
+      v = next_marked();
+    } else {
+      if (tid == 0) misc[1] = (int)atomicAdd(a.work_counter, 1u);
+      __syncthreads();
+      v = misc[1];
+      __syncthreads();
+    }
     if (v >= a.batch) break;
     if (singular_vector(a, v)) continue;
     stage_vector(a, v, L, smem, misc_f);
@@ -1215,7 +1234,7 @@ int kb_threads(int K, int P) {
 }
 
 cudaError_t launch_generic(const void* fn, const SearchArgs& a, const KbLayout& L, int T, int num_sms,
-                           cudaStream_t s) {
+                           cudaStream_t s, bool redo) {
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
@@ -1224,7 +1243,8 @@ cudaError_t launch_generic(const void* fn, const SearchArgs& a, const KbLayout& 
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   int grid = per_sm * num_sms;
   if (grid > a.batch) grid = a.batch;
-  kbest_kernel<<<grid, T, L.bytes, s>>>(a, L);
+  if (redo) grid = std::min(grid, (a.batch + T - 1) / T);
+  kbest_kernel<<<grid, T, L.bytes, s>>>(a, L, redo ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1243,14 +1263,16 @@ size_t kbest_smem_bytes(int n, int K, int P, bool complex_tree) {
 cudaError_t launch_kbest(const SearchArgs& a, int num_sms, cudaStream_t s) {
   if (a.batch <= 0) return cudaSuccess;
   KbLayout L;
-  if (a.flags & MDX_COMPLEX_TREE) {
+  if (a.flags & MDX_COMPLEX_TREE)
     kb_geometry_complex(L, a.n, a.K, a.P);
-    if (L.bytes > 227 * 1024) return cudaErrorInvalidConfiguration;
-    return launch_generic((const void*)kbest_kernel, a, L, L.T, num_sms, s);
-  }
-  kb_geometry(L, a.n, a.K, a.P);
+  else
+    kb_geometry(L, a.n, a.K, a.P);
   if (L.bytes > 227 * 1024) return cudaErrorInvalidConfiguration;
-  return launch_generic((const void*)kbest_kernel, a, L, L.T, num_sms, s);
+  // a vector per warp, and the few with a tie at a cut by the sorting kernel;
+  // where the warp form does not fit, all of them
+  const cudaError_t e = launch_kbest_warp(a, L.E > 0, s);
+  if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
+  return launch_generic((const void*)kbest_kernel, a, L, L.T, num_sms, s, e == cudaSuccess);
 }
 
 // Eight warps per CTA with as many K-best workspaces as fit (the best prefix

@@ -183,6 +183,11 @@ size_t sd_task_bytes();
 size_t sd_vec_state_bytes(int n);
 cudaError_t launch_sd(const SearchArgs& a, const SdWorkspace& w, int num_sms, cudaStream_t s);
 cudaError_t launch_kbest(const SearchArgs& a, int num_sms, cudaStream_t s);
+// One vector per warp (kbest_warp.cu); eight: row interference as eight FMA
+// chains (else one).  Vectors it leaves to the sorting kernel get this mark in
+// their singular flag.
+constexpr int kKbestRedo = 2;
+cudaError_t launch_kbest_warp(const SearchArgs& a, bool eight, cudaStream_t s);
 // Shared memory of the K-best kernel for (n, K, P, key capacity).
 size_t kbest_smem_bytes(int n, int K, int P, bool complex_tree);
 cudaError_t launch_hybrid(const SearchArgs& a, int num_sms, cudaStream_t s);
