@@ -35,7 +35,7 @@ constexpr i64 kFxHalf = 1ll << (kFxLimb - 1);  // rounds md to the nearest unit
 
 __host__ __device__ __forceinline__ int fx_lo(i64 a) { return (int)((unsigned)a << (32 - kFxLimb)) >> (32 - kFxLimb); }
 __host__ __device__ __forceinline__ int fx_hi(i64 a) { return (int)(a >> kFxLimb) + (int)((unsigned)fx_lo(a) >> 31); }
-// a b and c + a b as one wide multiply(-add).  (Written out: where the
+// a b as one wide multiply.  (Written out: where the
 // compiler can tell a limb's sign it may widen it with zeros and multiply in 64
 // bits, three instructions for one.)
 __host__ __device__ __forceinline__ i64 wide(int a, int b) {
@@ -47,15 +47,10 @@ __host__ __device__ __forceinline__ i64 wide(int a, int b) {
   return (i64)a * (i64)b;
 #endif
 }
-__host__ __device__ __forceinline__ i64 wide_add(int a, int b, i64 c) {
-#ifdef __CUDA_ARCH__
-  i64 r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-#else
-  return c + (i64)a * (i64)b;
-#endif
-}
+// c + a b: the multiply above and a plain addition fuse into one wide
+// multiply-add (mad.wide itself becomes a multiply and an addition: 2 x the
+// instructions, measured).
+__host__ __device__ __forceinline__ i64 wide_add(int a, int b, i64 c) { return c + wide(a, b); }
 
 // A complex number as limbs: {re high, re low, im high, im low}.
 __host__ __device__ __forceinline__ int4 fx_split(i64 re, i64 im) {

@@ -479,44 +479,46 @@ __device__ __forceinline__ void fx_unphase(i64 ar, i64 ai, int4 p, int e, u64& r
 }
 
 // u^H a summed over a lane's rows, one entry at a time (the low limbs'
-// products, below a quarter of a unit each, are left out).
+// products, below a quarter of a unit each, are left out).  A wide multiply-add
+// holds the multiplier for four cycles, so a complex product takes three real
+// ones instead of four: with k1 = ur ar, k2 = ui ai and p = (ur + ui)(ai - ar),
+// the real part is k1 + k2, the imaginary part p + k1 - k2.
 struct FxDot {
-  i64 rh = 0, rm = 0, rn = 0, ph = 0, pm = 0, qh = 0, qm = 0;
+  i64 k1h = 0, k1m = 0, k2h = 0, k2m = 0, ph = 0, pm = 0;
   __device__ __forceinline__ void add(int4 u, i64 ar, i64 ai) {
     const int4 a = fx_split(ar, ai);
-    rh = wide_add(u.x, a.x, rh);
-    rh = wide_add(u.z, a.z, rh);
-    rm = wide_add(u.x, a.y, rm);
-    rm = wide_add(u.y, a.x, rm);
-    rn = wide_add(u.z, a.w, rn);
-    rn = wide_add(u.w, a.z, rn);
-    ph = wide_add(u.x, a.z, ph);
-    pm = wide_add(u.x, a.w, pm);
-    pm = wide_add(u.y, a.z, pm);
-    qh = wide_add(u.z, a.x, qh);
-    qm = wide_add(u.z, a.y, qm);
-    qm = wide_add(u.w, a.x, qm);
+    const int sh = u.x + u.z, sl = u.y + u.w, dh = a.z - a.x, dl = a.w - a.y;
+    k1h = wide_add(u.x, a.x, k1h);
+    k1m = wide_add(u.x, a.y, k1m);
+    k1m = wide_add(u.y, a.x, k1m);
+    k2h = wide_add(u.z, a.z, k2h);
+    k2m = wide_add(u.z, a.w, k2m);
+    k2m = wide_add(u.w, a.z, k2m);
+    ph = wide_add(sh, dh, ph);
+    pm = wide_add(sh, dl, pm);
+    pm = wide_add(sl, dh, pm);
   }
-  __device__ __forceinline__ i64 re() const { return rh + ((rm + rn + kFxHalf) >> kFxLimb); }
-  __device__ __forceinline__ i64 im() const { return (ph - qh) + ((pm - qm + kFxHalf) >> kFxLimb); }
+  __device__ __forceinline__ i64 re() const { return (k1h + k2h) + ((k1m + k2m + kFxHalf) >> kFxLimb); }
+  __device__ __forceinline__ i64 im() const {
+    return (ph + (k1h - k2h)) + ((pm + (k1m - k2m) + kFxHalf) >> kFxLimb);
+  }
 };
-// a - u w (w limbs, nw the limbs of -w).
-__device__ __forceinline__ void fx_axpy(int4 u, int4 w, int4 nw, i64& ar, i64& ai) {
-  i64 mr = kFxHalf, mi = kFxHalf;
-  mr = wide_add(u.x, nw.y, mr);
-  mr = wide_add(u.y, nw.x, mr);
-  mr = wide_add(u.z, w.w, mr);
-  mr = wide_add(u.w, w.z, mr);
-  mi = wide_add(u.x, nw.w, mi);
-  mi = wide_add(u.y, nw.z, mi);
-  mi = wide_add(u.z, nw.y, mi);
-  mi = wide_add(u.w, nw.x, mi);
-  ar = wide_add(u.x, nw.x, ar);
-  ar = wide_add(u.z, w.z, ar);
-  ai = wide_add(u.x, nw.z, ai);
-  ai = wide_add(u.z, nw.x, ai);
-  ar += mr >> kFxLimb;
-  ai += mi >> kFxLimb;
+// The multiplier w of an update a - u w, as limbs: -wr, wi and -(wr + wi).
+struct FxMul {
+  int nrh, nrl, ih, il, nsh, nsl;
+  __device__ __forceinline__ FxMul(i64 wr, i64 wi)
+      : nrh(fx_hi(-wr)), nrl(fx_lo(-wr)), ih(fx_hi(wi)), il(fx_lo(wi)), nsh(fx_hi(-wr) - fx_hi(wi)),
+        nsl(fx_lo(-wr) - fx_lo(wi)) {}
+};
+// a - u w: with p1 = -ur wr, p2 = ui wi and p3 = -(ur + ui)(wr + wi), the real
+// part gains p1 + p2, the imaginary part p3 - p1 + p2.
+__device__ __forceinline__ void fx_axpy(int4 u, const FxMul& w, i64& ar, i64& ai) {
+  const int sh = u.x + u.z, sl = u.y + u.w;
+  const i64 h1 = wide(u.x, w.nrh), m1 = wide_add(u.y, w.nrh, wide(u.x, w.nrl));
+  const i64 h2 = wide(u.z, w.ih), m2 = wide_add(u.w, w.ih, wide_add(u.z, w.il, kFxHalf));
+  const i64 m3 = wide_add(sl, w.nsh, wide_add(sh, w.nsl, m2));
+  ar += h1 + h2 + ((m1 + m2) >> kFxLimb);
+  ai = wide_add(sh, w.nsh, ai) + (h2 - h1) + ((m3 - m1) >> kFxLimb);
 }
 // Sums of squares of a reflector column (see fx_reflector).
 struct FxNorm {
@@ -580,9 +582,9 @@ __device__ __forceinline__ void qs_apply(i64 (&ar)[SL], i64 (&ai)[SL], const int
     d.add(uu[q], ar[q], ai[q]);
   }
   const i64 wr = lanes_sum<L>(d.re()), wi = lanes_sum<L>(d.im());
-  const int4 w = fx_split(wr, wi), nw = fx_split(-wr, -wi);
+  const FxMul w(wr, wi);
 #pragma unroll
-  for (int q = Q0; q < SL; ++q) fx_axpy(uu[q], w, nw, ar[q], ai[q]);
+  for (int q = Q0; q < SL; ++q) fx_axpy(uu[q], w, ar[q], ai[q]);
 }
 
 // Reflectors L Q0 .. kend - 1 on column j (kend = j, or M for the y column
@@ -854,213 +856,245 @@ __global__ void qr_redo_kernel(QrBatch g) {
 }
 
 // ---------------------------------------------------------------------------
-// One CTA per matrix: [H | y] in shared memory (column-major, 16-byte fixed
-// point entries), right-looking.  Warp 0 runs one column ahead: in step k it
-// applies reflector k to column k + 1 alone and forms the next reflector,
-// while the other warps apply reflector k to the columns right of it, eight
-// lanes per column (a warp reads 8 consecutive entries of four columns: full
-// 128-byte wavefronts, the reflector's entries broadcast).  One barrier per
-// column; the reflector buffer is doubled.
-constexpr int kCtaLanes = 8;
+// One CTA per matrix, left-looking in a pipeline of warps.  A warp takes groups
+// of 32 / L columns in ascending order (L lanes per column, rows L q + h of
+// lane h in registers, y the last column), applies the reflectors of the
+// groups before as they appear, then forms its own.  A reflector is published
+// in shared memory under an mbarrier, so no warp waits for more than it reads:
+// while one warp is on the chain (apply, norm, scalars of the next reflector),
+// the others catch up on earlier ones.  Only the reflectors are in shared
+// memory (a triangle of 16-byte limb entries, half of the matrix).  The loop
+// over reflectors is compiled for the rows still touched in steps of 16.
+//
+// Bound by instruction issue (the multiply-add pipe 62-69 % busy on many
+// matrices) and, for few matrices, by the chain.  Against the matrix in shared
+// memory, right-looking, with one CTA barrier per column (us, before / now):
+// one matrix 16x16 41 / 28, 32x32 78 / 58, 64x64 190 / 165; 608 matrices 32x32
+// 176 / 92; 2,432 matrices 48x48 883 / 845, 64x64 1,673 / 1,609, 100x100
+// 6,101 / 5,895.
 
 struct QrCtaLayout {
-  size_t off_u, off_ph, off_e, off_sig, off_sg, off_flag, bytes;
+  size_t off_ph, off_bar, off_flag, bytes;
   __host__ __device__ void init(int N, int M) {
-    size_t o = sizeof(longlong2) * (size_t)(M + 1) * N;
-    off_u = o;
-    o += sizeof(int4) * 2 * (size_t)N;
+    size_t o = sizeof(int4) * (size_t)qs_vo(M, N);
     off_ph = o;
     o += sizeof(int4) * (size_t)M;
-    off_sig = o;
-    o += sizeof(i64) * (size_t)M;
-    off_e = o;
-    o += sizeof(int) * (size_t)(M + 1);
-    off_sg = o;
-    o += sizeof(int) * (size_t)M;
+    off_bar = o;
+    o += sizeof(u64) * (size_t)M;
     off_flag = o;
-    o += 2 * sizeof(int);
+    o += 16;
     bytes = o;
   }
 };
 
-// a_c <- (I - u u^H) a_c over rows k..N-1 by L lanes, two rows at a time (both
-// loads before the arithmetic: the compiler must assume that a store to the
-// column changes u).
-template <int L>
-__device__ __forceinline__ void qc_update(longlong2* col, const int4* u, int k, int N, int h, bool act) {
-  FxDot d;
-  const int end = act ? N : 0;
-  int r = k + h;
-  for (; r + L < end; r += 2 * L) {
-    const longlong2 a0 = col[r], a1 = col[r + L];
-    const int4 u0 = u[r], u1 = u[r + L];
-    d.add(u0, a0.x, a0.y);
-    d.add(u1, a1.x, a1.y);
+__device__ __forceinline__ unsigned smem_at(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+// Waits until the barrier's first phase is complete; false after a bounded
+// number of tries.
+__device__ __forceinline__ bool wait_published(const u64* bar) {
+  for (int it = 0; it < (1 << 20); ++it) {
+    unsigned done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(smem_at(bar))
+        : "memory");
+    if (done) return true;
   }
-  if (r < end) {
-    const longlong2 a0 = col[r];
-    d.add(u[r], a0.x, a0.y);
+  return false;
+}
+
+// Slots per piece of the loop over reflectors: 16 rows, or a slot.
+template <int L>
+constexpr int qc_step = L < 16 ? 16 / L : 1;
+
+// Reflector k (entries from row k on at u + r) on the rows L Q0 .. of the
+// lanes' columns; masked: also rows above k among the piece's first slots.
+template <int L, int SL, int Q0>
+__device__ __forceinline__ void qc_apply(i64 (&ar)[SL], i64 (&ai)[SL], const int4* u, int k, int N, int h, bool act) {
+  FxDot d;
+#pragma unroll
+  for (int q = Q0; q < SL; ++q) {
+    const int r = L * q + h;
+    const bool in = (q >= Q0 + qc_step<L> || r >= k) && r < N;
+    const int4 uu = in ? u[r] : make_int4(0, 0, 0, 0);
+    d.add(uu, ar[q], ai[q]);
   }
   const i64 wr = lanes_sum<L>(d.re()), wi = lanes_sum<L>(d.im());
-  const int4 w = fx_split(wr, wi), nw = fx_split(-wr, -wi);
-  for (r = k + h; r + L < end; r += 2 * L) {
-    longlong2 a0 = col[r], a1 = col[r + L];
-    const int4 u0 = u[r], u1 = u[r + L];
-    i64 x0 = a0.x, y0 = a0.y, x1 = a1.x, y1 = a1.y;
-    fx_axpy(u0, w, nw, x0, y0);
-    fx_axpy(u1, w, nw, x1, y1);
-    col[r] = make_longlong2(x0, y0);
-    col[r + L] = make_longlong2(x1, y1);
-  }
-  if (r < end) {
-    const longlong2 a0 = col[r];
-    i64 x0 = a0.x, y0 = a0.y;
-    fx_axpy(u[r], w, nw, x0, y0);
-    col[r] = make_longlong2(x0, y0);
+  const FxMul w(act ? wr : 0, act ? wi : 0);  // (0 leaves a column as it is)
+#pragma unroll
+  for (int q = Q0; q < SL; ++q) {
+    const int r = L * q + h;
+    const bool in = (q >= Q0 + qc_step<L> || r >= k) && r < N;
+    const int4 uu = in ? u[r] : make_int4(0, 0, 0, 0);
+    fx_axpy(uu, w, ar[q], ai[q]);
   }
 }
+template <int L, int SL, int Q0>
+struct QcApply {  // one reflector, by the piece of k
+  static __device__ __forceinline__ void run(i64 (&ar)[SL], i64 (&ai)[SL], const int4* u, int k, int N, int h,
+                                             bool act) {
+    if (k < L * (Q0 + qc_step<L>) || Q0 + qc_step<L> >= SL)
+      qc_apply<L, SL, Q0>(ar, ai, u, k, N, h, act);
+    else if constexpr (Q0 + qc_step<L> < SL)
+      QcApply<L, SL, Q0 + qc_step<L>>::run(ar, ai, u, k, N, h, act);
+  }
+};
 
-template <typename Src>
-__device__ void qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
+// Factorises the matrix with the calling CTA; false if it needs the FP64 form
+// (the outputs are then unfinished).
+template <int L, int SL, typename Src>
+__device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  QrCtaLayout L;
-  L.init(N, M);
-  longlong2* A = reinterpret_cast<longlong2*>(smem_raw);
-  int4* U = reinterpret_cast<int4*>(smem_raw + L.off_u);
-  int4* ph = reinterpret_cast<int4*>(smem_raw + L.off_ph);
-  i64* sig = reinterpret_cast<i64*>(smem_raw + L.off_sig);  // R_kk and its exponent
-  int* sg = reinterpret_cast<int*>(smem_raw + L.off_sg);
-  int* es = reinterpret_cast<int*>(smem_raw + L.off_e);
-  volatile int* flag = reinterpret_cast<volatile int*>(smem_raw + L.off_flag);
-  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
+  constexpr int kCols = 32 / L;  // columns of a group
+  QrCtaLayout lay;
+  lay.init(N, M);
+  int4* U = reinterpret_cast<int4*>(smem_raw);
+  int4* ph = reinterpret_cast<int4*>(smem_raw + lay.off_ph);
+  u64* bar = reinterpret_cast<u64*>(smem_raw + lay.off_bar);
+  volatile int* flag = reinterpret_cast<volatile int*>(smem_raw + lay.off_flag);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int h = lane % L, sub = lane / L, n = 2 * M;
   if (tid == 0) *flag = 0;
-  for (int t = tid; t < N * M; t += nthr) A[(size_t)(t % M) * N + t / M] = src(t / M, t % M);
-  for (int r = tid; r < N; r += nthr) A[(size_t)M * N + r] = src(r, M);
+  for (int k = tid; k < M; k += blockDim.x)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_at(bar + k)) : "memory");
   __syncthreads();
-  // the columns' scales, a warp per column
-  for (int c = warp; c <= M; c += nw) {
-    longlong2* col = A + (size_t)c * N;
+  int avail = 0;  // reflectors known to be published
+  for (int c0 = kCols * warp; c0 <= M; c0 += kCols * nw) {
+    const int c = c0 + sub;
+    const bool mine = c <= M;
+    // ---- the column, at its scale
+    i64 ar[SL], ai[SL];
     int ex = 0;
-    for (int r = lane; r < N; r += 32) {
-      const longlong2 z = col[r];
+#pragma unroll
+    for (int q = 0; q < SL; ++q) {
+      const int r = L * q + h;
+      longlong2 z = make_longlong2(0, 0);
+      if (mine && r < N) z = src(r, c);
+      ar[q] = z.x;
+      ai[q] = z.y;
       ex = max(ex, max(ex_of((u64)z.x), ex_of((u64)z.y)));
     }
-    ex = __reduce_max_sync(0xffffffffu, ex);
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
     float ss = 0.0f;
-    for (int r = lane; r < N; r += 32) {
-      const longlong2 z = col[r];
-      const float fr = fx_rel((u64)z.x, ex), fi = fx_rel((u64)z.y, ex);
+#pragma unroll
+    for (int q = 0; q < SL; ++q) {
+      const float fr = fx_rel((u64)ar[q], ex), fi = fx_rel((u64)ai[q], ex);
       ss = fmaf(fr, fr, fmaf(fi, fi, ss));
     }
-    ss = warp_sum(ss);
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     const bool fine = fx_in_range(ex);
     const int e = fine ? fx_scale(ex, ss) : 0;
-    for (int r = lane; r < N; r += 32) {
-      const longlong2 z = col[r];
-      col[r] = fine ? make_longlong2(fx_from((u64)z.x, e), fx_from((u64)z.y, e)) : make_longlong2(0, 0);
+    if (ex != 0 && !fine) *flag = 1;
+#pragma unroll
+    for (int q = 0; q < SL; ++q) {
+      ar[q] = fine ? fx_from((u64)ar[q], e) : 0;
+      ai[q] = fine ? fx_from((u64)ai[q], e) : 0;
     }
-    if (lane == 0) {
-      es[c] = e;
-      if (ex != 0 && !fine) *flag = 1;
-    }
-  }
-  __syncthreads();
-  // warp 0: reflector k from column k into U[k & 1]
-  auto reflect = [&](int k) {
-    const longlong2* col = A + (size_t)k * N;
-    FxNorm s;
-    for (int r = k + lane; r < N; r += 32) {
-      const longlong2 x = col[r];
-      s.add(x.x);
-      s.add(x.y);
-    }
-    const i64 hh = lanes_sum<32>(s.hh), md = lanes_sum<32>(s.md);
-    const u64 ll = (u64)lanes_sum<32>((i64)(s.ll >> 3));
-    int4* u = U + (size_t)(k & 1) * N;
-    FxReflector f;
-    const bool ok = fx_reflector(hh, md, ll, col[k].x, col[k].y, f);
-    for (int r = k + lane; r < N; r += 32) {
-      const longlong2 x = col[r];
-      u[r] = !ok ? make_int4(0, 0, 0, 0) : r == k ? fx_split(f.ur, f.ui) : fx_split(f.scale(x.x), f.scale(x.y));
-    }
-    if (lane == 0) {
-      if (!ok) *flag = 1;
-      ph[k] = fx_split(-f.pr, -f.pi);
-      sig[k] = (i64)f.sigma;
-      sg[k] = es[k] + f.s - 4;
-    }
-  };
-  if (warp == 0) reflect(0);
-  for (int k = 0; k < M; ++k) {
-    __syncthreads();
-    const int4* u = U + (size_t)(k & 1) * N;
-    if (warp == 0) {
-      qc_update<32>(A + (size_t)(k + 1) * N, u, k, N, lane, true);
-      __syncwarp();
-      if (k + 1 < M) reflect(k + 1);
-    } else {
-      const int ng = (nw - 1) * (32 / kCtaLanes);
-      for (int c0 = k + 2 + (warp - 1) * (32 / kCtaLanes); c0 <= M; c0 += ng) {
-        const int c = c0 + lane / kCtaLanes;
-        qc_update<kCtaLanes>(A + (size_t)min(c, M) * N, u, k, N, lane % kCtaLanes, c <= M);
+    // ---- the reflectors of the groups before
+    for (int k = 0; k < c0; ++k) {
+      if (k >= avail) {
+        if (!wait_published(bar + k)) *flag = 1;
+        avail = k + 1;
       }
+      QcApply<L, SL, 0>::run(ar, ai, U + qs_vo(k, N) - k, k, N, h, true);
+    }
+    // ---- the group's own
+    u64 sigma = 0;
+    int sexp = 0;
+    for (int t = 0; t < kCols && c0 + t < M; ++t) {
+      const int k = c0 + t;
+      FxNorm s;
+      i64 x0r = 0, x0i = 0;
+#pragma unroll
+      for (int q = 0; q < SL; ++q) {
+        const int r = L * q + h;
+        const bool in = r >= k && r < N;
+        s.add(in ? ar[q] : 0);
+        s.add(in ? ai[q] : 0);
+        if (r == k) {
+          x0r = ar[q];
+          x0i = ai[q];
+        }
+      }
+      const i64 hh = lanes_sum<L>(s.hh), md = lanes_sum<L>(s.md);
+      const u64 ll = (u64)lanes_sum<L>((i64)(s.ll >> 3));
+      const int h0 = (lane & ~(L - 1)) | (k % L);
+      x0r = __shfl_sync(0xffffffffu, x0r, h0);
+      x0i = __shfl_sync(0xffffffffu, x0i, h0);
+      FxReflector f;
+      const bool ok = fx_reflector(hh, md, ll, x0r, x0i, f);
+      int4* u = U + qs_vo(k, N) - k;
+      if (sub == t) {
+#pragma unroll
+        for (int q = 0; q < SL; ++q) {
+          const int r = L * q + h;
+          if (r >= k && r < N)
+            u[r] = !ok ? make_int4(0, 0, 0, 0)
+                       : r == k ? fx_split(f.ur, f.ui) : fx_split(f.scale(ar[q]), f.scale(ai[q]));
+        }
+        if (h == 0) {
+          if (!ok) *flag = 1;
+          ph[k] = fx_split(-f.pr, -f.pi);
+        }
+        sigma = f.sigma;
+        sexp = f.s;
+      }
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_at(bar + k)) : "memory");
+      if (t < kCols - 1) QcApply<L, SL, 0>::run(ar, ai, u, k, N, h, sub > t);
+    }
+    avail = max(avail, min(c0 + kCols, M));
+    // ---- out: rows above the diagonal (all their phases are published), the diagonal
+    if (mine) {
+#pragma unroll
+      for (int q = 0; q < SL; ++q) {
+        const int r = L * q + h;
+        if (r < min(c, M)) {
+          u64 re, im;
+          fx_unphase(ar[q], ai[q], ph[r], e, re, im);
+          if (c < M)
+            put_r(out, n, r, c, re, im);
+          else
+            put_y(out, r, re, im);
+        }
+      }
+      if (c < M && h == 0) put_r(out, n, c, c, fx_to_bits((i64)sigma, e + sexp - 4), 0);
     }
   }
   __syncthreads();
-  const bool redo = *flag != 0;
-  __syncthreads();  // every thread has read the flag that qr_one's data overwrites
-  if (redo) {
-    if constexpr (std::is_same<Src, SrcH>::value) {
-      qr64_one(N, M, reinterpret_cast<const double*>(src.H), reinterpret_cast<const double*>(src.y), out);
-    } else if constexpr (std::is_same<Src, SrcR>::value) {
-      if (tid == 0) *out.sorted = 0;
-      src.restore(out, tid, nthr);
-    } else {
-      if (tid == 0) *out.pk_bad = 1;
-    }
-    return;
-  }
-  if (tid == 0 && out.pk) *out.pk_bad = 0;
-  const int n = 2 * M, nb = M * (M + 1) / 2;  // complex entries (a, c) with a <= c
-  for (int t = tid; t < nb; t += nthr) {
-    int c = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // exact after the corrections below
-    while (c * (c + 1) / 2 > t) --c;
-    while ((c + 1) * (c + 2) / 2 <= t) ++c;
-    const int a = t - c * (c + 1) / 2;
-    u64 re, im = 0;
-    if (a < c) {
-      const longlong2 z = A[(size_t)c * N + a];
-      fx_unphase(z.x, z.y, ph[a], es[c], re, im);
-    } else {
-      re = fx_to_bits(sig[a], sg[a]);
-    }
-    put_r(out, n, a, c, re, im);
-  }
-  for (int a = tid; a < M; a += nthr) {
-    const longlong2 z = A[(size_t)M * N + a];
-    u64 re, im;
-    fx_unphase(z.x, z.y, ph[a], es[M], re, im);
-    put_y(out, a, re, im);
-  }
+  if (*flag) return false;
   if (out.Rdense)
-    for (int t = tid; t < n * n; t += nthr)
+    for (int t = tid; t < n * n; t += blockDim.x)
       if (t / n > t % n) out.Rdense[t] = 0.0;
-  if (tid == 0 && out.singular) *out.singular = 0;
+  return true;
 }
 
-template <int T, int B>
+template <int L, int SL, int T, int B>
 __global__ void __launch_bounds__(T, B) qr_cta_kernel(QrBatch g) {
   const double *Hb, *yb;
   const QrDst d = g.get(blockIdx.x, Hb, yb);
   const SrcH src{reinterpret_cast<const longlong2*>(Hb), reinterpret_cast<const longlong2*>(yb), g.M};
-  qr_cta_one(g.N, g.M, src, d);
+  const bool ok = qr_cta_one<L, SL>(g.N, g.M, src, d);
+  __syncthreads();  // the zeroed triangle, before the mark in it; the shared memory, before qr64_one
+  if (!ok && g.N <= 32)
+    qr64_one(g.N, g.M, Hb, yb, d);
+  else if (threadIdx.x == 0)
+    mark_redo(d, 2 * g.M, !ok);
 }
-__global__ void __launch_bounds__(256, 3) qr_reorder_cta_kernel(ReorderArgs g, int few) {
+template <int L, int SL>
+__global__ void __launch_bounds__(288, 2) qr_reorder_cta_kernel(ReorderArgs g, int few) {
   const int count = (int)*g.count;
   if (count > few || (int)blockIdx.x >= count) return;
   SrcR src;
   const QrDst d = reorder_at(g, blockIdx.x, src);
-  qr_cta_one(g.a.n_tx, g.a.n_tx, src, d);
+  if (!qr_cta_one<L, SL>(g.a.n_tx, g.a.n_tx, src, d)) {
+    __syncthreads();
+    if (threadIdx.x == 0) *d.sorted = 0;
+    src.restore(d, threadIdx.x, blockDim.x);
+  }
 }
 
 // The augmented systems of a batch (2 M x M, see linear.cu).
@@ -1085,16 +1119,25 @@ __global__ void __launch_bounds__(32) qr_aug_small_kernel(AugArgs g) {
   const QrDst d = aug_at(g, act ? i : 0, src);
   qr_small_pair<L, SL>(2 * g.a.n_tx, g.a.n_tx, act, src, d, reinterpret_cast<int4*>(smem_raw));
 }
-__global__ void __launch_bounds__(256, 3) qr_aug_cta_kernel(AugArgs g) {
+template <int L, int SL>
+__global__ void __launch_bounds__(288, 2) qr_aug_cta_kernel(AugArgs g) {
   SrcAug src;
   const QrDst d = aug_at(g, blockIdx.x, src);
-  qr_cta_one(2 * g.a.n_tx, g.a.n_tx, src, d);
+  const bool ok = qr_cta_one<L, SL>(2 * g.a.n_tx, g.a.n_tx, src, d);
+  if (threadIdx.x == 0) *d.pk_bad = ok ? 0 : 1;
 }
 
 size_t qr_cta_smem(int n_rx, int n_tx) {
   QrCtaLayout L;
   L.init(n_rx, n_tx);
-  return std::max(L.bytes, qr64_smem(n_rx, n_tx));
+  return n_rx <= 32 ? std::max(L.bytes, qr64_smem(n_rx, n_tx)) : L.bytes;
+}
+
+cudaError_t launch_redo(const QrBatch& g, cudaStream_t s) {
+  const size_t sm = qr64_smem(g.N, g.M);
+  cudaFuncSetAttribute(qr_redo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_redo_kernel<<<std::min((g.count + 127) / 128, 304), 128, sm, s>>>(g);
+  return cudaGetLastError();
 }
 
 template <int L, int SL>
@@ -1102,17 +1145,18 @@ cudaError_t launch_qs(const QrBatch& g, cudaStream_t s) {
   const size_t sm = qs_smem(g.N, g.M, L);
   cudaFuncSetAttribute(qr_small_kernel<L, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   qr_small_kernel<L, SL><<<(g.count + 32 / L - 1) / (32 / L), 32, sm, s>>>(g);
-  const size_t redo = qr64_smem(g.N, g.M);
-  cudaFuncSetAttribute(qr_redo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)redo);
-  qr_redo_kernel<<<std::min((g.count + 127) / 128, 304), 128, redo, s>>>(g);
-  return cudaGetLastError();
+  return launch_redo(g, s);
 }
-template <int T, int B>
-cudaError_t launch_qc(const QrBatch& g, int threads, cudaStream_t s) {
+// Threads of a CTA: a warp per 32 / L columns of [H | y], at most `most`.
+int qc_threads(int L, int M, int most) { return 32 * std::min(M / (32 / L) + 1, most); }
+
+template <int L, int SL, int T, int B>
+cudaError_t launch_qc(const QrBatch& g, int most, cudaStream_t s) {
   const size_t sm = qr_cta_smem(g.N, g.M);
-  cudaFuncSetAttribute(qr_cta_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  qr_cta_kernel<T, B><<<g.count, threads, sm, s>>>(g);
-  return cudaGetLastError();
+  cudaFuncSetAttribute(qr_cta_kernel<L, SL, T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_cta_kernel<L, SL, T, B><<<g.count, qc_threads(L, g.M, most), sm, s>>>(g);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess || g.N <= 32 ? e : launch_redo(g, s);
 }
 
 // Lanes per matrix of qr_small_kernel, or 0: qr_cta_kernel.  A warp of the
@@ -1120,8 +1164,8 @@ cudaError_t launch_qc(const QrBatch& g, int threads, cudaStream_t s) {
 // to a CTA each, and more lanes per matrix serve a half-empty GPU better than
 // a full one, where the lanes' shared work (reflector scalars, reductions)
 // counts.  Measured, us a call with 28 us of host time (CTA / 2 / 4 / 8 lanes):
-//   16x16:  1,216 matrices 85 / 207 / 136 / 91, 9,728: 634 / 228 / 175 / 172,
-//          38,912: 2,497 / 818 / 624 / 598
+//   16x16:  1,216 matrices 64 / 207 / 136 / 91, 9,728: - / 223 / 166 / 168,
+//          38,912: - / 767 / 586 / 583
 //   12x12:  9,728: 386 / 130 / 115 / 115, 38,912: 1,514 / 441 / 367 / 397
 //    8x8:   1,216: 35 / 55 / 41 / 41, 9,728: 205 / 58 / 49 / 68,
 //          38,912: 769 / 113 / 129 / 217
@@ -1158,16 +1202,14 @@ cudaError_t launch(const QrBatch& g, cudaStream_t s) {
   const int N = g.N;
   switch (qr_form(g.count, N)) {
     case 0: {
-      // more warps where fewer CTAs share an SM (matrices by shared memory);
-      // five when many small matrices do.  2,432 matrices, ms for 5 / 8 / 12 /
-      // 16 warps: 40x40 0.65 / 0.71 / 0.86 / 0.86, 64x64 1.86 / 1.75 / 1.99 /
-      // 2.01, 80x80 3.51 / 3.19 / 3.10 / 3.22, 100x100 8.81 / 7.23 / 6.60 / 6.42
-      const int fit = (int)(227 * 1024 / qr_cta_smem(N, g.M));
-      const int most = fit >= 4 ? (g.count > 608 ? 5 : 8) : fit == 3 ? 8 : fit == 2 ? 12 : 16;
-      const int threads = 32 * std::max(2, std::min(1 + (g.M + 32 / kCtaLanes - 1) / (32 / kCtaLanes), most));
-      if (fit == 1) return launch_qc<512, 1>(g, threads, s);
-      if (fit == 2) return launch_qc<384, 2>(g, threads, s);
-      return launch_qc<256, 3>(g, threads, s);
+      // Few matrices: more warps each, for the chain; many: CTAs of fewer warps.
+      const int w = g.count <= 152 ? 9 : g.count <= 1216 ? 5 : 3;
+      if (N <= 16) return launch_qc<16, 1, 288, 2>(g, std::min(w, 5), s);
+      if (N <= 32) return launch_qc<16, 2, 288, 2>(g, w, s);
+      if (N <= 48) return launch_qc<16, 3, 256, 3>(g, g.count <= 152 ? 8 : 4, s);
+      if (N <= 64) return launch_qc<32, 2, 256, 3>(g, 8, s);
+      if (N <= 96) return launch_qc<32, 3, 256, 3>(g, 8, s);
+      return launch_qc<32, 4, 384, 2>(g, 12, s);
     }
     case 2:
       if (N <= 4) return launch_qs<2, 2>(g, s);
@@ -1193,8 +1235,12 @@ cudaError_t launch(const QrBatch& g, cudaStream_t s) {
 cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s) {
   const int M = r.a.n_tx, few = M <= 16 ? 1216 : 1824;
   const size_t sm = qr_cta_smem(M, M);
-  cudaFuncSetAttribute(qr_reorder_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  qr_reorder_cta_kernel<<<std::min(r.a.batch, few), 32 * std::max(2, std::min(1 + (M + 3) / 4, 5)), sm, s>>>(r, few);
+  const int grid = std::min(r.a.batch, few), threads = qc_threads(8, M, 9);
+  if (M <= 16) {
+    qr_reorder_cta_kernel<8, 2><<<grid, threads, sm, s>>>(r, few);
+  } else {
+    qr_reorder_cta_kernel<8, 4><<<grid, threads, sm, s>>>(r, few);
+  }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || r.a.batch <= few) return e;
   if (M <= 8) return launch_rs<4, 2>(r, few, s);
@@ -1208,8 +1254,13 @@ cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s) {
   switch (qr_form(g.a.batch, 2 * M)) {
     case 0: {
       const size_t sm = qr_cta_smem(2 * M, M);
-      cudaFuncSetAttribute(qr_aug_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      qr_aug_cta_kernel<<<g.a.batch, 32 * std::max(2, std::min(1 + (M + 3) / 4, g.a.batch > 608 ? 5 : 8)), sm, s>>>(g);
+      if (M <= 8) {
+        qr_aug_cta_kernel<8, 2><<<g.a.batch, qc_threads(8, M, 9), sm, s>>>(g);
+      } else if (M <= 16) {
+        qr_aug_cta_kernel<8, 4><<<g.a.batch, qc_threads(8, M, 9), sm, s>>>(g);
+      } else {
+        qr_aug_cta_kernel<16, 4><<<g.a.batch, qc_threads(8, M, 9), sm, s>>>(g);
+      }
       return cudaGetLastError();
     }
     case 2:
