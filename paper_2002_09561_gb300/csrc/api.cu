@@ -347,7 +347,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
   a.metric_out = dmet;
   a.vstatus = dvst;
   a.stats = dstats;
-  e = cudaMemsetAsync(c->counter, 0, 3 * sizeof(unsigned int), s);
+  e = cudaMemsetAsync(c->counter, 0, 8 * sizeof(unsigned int), s);
   if (e != cudaSuccess) return cuda_fail(c, e, "work counter reset");
   if (algo == ALGO_SD && (complex_tree || natural)) {
     // complex-tree or natural-order SD: the persistent warp-per-vector kernel on a uniform batch
@@ -426,7 +426,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
     e = launch_linear(AugArgs{a, c->sd_vstate, sd_vec_state_bytes(n), c->sd_order}, mmse, c->num_sms, s);
   } else {
     if (ev) cudaEventRecord(ev[1], s);
-    e = launch_hybrid(a, c->num_sms, s);
+    e = launch_hybrid(a, HybridWork{c->sd_vstate, sd_vec_state_bytes(n), c->sd_order, c->counter + 1}, c->num_sms, s);
   }
   if (e == cudaErrorInvalidConfiguration)
     return fail(c, MDX_EUNSUPPORTED, "no launch configuration fits this size");
@@ -960,7 +960,7 @@ mdx_status mdx_create(mdx_ctx** out, int device, int max_batch, int max_n_rx, in
   chk(alloc(c, &c->R32, B * tri_stride32(n)));
   chk(alloc(c, &c->yb32, B * vec_stride32(n)));
   chk(alloc(c, &c->singular, B));
-  chk(alloc(c, &c->counter, 4));
+  chk(alloc(c, &c->counter, 8));
   chk(alloc(c, &c->counts, 2));
   chk(alloc(c, &c->sH, B * max_n_rx * max_n_tx * 2));
   chk(alloc(c, &c->sy, B * max_n_rx * 2));

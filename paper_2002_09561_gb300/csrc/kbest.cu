@@ -16,7 +16,9 @@
 // over the S Q keys of a level (one bitonic sort in shared memory when K Q is
 // too large for register runs, kbest_levels_complex).
 //
-// Hybrid.  The master part enumerates every depth-d prefix (rows n-1..n-d),
+// Hybrid, for what the faster forms (hybrid_warp.cu) leave: K above 64, prefixes
+// of more than four rows, node budgets, ties among the candidates.  The master
+// part enumerates every depth-d prefix (rows n-1..n-d),
 // keeps those inside the initial sphere and sorts them by partial distance;
 // the CTA then finishes them best-first, each by a K-best run over the
 // remaining rows under the current radius (a run stops as soon as all its
@@ -77,33 +79,6 @@ struct KbLayout {
     bytes = round_up((int)o, 16);
   }
 };
-
-// Ascending bitonic sort of Cs (a power of two) keys by T threads.  Thread t
-// handles the pairs t, t + T, ...; for strides up to 32 a warp's pairs lie in
-// its own 64 consecutive keys (when T >= Cs / 2), so a stage followed by such a
-// stage needs only a warp barrier; every other transition takes the CTA barrier.
-__device__ __forceinline__ void bitonic_sort(uint64_t* keys, int Cs, int tid, int T) {
-  const bool warp_local = T >= (Cs >> 1);
-  for (int size = 2; size <= Cs; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int p = tid; p < (Cs >> 1); p += T) {
-        const int lo = ((p & ~(stride - 1)) << 1) | (p & (stride - 1));
-        const int hi = lo + stride;
-        const bool asc = (lo & size) == 0;
-        const uint64_t x = keys[lo], y = keys[hi];
-        if ((x > y) == asc) {
-          keys[lo] = y;
-          keys[hi] = x;
-        }
-      }
-      // the next stage's stride: half this one, or the next size's first
-      const int next = stride > 1 ? stride >> 1 : size;
-      if (warp_local && stride <= 32 && next <= 32) __syncwarp();
-      else __syncthreads();
-    }
-  }
-  __syncthreads();
-}
 
 struct KbCtx {
   int n, P, K, pp, tid, T;
@@ -859,7 +834,9 @@ __host__ __device__ inline void hy_layout(HyLayout& L, int n, int K, int P, int 
   L.bytes = o;
 }
 
-__global__ void hybrid_kernel(SearchArgs a, HyLayout L) {
+// redo: only the vectors listed there (*listed of them, taken from the counter next).
+__global__ void hybrid_kernel(SearchArgs a, HyLayout L, const unsigned char* redo, size_t stride, const unsigned int* listed,
+                              unsigned int* next) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, T = blockDim.x, warp = tid >> 5, lane = tid & 31;
   const int n = a.n, P = a.P, d = a.depth, K = a.K;
@@ -883,11 +860,12 @@ __global__ void hybrid_kernel(SearchArgs a, HyLayout L) {
   for (int l = 0; l < d; ++l) np *= P;
 
   for (;;) {
-    if (tid == 0) misc[0] = (int)atomicAdd(a.work_counter, 1u);
+    if (tid == 0) misc[0] = (int)atomicAdd(next, 1u);
     __syncthreads();
-    const int v = misc[0];
+    int v = misc[0];
     __syncthreads();
-    if (v >= a.batch) break;
+    if (v >= (redo ? (int)*listed : a.batch)) break;
+    if (redo) v = *reinterpret_cast<const int*>(redo + (size_t)v * stride);
     if (singular_vector(a, v)) continue;
     {
       KbLayout dummy;
@@ -1287,7 +1265,7 @@ bool hy_fit(HyLayout& L, int n, int K, int P, size_t sort_bytes) {
   return false;
 }
 
-cudaError_t launch_hybrid(const SearchArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t launch_hybrid(const SearchArgs& a, const HybridWork& w, int num_sms, cudaStream_t s) {
   if (a.batch <= 0) return cudaSuccess;
   int np = 1;
   for (int l = 0; l < a.depth; ++l) np *= a.P;
@@ -1304,7 +1282,11 @@ cudaError_t launch_hybrid(const SearchArgs& a, int num_sms, cudaStream_t s) {
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   int grid = per_sm * num_sms;
   if (grid > a.batch) grid = a.batch;
-  hybrid_kernel<<<grid, W * 32, L.bytes, s>>>(a, L);
+  e = launch_hybrid_warp(a, w, num_sms, s);
+  if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
+  const bool redo = e == cudaSuccess;
+  hybrid_kernel<<<grid, W * 32, L.bytes, s>>>(a, L, redo ? w.state + hybrid_redo_offset() : nullptr, w.stride, w.counts + 1,
+                                              redo ? w.counts + 2 : a.work_counter);
   return cudaGetLastError();
 }
 

@@ -1,15 +1,11 @@
 // K-best (Sec. VI) with one received vector per warp, by selection instead of
 // sorting.
 //
-// A level needs the set of the K smallest of the S P children, not their
-// order: the order enters the result only where children at exactly the same
-// FP32 distance straddle the cut (ties go to the lower parent rank, then the
-// lower child).  So every lane keeps the children of its survivors' as 32-bit
-// distance bits in registers (SL survivors of C children each), the K-th
-// smallest is found by a search on the bits (each step one compare and add
-// per child and one warp reduction; interpolated on the counts, then bisected
-// -- about six steps, since any value between the K-th and the next child will
-// do), and the children up to it are compacted in lane order.  Sorting 64-bit
+// The selection is that of select_run.cuh (here ties go to the lower parent
+// rank, then the lower child): every lane keeps the children of its survivors
+// as 32-bit distance bits in registers (SL survivors of C children each), and a
+// search on the bits (one compare and add per child and one warp reduction a
+// step) finds the K-th smallest.  Sorting 64-bit
 // keys, the ALU work that bound the CTA kernel (kbest.cu), disappears, and so
 // do its CTA barriers.  A vector whose cut a tie straddles (about 1 in 3,000
 // at K = 64, 16x16) is marked and left to that kernel, which sorts.
@@ -23,7 +19,7 @@
 // 100,000 vectors 19.7 -> 5.5 ms; complex tree 16x16 64-QAM K = 32, 20,000
 // vectors 14.8 -> 2.3 ms; 8x8 64-QAM K = 16 from host memory, 50,000 vectors
 // 2.29 -> 1.2 ms.
-#include "warp_kbest.cuh"
+#include "select_run.cuh"
 
 namespace mdx {
 namespace {
@@ -93,48 +89,6 @@ __device__ __forceinline__ float interference1(const float* Rc, const float* yb,
       if (b + m < d) c = fmaf(-Rc[col_off(n - 1 - b - m) + i], level_of(w, m, alpha), c);
   }
   return c;
-}
-
-// The bits T such that exactly K of the warp's keys are <= T, or false if a
-// tie straddles the K-th (more than K keys are valid; hi: a value with at
-// least K keys up to it).
-template <int N>
-__device__ __forceinline__ bool select_cut(const unsigned (&key)[N], int K, unsigned lo, unsigned hi, int n_hi,
-                                           unsigned& T) {
-  // invariant: fewer than K keys are <= lo, more than K are <= hi
-  int n_lo = 0;
-  if (n_hi == K) {
-    T = hi;
-    return true;
-  }
-  for (int it = 0; hi - lo > 1u; ++it) {
-    const unsigned gap = hi - lo;
-    // where a uniform density would put the middle of the K-th gap, bisection
-    // every third step and once the counts stop helping
-    unsigned step = gap >> 1;
-    if (it % 3 != 2) {
-      const float f = ((float)(K - n_lo) + 0.5f) * __frcp_rn((float)(n_hi - n_lo) + 1.0f);
-      step = (unsigned)((float)gap * fminf(f, 1.0f));
-      step = min(max(step, 1u), gap - 1u);
-    }
-    const unsigned mid = lo + step;
-    int c = 0;
-#pragma unroll
-    for (int j = 0; j < N; ++j) c += key[j] <= mid ? 1 : 0;
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (c == K) {
-      T = mid;
-      return true;
-    }
-    if (c < K) {
-      lo = mid;
-      n_lo = c;
-    } else {
-      hi = mid;
-      n_hi = c;
-    }
-  }
-  return false;
 }
 
 // SL survivors per lane (K <= 32 SL), C children per survivor: the PAM size P
@@ -229,64 +183,13 @@ __global__ void __launch_bounds__(kWarps * 32) kbest_warp_kernel(SearchArgs a, K
       }
       nodes += S;
       flops += CPLX ? (long long)S * (4 * (n - 1 - i) + 10 * C) : (long long)S * (2 * (n - 1 - i) + 4 * C);
-      // ---- the cut
-      unsigned T = 0xfffffffeu;
+      unsigned T;
       int kept;
-      {
-        int valid = 0;
-        unsigned least = 0xffffffffu, most = 0u, own = 0u;
-#pragma unroll
-        for (int q = 0; q < SL; ++q) {
-          unsigned low = 0xffffffffu;
-#pragma unroll
-          for (int k = 0; k < C; ++k) {
-            const unsigned x = key[q * C + k];
-            valid += x != 0xffffffffu ? 1 : 0;
-            low = min(low, x);
-            most = max(most, x + 1u);  // (an empty key counts as 0)
-          }
-          least = min(least, low);
-          if (lane + 32 * q < S) own = max(own, low);
-        }
-        valid = __reduce_add_sync(0xffffffffu, valid);
-        kept = min(valid, K);
-        if (valid > K) {
-          least = __reduce_min_sync(0xffffffffu, least);
-          // the largest of the survivors' best children bounds the S smallest
-          const unsigned far = __reduce_max_sync(0xffffffffu, own);
-          unsigned hi = __reduce_max_sync(0xffffffffu, most) - 1u;
-          int n_hi = valid;
-          if (S >= K && far < hi) {
-            int c = 0;
-#pragma unroll
-            for (int j = 0; j < SL * C; ++j) c += key[j] <= far ? 1 : 0;
-            n_hi = __reduce_add_sync(0xffffffffu, c);
-            hi = far;
-          }
-          if (!select_cut<SL * C>(key, K, least - 1u, hi, n_hi, T)) {
-            tie = true;
-            break;
-          }
-        }
+      if (!level_cut<SL, C>(key, S, K, lane, T, kept)) {
+        tie = true;
+        break;
       }
-      // ---- compaction in lane order
-      int mine = 0;
-#pragma unroll
-      for (int j = 0; j < SL * C; ++j) mine += key[j] <= T ? 1 : 0;
-      int at = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, at, o);
-        if (lane >= o) at += t;
-      }
-      at -= mine;
-#pragma unroll
-      for (int j = 0; j < SL * C; ++j) {
-        if (key[j] <= T) {
-          ent[at] = make_uint2((unsigned)(lane + 32 * (j / C)) | ((unsigned)(j % C) << 16), key[j]);
-          ++at;
-        }
-      }
+      compact_level<SL, C>(key, T, ent, lane);
       __syncwarp();
       // ---- the new survivors' paths: the parent's rows so far and the child's
       const int wd = d >> 2, sh = 8 * (d & 3);  // a complex level's two rows share a word (d is even)

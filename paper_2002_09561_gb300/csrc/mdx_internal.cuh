@@ -190,7 +190,18 @@ constexpr int kKbestRedo = 2;
 cudaError_t launch_kbest_warp(const SearchArgs& a, bool eight, cudaStream_t s);
 // Shared memory of the K-best kernel for (n, K, P, key capacity).
 size_t kbest_smem_bytes(int n, int K, int P, bool complex_tree);
-cudaError_t launch_hybrid(const SearchArgs& a, int num_sms, cudaStream_t s);
+// Workspace of the hybrid: vectors handed from form to form.
+struct HybridWork {
+  unsigned char* state;  // batch x stride: per-vector radius, candidates and counts (sd_vec_state_bytes(n));
+                         // entry i also holds number i of the vectors left to the sorting form
+  size_t stride;
+  int* list;             // batch: vectors with prefixes left after their first run, few in front, many behind
+  unsigned int* counts;  // few, left, the sorting form's next, many, the large CTAs' next; zero before
+};
+cudaError_t launch_hybrid(const SearchArgs& a, const HybridWork& w, int num_sms, cudaStream_t s);
+size_t hybrid_redo_offset();  // of that number in an entry
+// The forms of hybrid_warp.cu, or cudaErrorNotSupported.
+cudaError_t launch_hybrid_warp(const SearchArgs& a, const HybridWork& w, int num_sms, cudaStream_t s);
 // Linear detectors (linear.cu): ZF or MMSE on the QR workspace.
 size_t linear_smem_bytes(int n, bool mmse);
 cudaError_t launch_linear(const AugArgs& g, bool mmse, int num_sms, cudaStream_t s);
@@ -383,6 +394,7 @@ __device__ __forceinline__ float error_scale_warp(int n, int P, float alpha, con
   return __shfl_sync(0xffffffffu, sqrtf(warp_sum(e2)) * kU32, 0);
 }
 
+#pragma unroll 8
 __host__ __device__ __forceinline__ int pow2ceil(int x) {
   int p = 1;
   while (p < x) p <<= 1;
