@@ -66,7 +66,9 @@ struct mdx_ctx {
   size_t mx_gslot = 16;
   unsigned char* mx_scratch = nullptr;
   size_t mx_scratch_bytes = 0;
-  int mx_W = 8, mx_slice = 12288;
+  int mx_W = 8, mx_slice = 14336;
+  int mx_walks = 0;     // exact SDs of the uploaded table, first in its order
+  int mx_used = 14336;  // the slice of the uploaded table (its walks' records at least)
   std::vector<std::pair<unsigned long long, int>> mx_modes;  // class key -> MIX_* bits
   cudaGraphExec_t mx_graph = nullptr;
   std::vector<const void*> mx_graph_key;
@@ -399,7 +401,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
     }
     m.gscratch = c->mx_scratch;
     if (ev) cudaEventRecord(ev[1], s);
-    e = launch_mixed(m, c->mx_W, 0, c->num_sms, s);
+    e = launch_mixed(m, 0, c->mx_W, 0, c->num_sms, s);
   } else if (algo == ALGO_SD) {
     if (ev) cudaEventRecord(ev[1], s);
     // The antenna order is the search's own business where nothing that the
@@ -453,13 +455,6 @@ unsigned long long class_key(const mdx_request& q) {
          ((unsigned long long)q.algo << 24) | ((unsigned long long)(q.algo == MDX_ALGO_KBEST ? q.K : 0) << 32);
 }
 
-bool mode_fits(int mode, int algo, int n, int K, int slice) {
-  size_t need = 0;
-  if (mode & MIX_STAGE_R) need += mixed_stage_bytes(n);
-  if (mode & MIX_STATE_SMEM) need += mixed_state_bytes(algo, n, K, 0);
-  return need <= (size_t)slice;
-}
-
 // Most shared-memory use that fits: everything, else the state, else R.
 int greedy_mode(int algo, int n, int K, int slice) { return mixed_greedy_mode(algo, n, K, 0, slice); }
 
@@ -467,7 +462,7 @@ int mode_for(const mdx_ctx* c, const mdx_request& q) {
   const int n = 2 * q.n_tx;
   const unsigned long long k = class_key(q);
   for (const auto& e : c->mx_modes)
-    if (e.first == k && mode_fits(e.second, q.algo, n, q.K, c->mx_slice)) return e.second;
+    if (e.first == k && mixed_mode_fits(e.second, q.algo, n, q.K, c->mx_slice)) return e.second;
   return greedy_mode(q.algo, n, q.K, c->mx_slice);
 }
 
@@ -504,7 +499,7 @@ mdx_status mixed_upload(mdx_ctx* c, int nreq, const mdx_request* reqs, cudaStrea
   if (same_table(c, nreq, reqs)) return MDX_OK;
   std::vector<MixedReq> d((size_t)nreq);
   long long roff = 0, yoff = 0;
-  int maxK = 0;
+  int maxK = 0, slice = c->mx_slice;
   size_t gslot = 16;
   std::vector<std::pair<double, int>> cost((size_t)nreq);
   for (int r = 0; r < nreq; ++r) {
@@ -534,14 +529,17 @@ mdx_status mixed_upload(mdx_ctx* c, int nreq, const mdx_request* reqs, cudaStrea
     roff += tri_stride32(m.n);
     yoff += vec_stride32(m.n);
     if (m.K > maxK) maxK = m.K;
-    if (!(m.mode & MIX_STATE_SMEM)) gslot = std::max(gslot, mixed_state_bytes(m.algo, m.n, m.K, m.P));
+    gslot = std::max(gslot, mixed_slot_bytes(m.mode, m.algo, m.n, m.K));
+    slice = std::max(slice, mixed_least_slice(m.algo, m.n, m.K));
     // a cost proxy for the order: the exact SD's tree grows fastest with n
     const double n = m.n;
     cost[r].first = (m.algo != MDX_ALGO_KBEST) ? n * n * n * m.P : n * m.K * (n + 8.0 * m.P);
     cost[r].second = r;
   }
-  std::stable_sort(cost.begin(), cost.end(),
-                   [](const std::pair<double, int>& a, const std::pair<double, int>& b) { return a.first > b.first; });
+  auto walk = [&](int r) { return reqs[r].algo == MDX_ALGO_SD; };
+  std::stable_sort(cost.begin(), cost.end(), [&](const std::pair<double, int>& a, const std::pair<double, int>& b) {
+    return walk(a.second) != walk(b.second) ? walk(a.second) : a.first > b.first;
+  });
   // QR runs: requests grouped by (n_rx, n_tx)
   std::vector<int> ids((size_t)nreq);
   for (int r = 0; r < nreq; ++r) ids[r] = r;
@@ -590,8 +588,8 @@ mdx_status mixed_upload(mdx_ctx* c, int nreq, const mdx_request* reqs, cudaStrea
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(c, e, "descriptor upload");
   // per-warp global state slots for the requests whose state is not in shared memory
-  const int warps = mixed_resident_warps(c->mx_W, c->mx_slice, maxK, c->num_sms);
-  if (warps < 1) return fail(c, MDX_EUNSUPPORTED, "no launch of %d warps x %d bytes fits", c->mx_W, c->mx_slice);
+  const int warps = mixed_resident_warps(c->mx_W, slice, maxK, c->num_sms);
+  if (warps < 1) return fail(c, MDX_EUNSUPPORTED, "no launch of %d warps x %d bytes fits", c->mx_W, slice);
   const size_t sbytes = (size_t)warps * gslot;
   if (c->mx_scratch_bytes < sbytes) {
     if (c->mx_graph) {
@@ -609,6 +607,8 @@ mdx_status mixed_upload(mdx_ctx* c, int nreq, const mdx_request* reqs, cudaStrea
   c->mx_qr = runs;
   c->mx_maxK = maxK;
   c->mx_gslot = gslot;
+  c->mx_used = slice;
+  c->mx_walks = (int)std::count_if(reqs, reqs + nreq, [](const mdx_request& q) { return q.algo == MDX_ALGO_SD; });
   ++c->mx_gen;
   return MDX_OK;
 }
@@ -627,7 +627,7 @@ cudaError_t mixed_launches(mdx_ctx* c, int nreq, const double* dH, const double*
                                            dreqs, dH, dy, q, s);
     if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaMemsetAsync(c->counter, 0, sizeof(unsigned int), s);
+  cudaError_t e = cudaMemsetAsync(c->counter, 0, 2 * sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], s);
   MixedArgs a{};
@@ -643,13 +643,13 @@ cudaError_t mixed_launches(mdx_ctx* c, int nreq, const double* dH, const double*
   a.counter = c->counter;
   a.gscratch = c->mx_scratch;
   a.gslot_bytes = c->mx_gslot;
-  a.slice_bytes = c->mx_slice;
+  a.slice_bytes = c->mx_used;
   a.flags = flags;
   a.sym_out = dsym;
   a.metric_out = dmet;
   a.vstatus = dvst;
   a.stats = dstats;
-  e = launch_mixed(a, c->mx_W, c->mx_maxK, c->num_sms, s);
+  e = launch_mixed(a, c->mx_walks, c->mx_W, c->mx_maxK, c->num_sms, s);
   if (ev && e == cudaSuccess) cudaEventRecord(ev[2], s);
   return e;
 }
@@ -843,7 +843,7 @@ mdx_status run_autotune(mdx_ctx* c, int nreq, const mdx_request* reqs, const dou
     int win = greedy;
     float win_ms = INFINITY;
     for (int m : {greedy, 0, (int)MIX_STAGE_R, (int)MIX_STATE_SMEM, (int)(MIX_STAGE_R | MIX_STATE_SMEM)}) {
-      if (!mode_fits(m, q0.algo, n, q0.K, bestS) || (m == greedy && win_ms < INFINITY)) continue;
+      if (!mixed_mode_fits(m, q0.algo, n, q0.K, bestS) || (m == greedy && win_ms < INFINITY)) continue;
       std::vector<std::pair<unsigned long long, int>> trial = modes;
       trial.push_back({k, m});
       set_tuning(c, bestW, bestS, trial);

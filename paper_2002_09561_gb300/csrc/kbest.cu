@@ -18,15 +18,15 @@
 //
 // Hybrid, for what the faster forms (hybrid_warp.cu) leave: K above 64, prefixes
 // of more than four rows, node budgets, ties among the candidates.  The master
-// part enumerates every depth-d prefix (rows n-1..n-d),
-// keeps those inside the initial sphere and sorts them by partial distance;
-// the CTA then finishes them best-first, each by a K-best run over the
-// remaining rows under the current radius (a run stops as soon as all its
-// survivors leave the sphere), and shrinks the radius with the run's best
-// leaf: the best prefix on the whole CTA (cta_kbest_levels), the others one
-// per warp (warp_kbest) on the warps that hold a K-best workspace.  Prefixes are taken while their own partial distance is inside the
-// sphere; the first one outside ends the vector, since all later ones are
-// farther.  The answer is the best K-best leaf over the prefixes inside the
+// part enumerates every depth-d prefix (rows n-1..n-d), keeps those inside the
+// initial sphere and sorts them by partial distance; the CTA then finishes them
+// best-first, each by a K-best run over the remaining rows under the current
+// radius (a run stops as soon as all its survivors leave the sphere), and
+// shrinks the radius with the run's best leaf: the best prefix on the whole CTA
+// (cta_kbest_levels), the others one per warp (warp_kbest) on the warps that
+// hold a K-best workspace.  Prefixes are taken while their own partial distance
+// is inside the sphere; the first one outside ends the vector, since all later
+// ones are farther.  The answer is the best K-best leaf over the prefixes inside the
 // initial sphere, whatever the order, because a radius above the answer only
 // removes nodes that could not lead to it.
 //

@@ -162,9 +162,16 @@ size_t mixed_stage_bytes(int n);
 size_t mixed_state_bytes(int algo, int n, int K, int P);
 // Warps a launch with this shape keeps resident (for sizing gscratch).
 int mixed_resident_warps(int warps_per_cta, int slice_bytes, int max_K, int num_sms);
-cudaError_t launch_mixed(const MixedArgs& a, int warps_per_cta, int max_K, int num_sms, cudaStream_t s);
+// The first `walks` requests of the order are exact SDs in sorted order; uses
+// counter[0] and counter[1], zero before.
+cudaError_t launch_mixed(const MixedArgs& a, int walks, int warps_per_cta, int max_K, int num_sms, cudaStream_t s);
 // Placement of a uniform batch's vectors for a slice size (MIX_* bits).
 int mixed_greedy_mode(int algo, int n, int K, int P, int slice_bytes);
+// Whether a placement fits the slice; the bytes of global slot it needs.
+bool mixed_mode_fits(int mode, int algo, int n, int K, int slice_bytes);
+size_t mixed_slot_bytes(int mode, int algo, int n, int K);
+// The least slice a request's form needs.
+int mixed_least_slice(int algo, int n, int K);
 // Global workspace of the sphere decoder's task queue (see sd.cu).
 struct SdWorkspace {
   void* shared;          // sd_shared_bytes()
@@ -387,6 +394,7 @@ __device__ __forceinline__ float error_scale_warp(int n, int P, float alpha, con
   float e2 = 0.0f;
   for (int r = lane; r < n; r += 32) {
     float T = fabsf(yb[r]);
+#pragma unroll 8
     for (int j = r; j < n; ++j) T += amax * fabsf(Rc[col_off(j) + r]);
     const float w = (float)(n - r + 1) * T;
     e2 += w * w;
@@ -394,7 +402,6 @@ __device__ __forceinline__ float error_scale_warp(int n, int P, float alpha, con
   return __shfl_sync(0xffffffffu, sqrtf(warp_sum(e2)) * kU32, 0);
 }
 
-#pragma unroll 8
 __host__ __device__ __forceinline__ int pow2ceil(int x) {
   int p = 1;
   while (p < x) p <<= 1;

@@ -6,23 +6,26 @@
 // the host chose (heaviest classes first), and searches each one alone:
 //   exact SD   Algorithm 1 with Schnorr-Euchner child order (Sec. IV-A) and
 //              incremental partial distances (Eq. inc), one warp walking the
-//              whole tree: lanes own rows, the residual of every row below the
-//              current level sits in a stack zs[level][row], so a descent
-//              costs one FMA per lower row, every lane forms the next
-//              interference from row i - 1 itself, and a node whose nearest
-//              child is outside the sphere is counted but not entered;
-//   K-best     Sec. VI, selection of the K best children per level by a
-//              warp tournament over the survivors' Schnorr-Euchner child
-//              streams (warp_kbest.cuh).
+//              whole tree (sd_walk);
+//   K-best     Sec. VI, selection of the K best children per level
+//              (select_run.cuh for K <= 64; for larger K a warp tournament over
+//              the survivors' Schnorr-Euchner child streams, warp_kbest.cuh).
+// What bounds a batch is the longest walk: one warp, one node after another,
+// thousands of them, or one K-best level after another.  Both are therefore
+// written for the latency of a step (see sd_walk), and the grid holds as many
+// warps as the shared memory of a walk allows.
 // Each warp owns a slice of the CTA's shared memory and a slot of global
-// memory.  Per request class the tuner decides whether R and ybar are copied
-// into the slice (MIX_STAGE_R) and whether the search state (SD stacks and
-// leaf candidates, or K-best survivor paths) lives in the slice
+// memory.  SD walks and K-best selections use what fits of them by themselves.
+// For the other forms (natural-order and complex-tree SD, K > 64) the tuner
+// decides per request class whether R and ybar are copied into the slice
+// (MIX_STAGE_R) and whether the search state lives in the slice
 // (MIX_STATE_SMEM) or in the global slot; the kernel uses generic pointers,
 // so one code path serves every placement.  Leaves within the FP32 error
 // bound of the best are re-scored in FP64 against the FP64 R and ybar.
+#include <algorithm>
+
 #include "mdx_internal.cuh"
-#include "warp_kbest.cuh"
+#include "select_run.cuh"
 
 namespace mdx {
 namespace {
@@ -37,7 +40,7 @@ __host__ __device__ inline int mix_path_pad(int n) { return round_up(n, 16); }
 
 __host__ __device__ inline size_t sd_state_bytes(int n) {
   const size_t n4 = (size_t)round_up(n, 4);
-  const size_t b = sizeof(float) * (round_up(tri(n), 4) + 5 * n4) + sizeof(int) * n4 + sizeof(float) * kMixCand +
+  const size_t b = sizeof(float) * (round_up(tri(n), 4) + 3 * n4) + sizeof(int) * n4 + sizeof(float) * kMixCand +
                    (size_t)mix_path_pad(n) * (1 + kMixCand);
   return (b + 15) / 16 * 16;
 }
@@ -125,37 +128,50 @@ __device__ void finish_request(const MixedArgs& g, const MixedReq& q, int r, con
   }
 }
 
-// Exact SD of one request by one warp (ROWS = rows per lane, n <= 32 ROWS).
-// In Schnorr-Euchner order a visited node's next sibling is evaluated with
-// it; outside the sphere it finishes the level (the bound only shrinks), and
-// a pop goes straight to the nearest level above with a sibling left inside
-// (each level keeps that return level), so no iteration is spent climbing
-// through finished levels.  NAT: children in natural index order (the
-// unsorted depth-first search the paper compares against, Sec. IV-A)
-// instead; a child outside the sphere then does not end its level, and pops
-// go up one level at a time.
-template <int ROWS, bool NAT>
-__device__ void sd_request(const MixedArgs& g, const MixedReq& q, int r, const float* Rc, const float* yb,
+// Keeps the leaf xs at distance ped among the kMixCand best.
+__device__ void keep_leaf(const uint8_t* xs, int n, float ped, uint8_t* cx, int cs, float* cped, int& ncand, int lane) {
+  int at = -1;
+  if (ncand < kMixCand) {
+    at = ncand;
+  } else {
+    float worst = -1.0f;
+    for (int t = 0; t < kMixCand; ++t)
+      if (cped[t] > worst) {
+        worst = cped[t];
+        at = t;
+      }
+    if (!(ped < worst)) at = -1;
+  }
+  __syncwarp();
+  if (at >= 0) {
+    for (int rr = lane; rr < n; rr += 32) cx[(size_t)at * cs + rr] = xs[rr];
+    if (lane == 0) cped[at] = ped;
+    if (at == ncand) ++ncand;
+  }
+  __syncwarp();
+}
+
+// Unsorted depth-first search (children in natural index order, the variant
+// the paper compares against, Sec. IV-A) of one request by one warp (ROWS =
+// rows per lane, n <= 32 ROWS): lanes own rows, the residual of every row below
+// the current level sits in a stack zs[level][row].  A child outside the sphere
+// does not end its level, and pops go up one level at a time.
+template <int ROWS>
+__device__ void sd_natural(const MixedArgs& g, const MixedReq& q, int r, const float* Rc, const float* yb,
                            unsigned char* st, float E, int lane) {
   const int n = q.n, P = q.P, n4 = round_up(n, 4);
-  const float alpha = q.alpha, uoff = 0.5f * (float)(P - 1);
+  const float alpha = q.alpha;
   float* zs = reinterpret_cast<float*>(st);
   float* lv_ped = zs + round_up(tri(n), 4);
   float* lv_c = lv_ped + n4;
-  float* lv_u = lv_c + n4;
-  float* lv_rii = lv_u + n4;
-  float* lv_rinv = lv_rii + n4;
-  int* lv_lohi = reinterpret_cast<int*>(lv_rinv + n4);
-  float* cped = reinterpret_cast<float*>(lv_lohi + n4);
+  float* lv_rii = lv_c + n4;
+  int* lv_k = reinterpret_cast<int*>(lv_rii + n4);
+  float* cped = reinterpret_cast<float*>(lv_k + n4);
   uint8_t* xs = reinterpret_cast<uint8_t*>(cped + kMixCand);
   uint8_t* cx = xs + mix_path_pad(n);
   const int cs = mix_path_pad(n);
 
-  for (int rr = lane; rr < n; rr += 32) {
-    const float d = Rc[col_off(rr) + rr];
-    lv_rii[rr] = d;
-    lv_rinv[rr] = 0.5f / (alpha * d);
-  }
+  for (int rr = lane; rr < n; rr += 32) lv_rii[rr] = Rc[col_off(rr) + rr];
   float r2_start = initial_r2(g, q, r);
   float r2 = r2_start;
   long long nodes = 0, peds = 0, flops = 0;
@@ -170,95 +186,35 @@ __device__ void sd_request(const MixedArgs& g, const MixedReq& q, int r, const f
     }
     __syncwarp();
     float bnd = prune_bound(r2, E, n);
-    int i = n - 1;
-    // sorted order: the level a pop from level i goes to, the nearest level
-    // above whose next child was inside the sphere when the path left it
-    // (n: none); the levels in between have no child left to try
-    int ret = n;
+    int i = n - 1, next = 0;
     float ped_par = 0.0f;
     float c = zs[col_off(i) + i];
     float rii = lv_rii[i];
-    float u = fmaf(c, lv_rinv[i], uoff);
-    int lo = NAT ? 0 : min(max((int)ceilf(u - 0.5f), 0), P - 1);
-    int hi = NAT ? P : lo + 1;
     ++nodes;
     flops += 4 * P;
     for (;;) {
-      int k = -1;
-      if (NAT) {
-        if (lo < P) k = lo++;
-      } else if (lo >= 0 || hi < P) {
-        if (hi >= P || (lo >= 0 && fabsf(u - (float)lo) <= fabsf((float)hi - u))) k = lo--;
-        else k = hi++;
+      if (next >= P) {
+        if (i == n - 1) break;  // the root is exhausted
+        ++i;                    // backtrack
+        ped_par = lv_ped[i];
+        c = lv_c[i];
+        rii = lv_rii[i];
+        next = lv_k[i];
+        continue;
       }
-      float ped = INFINITY;
-      if (k >= 0) {
-        const float d = fmaf(-rii, (float)(2 * k - (P - 1)) * alpha, c);
-        ped = fmaf(d, d, ped_par);
-        ++peds;
-      }
-      if (NAT && k >= 0 && !(ped < bnd)) continue;  // unsorted: try the next child
-      // sorted order: whether the level's next child (the one a later
-      // iteration would take) is outside the sphere now, evaluated with the
-      // same operations; the bound only shrinks, so then it is outside then
-      // and nothing at this level is left to try
-      auto level_done = [&]() {
-        if (lo < 0 && hi >= P) return true;
-        const int k2 = (hi >= P || (lo >= 0 && fabsf(u - (float)lo) <= fabsf((float)hi - u))) ? lo : hi;
-        const float d2 = fmaf(-rii, (float)(2 * k2 - (P - 1)) * alpha, c);
-        if (fmaf(d2, d2, ped_par) < bnd) return false;
-        ++peds;  // the evaluation that ends the level, made here
-        return true;
-      };
-      bool up = k < 0 || !(ped < bnd);
-      if (i == 0 && !up) {
-        // leaf inside the sphere: keep it among the kMixCand best, shrink the radius
-        int slot = -1;
-        if (lane == 0) {
-          xs[0] = (uint8_t)k;
-          if (ncand < kMixCand) {
-            slot = ncand;
-          } else {
-            float worst = -1.0f;
-            for (int t = 0; t < kMixCand; ++t)
-              if (cped[t] > worst) {
-                worst = cped[t];
-                slot = t;
-              }
-            if (!(ped < worst)) slot = -1;
-          }
-        }
-        slot = __shfl_sync(0xffffffffu, slot, 0);
+      const int k = next++;
+      const float d = fmaf(-rii, (float)(2 * k - (P - 1)) * alpha, c);
+      const float ped = fmaf(d, d, ped_par);
+      ++peds;
+      if (!(ped < bnd)) continue;
+      if (i == 0) {
+        if (lane == 0) xs[0] = (uint8_t)k;
         __syncwarp();
-        if (slot >= 0) {
-          for (int rr = lane; rr < n; rr += 32) cx[(size_t)slot * cs + rr] = xs[rr];
-          if (lane == 0) cped[slot] = ped;
-          if (slot == ncand) ++ncand;
-        }
-        __syncwarp();
+        keep_leaf(xs, n, ped, cx, cs, cped, ncand, lane);
         if (ped < r2) {
           r2 = ped;
           bnd = prune_bound(r2, E, n);
         }
-        if (NAT || !level_done()) continue;
-        up = true;
-      }
-      if (up) {
-        if (NAT) {
-          if (i == n - 1) break;  // the root is exhausted
-          ++i;                    // backtrack
-        } else {
-          if (ret >= n) break;  // no level above has a child left
-          i = ret;              // back to the nearest level with one
-        }
-        ped_par = lv_ped[i];
-        c = lv_c[i];
-        u = lv_u[i];
-        rii = lv_rii[i];
-        const int lh = lv_lohi[i];
-        lo = (lh & 0xff) - 1;
-        if (!NAT) ret = (lh >> 8) & 0xff;
-        hi = lh >> 16;
         continue;
       }
       if (q.budget > 0 && nodes >= q.budget) {
@@ -269,46 +225,13 @@ __device__ void sd_request(const MixedArgs& g, const MixedReq& q, int r, const f
       const float av = (float)(2 * k - (P - 1)) * alpha;
       const float* zin = zs + col_off(i);
       const float* rc = Rc + col_off(i);
-      // the next level's interference, computed by every lane from row i - 1
-      // (the same FMA as that row's residual below; the column was written
-      // before the last warp barrier), and the new level's first child, the
-      // PAM index nearest u (sorted order only): outside the sphere it rules
-      // out every child, so the node is counted with that one evaluation and
-      // the search goes on at level i
       const float cnext = fmaf(-rc[i - 1], av, zin[i - 1]);
-      const float unext = fmaf(cnext, lv_rinv[i - 1], uoff);
-      const int lonext = NAT ? 0 : min(max((int)ceilf(unext - 0.5f), 0), P - 1);
-      bool done_here = false;
-      if (!NAT) {
-        const float d1 = fmaf(-lv_rii[i - 1], (float)(2 * lonext - (P - 1)) * alpha, cnext);
-        done_here = level_done();
-        if (!(fmaf(d1, d1, ped) < bnd)) {
-          ++nodes;
-          ++peds;
-          flops += 2 * (n - i) + 4 * P;
-          if (!done_here) continue;
-          // nothing else at this level: back to the return level
-          if (ret >= n) break;
-          i = ret;
-          ped_par = lv_ped[i];
-          c = lv_c[i];
-          u = lv_u[i];
-          rii = lv_rii[i];
-          const int lh = lv_lohi[i];
-          lo = (lh & 0xff) - 1;
-          ret = (lh >> 8) & 0xff;
-          hi = lh >> 16;
-          continue;
-        }
-      }
       if (lane == 0) {
         lv_ped[i] = ped_par;
         lv_c[i] = c;
-        lv_u[i] = u;
-        lv_lohi[i] = (lo + 1) | (NAT ? 0 : ret << 8) | (hi << 16);
+        lv_k[i] = next;
         xs[i] = (uint8_t)k;
       }
-      if (!NAT && !done_here) ret = i;
       float* zout = zs + col_off(i - 1);
 #pragma unroll
       for (int t = 0; t < ROWS; ++t) {
@@ -320,11 +243,278 @@ __device__ void sd_request(const MixedArgs& g, const MixedReq& q, int r, const f
       c = cnext;
       ped_par = ped;
       rii = lv_rii[i];
-      u = unext;
-      lo = lonext;
-      hi = NAT ? P : lo + 1;
+      next = 0;
       ++nodes;
       flops += 2 * (n - 1 - i) + 4 * P;
+    }
+    if (ncand == 0 && !bh && r2_start < INFINITY && restarts < 64) {
+      // empty sphere: r^2 <- 2 r^2 and search again
+      r2_start *= 2.0f;
+      r2 = r2_start;
+      ++restarts;
+      continue;
+    }
+    break;
+  }
+  __syncwarp();
+  const int status = bh ? MDX_V_BUDGET_EXCEEDED : (restarts > 0 ? MDX_V_EMPTY_RETRIED : MDX_V_OK);
+  finish_request(g, q, r, cx, cs, cped, ncand, E, status, nodes, peds, restarts, flops, lane);
+}
+
+// Schnorr-Euchner orders of a level's children as nibbles, by the first child
+// k0 and whether u lies above it: entry 2 k0 + (u > k0) for P = 2, 4, 8.  From
+// k0 (the index nearest u) the order alternates sides, starting on u's side
+// (below on a tie), until one side is used up: the order in which comparing
+// |u - lo| <= |hi - u| takes them, since within the constellation those
+// differences decide as in exact arithmetic (for u >= k0 both are multiples of
+// ulp(u) no larger than u, so exact; below k0 rounding cannot pass the integer
+// that separates them), and outside it only one side is left.
+constexpr unsigned zigzag(int P, int k0, bool above) {
+  unsigned w = (unsigned)k0;
+  int lo = k0 - 1, hi = k0 + 1;
+  for (int t = 1; t < P; ++t) {
+    const bool low = lo >= 0 && (hi >= P || k0 - lo < hi - k0 || (k0 - lo == hi - k0 && !above));
+    w |= (unsigned)(low ? lo-- : hi++) << (4 * t);
+  }
+  return w;
+}
+struct Zigzag {
+  unsigned at[3][16];
+  constexpr Zigzag() : at{} {
+    for (int p = 0; p < 3; ++p)
+      for (int k = 0; k < (2 << p); ++k) {
+        at[p][2 * k] = zigzag(2 << p, k, false);
+        at[p][2 * k + 1] = zigzag(2 << p, k, true);
+      }
+  }
+};
+__constant__ Zigzag kZigzag;
+
+// Exact SD of one request by one warp (ROWS = rows per lane, n <= 32 ROWS).
+// In Schnorr-Euchner order a visited node's next sibling is evaluated with it;
+// outside the sphere it finishes the level (the bound only shrinks), and a pop
+// goes straight to the nearest level above with a sibling left inside (each
+// level keeps that return level).  A node whose nearest child is outside the
+// sphere is counted but not entered.
+//
+// A walk is one dependent chain, so a step is kept short: every lane forms the
+// chain's values itself; what a level's descent will need (its column's entries
+// for the next rows, the residual two rows down, the next row's constants) is
+// loaded when the level is reached, and the next row's interference is one FMA
+// from it; each child is evaluated once, its sibling kept in the level's
+// record; the child order is a table of nibbles; indexes become levels in the
+// FP32 adder instead of by conversions.  The residuals of the current level
+// are in registers (lanes own rows), a stack zs[level][row] holds the levels
+// above for pops.  The lowest levels, where a walk spends its time, have R's
+// columns and the stack in the slice (as many as fit), the levels above in
+// global memory, so walks of every size leave the SM full; the placement is two
+// selected pointers, since branches cost more (n = 128: 9.6 ms for the 7.4).
+// Measured (333 requests of 64-QAM with the QR, walks up to 20,000 nodes; before:
+// the rows' update, the sibling and the first child evaluated one after
+// another, everything in global memory where the stack did not fit): n = 16
+// 6.8 -> 4.6 ms, n = 128 10.6 -> 7.7, n = 200 19 -> 8.9.
+__host__ __device__ inline size_t walk_record_bytes(int n) { return (sizeof(float4) + sizeof(float2)) * (size_t)n; }
+__host__ __device__ inline size_t walk_slot_bytes(int n) {
+  const size_t b = sizeof(float) * round_up(tri(n), 4) + sizeof(float) * kMixCand +
+                   (size_t)mix_path_pad(n) * kMixCand;
+  return (b + 15) / 16 * 16;
+}
+
+template <int ROWS>
+__device__ void sd_walk(const MixedArgs& g, const MixedReq& q, int r, const float* __restrict__ Rg,
+                        const float* __restrict__ yg, unsigned char* slot, float E, int lane) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned char* slice = smem + (size_t)(threadIdx.x >> 5) * g.slice_bytes;
+  const int n = q.n, P = q.P;
+  const float alpha = q.alpha, alpha2 = 2.0f * alpha, half = 0.5f * (float)(P - 1), mid = level_mid(P);
+  const unsigned* zz = kZigzag.at[P == 2 ? 0 : P == 4 ? 1 : 2];
+  // ---- placement (the slice holds the records at least)
+  float* zg = reinterpret_cast<float*>(slot);
+  float4* rec = reinterpret_cast<float4*>(slice);
+  float2* cst = reinterpret_cast<float2*>(rec + n);
+  float* cped = reinterpret_cast<float*>(slot + sizeof(float) * round_up(tri(n), 4));
+  uint8_t* cx = reinterpret_cast<uint8_t*>(cped + kMixCand);
+  const int cs = mix_path_pad(n);
+  const int room = (g.slice_bytes - (int)walk_record_bytes(n)) / 8 - 3;
+  int low = room > 0 ? min(n, (int)(0.5f * (sqrtf(8.0f * (float)room + 1.0f) - 1.0f))) : 0;  // levels in the slice
+  while (low > 0 && tri(low) > room) --low;
+  float* Rs = reinterpret_cast<float*>(cst + n);
+  float* zl = Rs + round_up(tri(low), 4);
+  for (int k = lane; k < tri(low); k += 32) Rs[k] = Rg[k];
+  for (int rr = lane; rr < n; rr += 32) {
+    const float d = Rg[col_off(rr) + rr];
+    cst[rr] = make_float2(d, 0.5f / (alpha * d));
+  }
+  __syncwarp();
+
+  float r2_start = initial_r2(g, q, r);
+  float r2 = r2_start;
+  const long long limit = q.budget > 0 ? q.budget : 0x7fffffffffffffffll;
+  long long nodes = 0, peds = 0, flops = 0;
+  int restarts = 0, ncand = 0;
+  bool bh = false;
+  for (;;) {
+    float z[ROWS], rc[ROWS];  // residuals at the current level, its column
+#pragma unroll
+    for (int t = 0; t < ROWS; ++t) z[t] = lane + 32 * t < n ? yg[lane + 32 * t] : 0.0f;
+    auto col = [&](int j) { return (j < low ? (const float*)Rs : Rg) + col_off(j); };
+    auto res = [&](int j) { return (j < low ? zl : zg) + col_off(j); };
+#pragma unroll
+    for (int t = 0; t < ROWS; ++t)
+      if (lane + 32 * t < n) res(n - 1)[lane + 32 * t] = z[t];
+    __syncwarp();
+    float bnd = prune_bound(r2, E, n);
+    int i = n - 1, ret = n;  // ret: the level a pop goes to (n: none)
+    float ped_par = 0.0f, c = yg[n - 1], z1 = yg[n - 2];
+    float2 ri = cst[n - 1];
+    float ra = 0.0f, rb = 0.0f, z2 = 0.0f;
+    float2 nx = make_float2(0.0f, 0.0f);
+    // what a descent from level i needs
+    auto reach = [&]() {
+      const float* rp = col(i);
+      if (i > 0) {
+        ra = rp[i - 1];
+        nx = cst[i - 1];
+      }
+      if (i > 1) {
+        rb = rp[i - 2];
+        z2 = res(i)[i - 2];
+      }
+#pragma unroll
+      for (int t = 0; t < ROWS; ++t) rc[t] = lane + 32 * t < i ? rp[lane + 32 * t] : 0.0f;
+    };
+    // the child nearest to u: its index, level and distance, and its order
+    auto first = [&](float cc, float2 rr, float par, int& k, float& lev, float& ped, int& pat) {
+      const float u = fmaf(cc, rr.y, half);
+      const float kf =
+          __fadd_ru(fminf(fmaxf(u - 0.5f, 0.0f), (float)(P - 1)), 8388608.0f) - 8388608.0f;
+      k = __float_as_int(kf + 8388608.0f) & 15;
+      lev = (kf - half) * alpha2;
+      pat = 2 * k + (u > kf ? 1 : 0);
+      const float d = fmaf(-rr.x, lev, cc);
+      ped = fmaf(d, d, par);
+    };
+    int k, pat, idx = 1;
+    float lev, ped;
+    first(c, ri, 0.0f, k, lev, ped, pat);
+    unsigned ord = zz[pat];
+    ++nodes;
+    flops += 4 * P;
+    ++peds;
+    bool inside = ped < bnd;
+    if (inside) reach();
+    while (inside) {
+      // child k of level i, inside the sphere
+      if (i == 0) {
+        // leaf: keep it among the kMixCand best, shrink the radius
+        int at = -1;
+        if (ncand < kMixCand) {
+          at = ncand;
+        } else {
+          float worst = -1.0f;
+          for (int t = 0; t < kMixCand; ++t)
+            if (cped[t] > worst) {
+              worst = cped[t];
+              at = t;
+            }
+          if (!(ped < worst)) at = -1;
+        }
+        __syncwarp();
+        if (at >= 0) {
+          for (int rr = lane; rr < n; rr += 32)
+            cx[(size_t)at * cs + rr] = (uint8_t)(rr == 0 ? k : __float_as_int(rec[rr].w) & 15);
+          if (lane == 0) cped[at] = ped;
+          if (at == ncand) ++ncand;
+        }
+        __syncwarp();
+        if (ped < r2) {
+          r2 = ped;
+          bnd = prune_bound(r2, E, n);
+        }
+      } else if (nodes >= limit) {
+        bh = true;
+        break;
+      }
+      // its next sibling: outside the sphere, nothing at this level is left
+      const bool more = idx < P;
+      const float lev2 = level_at(ord >> (4 * idx - 1), mid, alpha2);
+      const float d2 = fmaf(-ri.x, lev2, c);
+      const float ped2 = fmaf(d2, d2, ped_par);
+      const bool done = !(more && ped2 < bnd);
+      if (more && done) ++peds;
+      if (i > 0) {
+        // the next level's nearest child: outside the sphere it rules out every child
+        const float cn = fmaf(-ra, lev, z1);
+        int kn, patn;
+        float levn, pedn;
+        first(cn, nx, ped, kn, levn, pedn, patn);
+        ++nodes;
+        ++peds;
+        flops += 2 * (n - i) + 4 * P;
+        if (pedn < bnd) {
+          // descend: push level i, update the residuals of the rows below
+          rec[i] = make_float4(c, ped_par, ped2, __int_as_float(k | idx << 4 | pat << 8 | ret << 16));
+          if (!done) ret = i;
+          float* zo = res(i - 1);
+#pragma unroll
+          for (int t = 0; t < ROWS; ++t) {
+            z[t] = fmaf(-rc[t], lev, z[t]);
+            if (lane + 32 * t < i) zo[lane + 32 * t] = z[t];
+          }
+          z1 = fmaf(-rb, lev, z2);
+          --i;
+          c = cn;
+          ri = nx;
+          ped_par = ped;
+          k = kn;
+          lev = levn;
+          ped = pedn;
+          pat = patn;
+          ord = zz[pat];
+          idx = 1;
+          __syncwarp();
+          reach();
+          continue;
+        }
+      }
+      if (!done) {
+        k = (int)(ord >> (4 * idx)) & 15;
+        lev = lev2;
+        ped = ped2;
+        ++idx;
+        ++peds;
+        continue;
+      }
+      // back to the nearest level above with a child inside
+      inside = false;
+      float4 s4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      while (ret < n) {
+        i = ret;
+        s4 = rec[i];
+        ret = __float_as_int(s4.w) >> 16;
+        ++peds;
+        if (s4.z < bnd) {
+          inside = true;
+          break;
+        }
+      }
+      if (!inside) break;
+      const int w = __float_as_int(s4.w);
+      c = s4.x;
+      ped_par = s4.y;
+      ped = s4.z;
+      idx = (w >> 4) & 15;
+      pat = (w >> 8) & 15;
+      ord = zz[pat];
+      k = (int)(ord >> (4 * idx)) & 15;
+      lev = level_at(ord >> (4 * idx - 1), mid, alpha2);
+      ++idx;
+      ri = cst[i];
+      const float* zi = res(i);
+#pragma unroll
+      for (int t = 0; t < ROWS; ++t) z[t] = lane + 32 * t < i ? zi[lane + 32 * t] : 0.0f;
+      z1 = i > 0 ? zi[i - 1] : 0.0f;
+      reach();
     }
     if (ncand == 0 && !bh && r2_start < INFINITY && restarts < 64) {
       // empty sphere: r^2 <- 2 r^2 and search again
@@ -420,30 +610,12 @@ __device__ void sdc_request(const MixedArgs& g, const MixedReq& q, int r, const 
       const int kre = qk / P, kim = qk - kre * P;
       if (j == 0) {
         // leaf inside the sphere: keep it among the kMixCand best, shrink the radius
-        int slot = -1;
         if (lane == 0) {
           xs[1] = (uint8_t)kim;
           xs[0] = (uint8_t)kre;
-          if (ncand < kMixCand) {
-            slot = ncand;
-          } else {
-            float worst = -1.0f;
-            for (int t = 0; t < kMixCand; ++t)
-              if (cped[t] > worst) {
-                worst = cped[t];
-                slot = t;
-              }
-            if (!(ped < worst)) slot = -1;
-          }
-        }
-        slot = __shfl_sync(0xffffffffu, slot, 0);
-        __syncwarp();
-        if (slot >= 0) {
-          for (int rr = lane; rr < n; rr += 32) cx[(size_t)slot * cs + rr] = xs[rr];
-          if (lane == 0) cped[slot] = ped;
-          if (slot == ncand) ++ncand;
         }
         __syncwarp();
+        keep_leaf(xs, n, ped, cx, cs, cped, ncand, lane);
         if (ped < r2) {
           r2 = ped;
           bnd = prune_bound(r2, E, n);
@@ -539,19 +711,49 @@ __device__ void kb_request(const MixedArgs& g, const MixedReq& q, int r, const f
                  nodes * P, restarts, flops, lane);
 }
 
-template <int KSPL>
-__global__ void mixed_kernel(MixedArgs g) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
-  unsigned char* slice = smem + (size_t)warp * g.slice_bytes;
-  unsigned char* gslot = g.gscratch + ((size_t)blockIdx.x * W + warp) * g.gslot_bytes;
+// The same by selection (K <= 32 SL).
+template <int SL>
+__device__ void kb_select(const MixedArgs& g, const MixedReq& q, int r, const float* Rg, const float* yg,
+                          unsigned char* slice, unsigned char* slot, float E, int lane) {
+  const int n = q.n, P = q.P, K = q.K, cs = mix_path_pad(n);
+  const SelectWs ws = select_ws(slice, g.slice_bytes, slot, n, K);
+  float* cped = reinterpret_cast<float*>(ws.ent);
+  uint8_t* cx = slot + select_path_bytes(n, K);
+  for (int ranked = 0; ranked < 2; ++ranked) {
+    float r2 = initial_r2(g, q, r);
+    RunCost cost;
+    int restarts = 0, S = 0;
+    Survivors<SL> v;
+    for (;;) {
+      const float bnd = prune_bound(r2, E, n);
+#pragma unroll
+      for (int t = 0; t < SL; ++t) {
+        v.ped[t] = 0.0f;
+        v.cur[t] = 0u;
+      }
+      if (P == 8) S = select_run<SL, 8>(Rg, yg, n, K, q.alpha, 0, 1, bnd, ranked, ws, lane, v, cost);
+      else if (P == 4) S = select_run<SL, 4>(Rg, yg, n, K, q.alpha, 0, 1, bnd, ranked, ws, lane, v, cost);
+      else S = select_run<SL, 2>(Rg, yg, n, K, q.alpha, 0, 1, bnd, ranked, ws, lane, v, cost);
+      if (S != 0 || !(r2 < INFINITY) || restarts >= 64) break;
+      r2 *= 2.0f;  // every survivor left the sphere: r^2 <- 2 r^2
+      ++restarts;
+    }
+    if (S < 0 || !select_leaves<SL>(v, S, ranked, n, ws.x, ws.KS, cx, cs, cped, lane)) continue;
+    finish_request(g, q, r, cx, cs, cped, min(S, kCandMax), E, restarts > 0 ? MDX_V_EMPTY_RETRIED : MDX_V_OK,
+                   cost.nodes, cost.nodes * P, restarts, cost.flops, lane);
+    break;
+  }
+}
+
+// The next request of the launch's order to the calling warp (-1: none left),
+// its descriptor in q; singular ones are answered here.
+__device__ __forceinline__ int next_request(const MixedArgs& g, MixedReq& q, int lane) {
   for (;;) {
     unsigned int t = 0;
     if (lane == 0) t = atomicAdd(g.counter, 1u);
     t = __shfl_sync(0xffffffffu, t, 0);
-    if (t >= (unsigned int)g.nreq) break;
+    if (t >= (unsigned int)g.nreq) return -1;
     const int r = g.order ? g.order[t] : (int)t;
-    MixedReq q;
     if (g.reqs) {
       q = g.reqs[r];
     } else {
@@ -562,18 +764,51 @@ __global__ void mixed_kernel(MixedArgs g) {
       q.y_off64 = (long long)r * vec_stride64(q.n);
       q.sym_off = (long long)r * q.n_tx;
     }
-    if (g.singular[r]) {
-      for (int j = lane; j < q.n_tx; j += 32) g.sym_out[q.sym_off + j] = 0;
-      if (lane == 0) {
-        g.metric_out[r] = 0.0;
-        g.vstatus[r] = MDX_V_SINGULAR;
-        if (g.stats)
-          for (int k = 0; k < kStats; ++k) g.stats[(size_t)r * kStats + k] = 0;
-      }
-      continue;
+    if (!g.singular[r]) return r;
+    for (int j = lane; j < q.n_tx; j += 32) g.sym_out[q.sym_off + j] = 0;
+    if (lane == 0) {
+      g.metric_out[r] = 0.0;
+      g.vstatus[r] = MDX_V_SINGULAR;
+      if (g.stats)
+        for (int k = 0; k < kStats; ++k) g.stats[(size_t)r * kStats + k] = 0;
     }
+  }
+}
+
+// The walks have a kernel of their own: a step is a chain of a hundred
+// instructions, and registers spilled for the other forms' sake lengthen it
+// (the classes of sd_walk in one kernel with the selection: 6.5, 13.0, 14.9 ms).
+__global__ void __launch_bounds__(512) walk_kernel(MixedArgs g) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  unsigned char* gslot = g.gscratch + ((size_t)blockIdx.x * W + warp) * g.gslot_bytes;
+  MixedReq q;
+  for (int r; (r = next_request(g, q, lane)) >= 0; __syncwarp()) {
     const float* Rc = g.R32 + q.r_off;
     const float* yb = g.yb32 + q.y_off;
+    const float E = error_scale_warp(q.n, q.P, q.alpha, Rc, yb, lane);
+    if (q.n <= 32) sd_walk<1>(g, q, r, Rc, yb, gslot, E, lane);
+    else if (q.n <= 64) sd_walk<2>(g, q, r, Rc, yb, gslot, E, lane);
+    else if (q.n <= 128) sd_walk<4>(g, q, r, Rc, yb, gslot, E, lane);
+    else sd_walk<7>(g, q, r, Rc, yb, gslot, E, lane);
+  }
+}
+
+template <int KSPL>
+__global__ void __launch_bounds__(512) mixed_kernel(MixedArgs g) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  unsigned char* slice = smem + (size_t)warp * g.slice_bytes;
+  unsigned char* gslot = g.gscratch + ((size_t)blockIdx.x * W + warp) * g.gslot_bytes;
+  MixedReq q;
+  for (int r; (r = next_request(g, q, lane)) >= 0; __syncwarp()) {
+    const float* Rc = g.R32 + q.r_off;
+    const float* yb = g.yb32 + q.y_off;
+    if (q.algo == MDX_ALGO_KBEST && q.K <= 64) {
+      const float E = error_scale_warp(q.n, q.P, q.alpha, Rc, yb, lane);
+      if (q.K <= 32) kb_select<1>(g, q, r, Rc, yb, slice, gslot, E, lane);
+      else kb_select<2>(g, q, r, Rc, yb, slice, gslot, E, lane);
+      continue;
+    }
     unsigned char* st = gslot;
     if (q.mode & MIX_STAGE_R) {
       const int ts = tri_stride32(q.n);
@@ -590,45 +825,36 @@ __global__ void mixed_kernel(MixedArgs g) {
     }
     __syncwarp();
     const float E = error_scale_warp(q.n, q.P, q.alpha, Rc, yb, lane);
-    if (q.algo == MDX_ALGO_SD) {
-      if (q.n <= 32) sd_request<1, false>(g, q, r, Rc, yb, st, E, lane);
-      else if (q.n <= 64) sd_request<2, false>(g, q, r, Rc, yb, st, E, lane);
-      else if (q.n <= 128) sd_request<4, false>(g, q, r, Rc, yb, st, E, lane);
-      else sd_request<7, false>(g, q, r, Rc, yb, st, E, lane);
-    } else if (q.algo == MIX_ALGO_SD_NATURAL) {
-      if (q.n <= 32) sd_request<1, true>(g, q, r, Rc, yb, st, E, lane);
-      else if (q.n <= 64) sd_request<2, true>(g, q, r, Rc, yb, st, E, lane);
-      else if (q.n <= 128) sd_request<4, true>(g, q, r, Rc, yb, st, E, lane);
-      else sd_request<7, true>(g, q, r, Rc, yb, st, E, lane);
+    if (q.algo == MIX_ALGO_SD_NATURAL) {
+      if (q.n <= 32) sd_natural<1>(g, q, r, Rc, yb, st, E, lane);
+      else if (q.n <= 64) sd_natural<2>(g, q, r, Rc, yb, st, E, lane);
+      else if (q.n <= 128) sd_natural<4>(g, q, r, Rc, yb, st, E, lane);
+      else sd_natural<7>(g, q, r, Rc, yb, st, E, lane);
     } else if (q.algo == MIX_ALGO_SD_COMPLEX) {
       if (q.n <= 32) sdc_request<1>(g, q, r, Rc, yb, st, E, lane);
       else if (q.n <= 64) sdc_request<2>(g, q, r, Rc, yb, st, E, lane);
       else if (q.n <= 128) sdc_request<4>(g, q, r, Rc, yb, st, E, lane);
       else sdc_request<7>(g, q, r, Rc, yb, st, E, lane);
-    } else {
-      if (q.K <= 32) kb_request<1>(g, q, r, Rc, yb, st, E, lane);
-      else if (KSPL <= 2 || q.K <= 64) kb_request<2>(g, q, r, Rc, yb, st, E, lane);
-      else if constexpr (KSPL > 2) {
-        if (q.K <= 128) kb_request<4>(g, q, r, Rc, yb, st, E, lane);
-        else kb_request<8>(g, q, r, Rc, yb, st, E, lane);
-      }
+    } else if constexpr (KSPL > 2) {
+      if (q.K <= 128) kb_request<4>(g, q, r, Rc, yb, st, E, lane);
+      else kb_request<8>(g, q, r, Rc, yb, st, E, lane);
     }
-    __syncwarp();
   }
 }
 
-template <int KSPL>
-cudaError_t prepare(int W, int slice_bytes, int num_sms, int* grid) {
+cudaError_t prepare(const void* fn, int W, int slice_bytes, int num_sms, int* grid) {
   const int smem = W * slice_bytes;
-  cudaError_t e = cudaFuncSetAttribute(mixed_kernel<KSPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mixed_kernel<KSPL>, W * 32, (size_t)smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, W * 32, (size_t)smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   *grid = per_sm * num_sms;
   return cudaSuccess;
 }
+const void* walk_fn() { return (const void*)walk_kernel; }
+const void* mixed_fn(int max_K) { return max_K > 64 ? (const void*)mixed_kernel<8> : (const void*)mixed_kernel<2>; }
 
 }  // namespace
 
@@ -636,12 +862,16 @@ size_t mixed_stage_bytes(int n) { return stage_bytes(n); }
 
 size_t mixed_state_bytes(int algo, int n, int K, int P) {
   (void)P;
-  if (algo == MDX_ALGO_SD || algo == MIX_ALGO_SD_NATURAL) return sd_state_bytes(n);
+  if (algo == MIX_ALGO_SD_NATURAL) return sd_state_bytes(n);
   if (algo == MIX_ALGO_SD_COMPLEX) return sdc_state_bytes(n);
   return kb_state_bytes(n, K);
 }
 
+// Forms that use slice and slot by themselves: placement bits say nothing.
+static bool self_placed(int algo, int K) { return algo == MDX_ALGO_SD || (algo == MDX_ALGO_KBEST && K <= 64); }
+
 int mixed_greedy_mode(int algo, int n, int K, int P, int slice) {
+  if (self_placed(algo, K)) return 0;
   const size_t stage = stage_bytes(n), state = mixed_state_bytes(algo, n, K, P);
   if (stage + state <= (size_t)slice) return MIX_STAGE_R | MIX_STATE_SMEM;
   if (state <= (size_t)slice) return MIX_STATE_SMEM;
@@ -649,28 +879,57 @@ int mixed_greedy_mode(int algo, int n, int K, int P, int slice) {
   return 0;
 }
 
+bool mixed_mode_fits(int mode, int algo, int n, int K, int slice) {
+  if (self_placed(algo, K)) return mode == 0;
+  size_t need = 0;
+  if (mode & MIX_STAGE_R) need += mixed_stage_bytes(n);
+  if (mode & MIX_STATE_SMEM) need += mixed_state_bytes(algo, n, K, 0);
+  return need <= (size_t)slice;
+}
+
+int mixed_least_slice(int algo, int n, int K) {
+  if (algo == MDX_ALGO_SD) return (int)((walk_record_bytes(n) + 15) / 16 * 16);
+  return self_placed(algo, K) ? (int)((select_level_bytes(n, K) + 15) / 16 * 16) : 0;
+}
+
+size_t mixed_slot_bytes(int mode, int algo, int n, int K) {
+  if (algo == MDX_ALGO_SD) return walk_slot_bytes(n);
+  if (self_placed(algo, K)) return (select_path_bytes(n, K) + (size_t)kCandMax * mix_path_pad(n) + 15) / 16 * 16;
+  return (mode & MIX_STATE_SMEM) ? 16 : mixed_state_bytes(algo, n, K, 0);
+}
+
 int mixed_resident_warps(int W, int slice_bytes, int max_K, int num_sms) {
-  int grid = 0;
-  const cudaError_t e = (max_K > 64) ? prepare<8>(W, slice_bytes, num_sms, &grid)
-                                     : prepare<2>(W, slice_bytes, num_sms, &grid);
+  int walks = 0, others = 0;
+  cudaError_t e = prepare(walk_fn(), W, slice_bytes, num_sms, &walks);
+  if (e == cudaSuccess) e = prepare(mixed_fn(max_K), W, slice_bytes, num_sms, &others);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  return grid * W;
+  return std::max(walks, others) * W;
 }
 
-cudaError_t launch_mixed(const MixedArgs& a, int W, int max_K, int num_sms, cudaStream_t s) {
-  if (a.nreq <= 0) return cudaSuccess;
-  if (W < 1 || W > 32 || a.slice_bytes < 0 || (a.slice_bytes & 15)) return cudaErrorInvalidConfiguration;
-  int grid = 0;
-  cudaError_t e = (max_K > 64) ? prepare<8>(W, a.slice_bytes, num_sms, &grid)
-                               : prepare<2>(W, a.slice_bytes, num_sms, &grid);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_mixed(const MixedArgs& a, int walks, int W, int max_K, int num_sms, cudaStream_t s) {
+  if (W < 1 || W > 16 || a.slice_bytes < 0 || (a.slice_bytes & 15)) return cudaErrorInvalidConfiguration;
   const size_t smem = (size_t)W * a.slice_bytes;
-  if (max_K > 64) mixed_kernel<8><<<grid, W * 32, smem, s>>>(a);
-  else mixed_kernel<2><<<grid, W * 32, smem, s>>>(a);
-  return cudaGetLastError();
+  for (int form = 0; form < 2; ++form) {
+    MixedArgs g = a;
+    g.nreq = form == 0 ? walks : a.nreq - walks;
+    if (g.nreq <= 0) continue;
+    if (form == 1) {
+      if (a.order) g.order = a.order + walks;
+      g.counter = a.counter + 1;
+    }
+    int grid = 0;
+    cudaError_t e = prepare(form == 0 ? walk_fn() : mixed_fn(max_K), W, a.slice_bytes, num_sms, &grid);
+    if (e != cudaSuccess) return e;
+    if (form == 0) walk_kernel<<<grid, W * 32, smem, s>>>(g);
+    else if (max_K > 64) mixed_kernel<8><<<grid, W * 32, smem, s>>>(g);
+    else mixed_kernel<2><<<grid, W * 32, smem, s>>>(g);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace mdx
