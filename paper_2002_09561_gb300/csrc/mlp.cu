@@ -21,6 +21,8 @@
 // ReLU-mask for the backward pass, FP32 or BF16 output, optional transposed
 // BF16 copy).  Every mbarrier wait is bounded: on expiry the kernel records
 // an error, waits (bounded) for its copies in flight, frees TMEM and returns.
+#include <algorithm>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -136,9 +138,10 @@ enum { TC_F32 = 0, TC_BIAS_RELU = 1, TC_MASK = 2 };
 
 namespace {
 
-template <int TN>
-__global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                         const __grid_constant__ CUtensorMap tmB, int K, TcEpi epi) {
+// One 128 x TN tile at (m0, n0), the sum over nk stages, kStages of them in the ring.
+template <int TN, int kStages>
+__device__ __forceinline__ void tc_tile(const CUtensorMap* tmA, const CUtensorMap* tmB, int m0, int n0, int nk,
+                                        const TcEpi& epi) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr int A_BYTES = kTM * kTK * 2;
@@ -153,8 +156,6 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
   int* fail = reinterpret_cast<int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * kTM, n0 = blockIdx.y * TN;
-  const int nk = K / kTK;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -182,8 +183,8 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     const int pro = nk < kStages ? nk : kStages;
     for (int s = 0; s < pro; ++s) {
       mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
-      tma_load_2d(sA + s * A_BYTES, &tmA, s * kTK, m0, &full[s]);
-      tma_load_2d(sB + s * B_BYTES, &tmB, s * kTK, n0, &full[s]);
+      tma_load_2d(sA + s * A_BYTES, tmA, s * kTK, m0, &full[s]);
+      tma_load_2d(sB + s * B_BYTES, tmB, s * kTK, n0, &full[s]);
       ++issued;
     }
     bool ok = true;
@@ -208,8 +209,8 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
           break;
         }
         mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
-        tma_load_2d(sA + s * A_BYTES, &tmA, (kb + kStages) * kTK, m0, &full[s]);
-        tma_load_2d(sB + s * B_BYTES, &tmB, (kb + kStages) * kTK, n0, &full[s]);
+        tma_load_2d(sA + s * A_BYTES, tmA, (kb + kStages) * kTK, m0, &full[s]);
+        tma_load_2d(sB + s * B_BYTES, tmB, (kb + kStages) * kTK, n0, &full[s]);
         ++issued;
       }
     }
@@ -300,6 +301,38 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
   }
 }
 
+template <int TN>
+__global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
+                                                         const __grid_constant__ CUtensorMap tmB, int K, TcEpi epi) {
+  tc_tile<TN, kStages>(&tmA, &tmB, blockIdx.x * kTM, blockIdx.y * TN, K / kTK, epi);
+}
+
+// The weight gradients dW = dA^T B of the three layers in one launch: 128 x 64
+// tiles, so that all layers' are a wave together, each the whole sum over the
+// batch.  Such a tile is a chain of loads (its stages are short), so the ring has
+// eight stages.  A launch per layer with the widest tiles, 2 to 6 CTAs each, took
+// 3 x 41 us for 4,096 vectors, this 30.  (The batch in pieces to partial sums is
+// 10 us faster still, but adds up in another order, up to 1.4e-5 off; this order is
+// that of one tile per layer, to the bit.)
+constexpr int kWgradN = 64, kWgradStages = 8;
+struct WgradArgs {
+  CUtensorMap a[3], b[3];
+  int tiles_n[3], first[4];  // column tiles and first block of each layer
+  int rows;
+  float* out[3];
+  int ld[3];
+  int* err;
+};
+__global__ void __launch_bounds__(128) tc_wgrad_kernel(const __grid_constant__ WgradArgs g) {
+  const int id = blockIdx.x, l = id >= g.first[2] ? 2 : id >= g.first[1] ? 1 : 0, t = id - g.first[l];
+  TcEpi epi{};
+  epi.mode = TC_F32;
+  epi.outf = g.out[l];
+  epi.ldf = g.ld[l];
+  epi.err = g.err;
+  tc_tile<kWgradN, kWgradStages>(&g.a[l], &g.b[l], t / g.tiles_n[l] * kTM, t % g.tiles_n[l] * kWgradN, g.rows / kTK, epi);
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no -lcuda).
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -362,11 +395,40 @@ cudaError_t tc_gemm(const void* A, int lda, const void* B, int ldb, int M, int N
   if (epi.mode == TC_BIAS_RELU && (!epi.bias || misaligned(epi.bias))) return cudaErrorInvalidValue;
   if (epi.mode == TC_F32 && epi.bias && misaligned(epi.bias)) return cudaErrorInvalidValue;
   if (epi.mode == TC_MASK && (!epi.mask || misaligned(epi.mask) || epi.ldm % 8)) return cudaErrorInvalidValue;
-  if (N % 256 == 0) return launch_tc<256>(A, lda, B, ldb, M, N, K, epi, s);
-  if (N % 192 == 0) return launch_tc<192>(A, lda, B, ldb, M, N, K, epi, s);
-  if (N % 128 == 0) return launch_tc<128>(A, lda, B, ldb, M, N, K, epi, s);
+  // the widest tile that fills the SMs, else the narrowest: a training batch's
+  // GEMM is one wave of short CTAs, epilogue included (4,096 x 256 x 576 with the
+  // transposed copy: 15 / 9.8 us with 256 / 64 columns)
+  auto fills = [&](int tn) { return N % tn == 0 && (M / kTM) * (N / tn) >= 128; };
+  if (fills(256)) return launch_tc<256>(A, lda, B, ldb, M, N, K, epi, s);
+  if (fills(192)) return launch_tc<192>(A, lda, B, ldb, M, N, K, epi, s);
+  if (fills(128)) return launch_tc<128>(A, lda, B, ldb, M, N, K, epi, s);
   if (N % 64 == 0) return launch_tc<64>(A, lda, B, ldb, M, N, K, epi, s);
   return cudaErrorInvalidValue;
+}
+
+// One layer's weight gradient: out[M x N] = A[M x rows] B[N x rows]^T, all row-major.
+struct Wgrad {
+  const __nv_bfloat16 *A, *B;
+  int M, N;
+  float* out;
+};
+cudaError_t tc_wgrad(const Wgrad (&w)[3], int rows, int* err, cudaStream_t s) {
+  WgradArgs g{};
+  for (int l = 0; l < 3; ++l) {
+    if (!make_tmap(&g.a[l], w[l].A, w[l].M, rows, rows, kTM) || !make_tmap(&g.b[l], w[l].B, w[l].N, rows, rows, kWgradN))
+      return cudaErrorInvalidValue;
+    g.tiles_n[l] = w[l].N / kWgradN;
+    g.first[l + 1] = g.first[l] + w[l].M / kTM * g.tiles_n[l];
+    g.out[l] = w[l].out;
+    g.ld[l] = w[l].N;
+  }
+  g.rows = rows;
+  g.err = err;
+  const size_t smem = 1024 + (size_t)kWgradStages * (kTM + kWgradN) * kTK * 2 + 256;
+  const cudaError_t e = cudaFuncSetAttribute(tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  tc_wgrad_kernel<<<g.first[3], 128, smem, s>>>(g);
+  return cudaGetLastError();
 }
 
 }  // namespace mdx
@@ -381,7 +443,7 @@ constexpr int kH = 256;
 
 __global__ void mlp_features_kernel(int batch, int rows, int n, int D0, const float* __restrict__ R32,
                                     const float* __restrict__ yb32, const double* __restrict__ nv,
-                                    __nv_bfloat16* X, __nv_bfloat16* Xt, float* F) {
+                                    __nv_bfloat16* X, float* F) {
   // a warp per vector row, its lanes over the features (no index division)
   const int T = n * (n + 1) / 2;
   const int ts = tri_stride32(n), vs = vec_stride32(n);
@@ -398,14 +460,61 @@ __global__ void mlp_features_kernel(int batch, int rows, int n, int D0, const fl
       }
       const __nv_bfloat16 b = __float2bfloat16(x);
       X[(size_t)v * D0 + f] = b;
-      if (Xt) Xt[(size_t)f * rows + v] = b;
       if (F && v < batch) F[(size_t)v * D0 + f] = x;
     }
   }
 }
 
-// One warp per vector: pinball loss on o[0] (target log(d_ML / sigma^2)) and
-// cross-entropy of every row's ML PAM index; writes dL/do (BF16, both layouts).
+// Rows [32][cols] of a bf16 tile in shared memory (element (c, v) at
+// t[c * kTileLd + v]) to a row-major matrix and its transpose: 16-byte pieces of
+// rows would need another layout, pairs of columns and whole 64-byte row pieces
+// of the transpose do not (written element by element from a row each, as
+// before, a transpose costs a 32-byte sector per element).
+constexpr int kTileLd = 34;
+__device__ __forceinline__ void store_tile_t(const __nv_bfloat16* t, int cols, int c0, int v0, int rows,
+                                             __nv_bfloat16* Mt) {
+  for (int e = threadIdx.x; e < cols * 16; e += blockDim.x) {
+    const int c = e >> 4, v = (e & 15) * 2;
+    *reinterpret_cast<uint32_t*>(Mt + (size_t)(c0 + c) * rows + v0 + v) =
+        *reinterpret_cast<const uint32_t*>(t + c * kTileLd + v);
+  }
+}
+
+// The training batch's features and their transpose: 32 vectors per CTA, 64
+// features at a time (D0 is a multiple of 64).  4,096 vectors 16x16: 35 us with
+// the transpose written in place, 12 so.
+__global__ void __launch_bounds__(256) train_features_kernel(int batch, int rows, int n, int D0,
+                                                             const float* __restrict__ R32,
+                                                             const float* __restrict__ yb32,
+                                                             const double* __restrict__ nv, __nv_bfloat16* X,
+                                                             __nv_bfloat16* Xt, float* F) {
+  __shared__ __align__(4) __nv_bfloat16 tile[64 * kTileLd];
+  __shared__ float snr[32];
+  const int T = n * (n + 1) / 2, ts = tri_stride32(n), vs = vec_stride32(n);
+  const int v0 = blockIdx.x * 32, f0 = blockIdx.y * 64;
+  if (f0 <= T + n && T + n < f0 + 64) {
+    // FP64 logarithms take microseconds: the 32 of them side by side
+    if (threadIdx.x < 32 && v0 + (int)threadIdx.x < batch)
+      snr[threadIdx.x] = (float)(-10.0 * log10(nv[v0 + threadIdx.x]) / 30.0);
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < 32 * 64; e += blockDim.x) {
+    const int v = v0 + (e >> 6), f = f0 + (e & 63);
+    float x = 0.0f;
+    if (v < batch) {
+      if (f < T) x = R32[(size_t)v * ts + f];
+      else if (f < T + n) x = yb32[(size_t)v * vs + (f - T)];
+      else if (f == T + n) x = snr[e >> 6];
+    }
+    const __nv_bfloat16 b = __float2bfloat16(x);
+    X[(size_t)v * D0 + f] = b;
+    if (F && v < batch) F[(size_t)v * D0 + f] = x;
+    tile[(e & 63) * kTileLd + (e >> 6)] = b;
+  }
+  __syncthreads();
+  store_tile_t(tile, 64, f0, v0, rows, Xt);
+}
+
 // Summary features of a large system (n_tx > 32), one warp per vector: log R_ii
 // (n values), log(d_B / sigma^2) / 10 with d_B the FP32 distance of the Babai
 // point (successive rounding, top row first, clipped to the PAM grid),
@@ -466,55 +575,99 @@ __global__ void reduced_features_kernel(int batch, int rows, int n, int P, float
   }
 }
 
-__global__ void mlp_loss_kernel(int batch, int rows, int n, int P, int n_tx, int DO, const float* __restrict__ O,
-                                const double* __restrict__ ml_metric, const double* __restrict__ nv,
-                                const uint8_t* __restrict__ ml_sym, float tau, float lambda, int ce_rows,
-                                __nv_bfloat16* dO, __nv_bfloat16* dOt, float* loss) {
-  const int warps = blockDim.x / 32;
-  const int v = blockIdx.x * warps + threadIdx.x / 32, lane = threadIdx.x & 31;
-  if (v >= rows) return;
+// Pinball loss on o[0] (target log(d_ML / sigma^2)) and cross-entropy of every
+// row's ML PAM index; writes dL/do (BF16, both layouts).
+// 32 vectors per CTA, a warp per vector and a lane per row, through a shared
+// tile (see store_tile_t; 4,096 vectors of 16x16 16-QAM: 30 us with a lane per
+// output and the transpose written in place, 16 so).
+__global__ void __launch_bounds__(256) mlp_loss_kernel(int batch, int rows, int n, int P, int n_tx, int DO,
+                                                       const float* __restrict__ O,
+                                                       const double* __restrict__ ml_metric,
+                                                       const double* __restrict__ nv,
+                                                       const uint8_t* __restrict__ ml_sym, float tau, float lambda,
+                                                       int ce_rows, __nv_bfloat16* dO, __nv_bfloat16* dOt, float* loss) {
+  extern __shared__ __align__(16) unsigned char loss_smem[];
+  __nv_bfloat16* tile = reinterpret_cast<__nv_bfloat16*>(loss_smem);
+  const int lane = threadIdx.x & 31, v0 = blockIdx.x * 32;
   const float inv_b = 1.0f / (float)batch;
+  const __nv_bfloat16 zero = __float2bfloat16(0.0f);
   float lr = 0.0f, lc = 0.0f;
-  for (int j = lane; j < DO; j += 32) {
+  if (threadIdx.x >= 224) {  // the radius head, a lane per vector (FP64 logarithms side by side)
+    const int v = v0 + lane;
     float g = 0.0f;
     if (v < batch) {
-      if (j == 0) {
-        const float t = (float)log(ml_metric[v] / nv[v]);
-        const float e = t - O[(size_t)v * DO];
-        lr = (e >= 0.0f ? tau * e : (tau - 1.0f) * e);
-        g = (e > 0.0f ? -tau : (1.0f - tau)) * inv_b;
-      } else if (j < 1 + ce_rows * P) {
-        const int r = (j - 1) / P, k = (j - 1) % P;
-        const float* lg = O + (size_t)v * DO + 1 + r * P;
-        float mx = lg[0];
-        for (int q = 1; q < P; ++q) mx = fmaxf(mx, lg[q]);
-        float s = 0.0f;
-        for (int q = 0; q < P; ++q) s += __expf(lg[q] - mx);
-        const int qs = ml_sym[(size_t)v * n_tx + r / 2];
-        const int kt = (r & 1) ? (qs % P) : (qs / P);
-        const float pk = __expf(lg[k] - mx) / s;
-        g = lambda * (pk - (k == kt ? 1.0f : 0.0f)) * inv_b / (float)n;
-        if (k == kt) lc += -logf(fmaxf(pk, 1e-30f)) / (float)n;
-      }
+      const float t = (float)log(ml_metric[v] / nv[v]);
+      const float e = t - O[(size_t)v * DO];
+      lr = (e >= 0.0f ? tau * e : (tau - 1.0f) * e);
+      g = (e > 0.0f ? -tau : (1.0f - tau)) * inv_b;
     }
-    const __nv_bfloat16 b = __float2bfloat16(g);
-    dO[(size_t)v * DO + j] = b;
-    dOt[(size_t)j * rows + v] = b;
+    tile[lane] = __float2bfloat16(g);
   }
+  for (int i = threadIdx.x >> 5; i < 32; i += 8) {
+    const int v = v0 + i;
+    const bool act = v < batch;
+    for (int r = lane; r < ce_rows; r += 32) {
+      float lg[8], mx = -INFINITY, s = 0.0f;  // (P <= 8)
+      int kt = 0;
+      if (act) {
+        const float* l = O + (size_t)v * DO + 1 + r * P;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (q < P) {
+            lg[q] = l[q];
+            mx = fmaxf(mx, lg[q]);
+          }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (q < P) s += __expf(lg[q] - mx);
+        const int qs = ml_sym[(size_t)v * n_tx + r / 2];
+        kt = (r & 1) ? (qs % P) : (qs / P);
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < P) {
+          float g = 0.0f;
+          if (act) {
+            const float pk = __expf(lg[k] - mx) / s;
+            g = lambda * (pk - (k == kt ? 1.0f : 0.0f)) * inv_b / (float)n;
+            if (k == kt) lc += -logf(fmaxf(pk, 1e-30f)) / (float)n;
+          }
+          tile[(1 + r * P + k) * kTileLd + i] = __float2bfloat16(g);
+        }
+    }
+    for (int j = 1 + ce_rows * P + lane; j < DO; j += 32) tile[j * kTileLd + i] = zero;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 32 * (DO / 2); e += blockDim.x) {
+    const int v = e / (DO / 2), j = e % (DO / 2) * 2;
+    __nv_bfloat162 b;
+    b.x = tile[j * kTileLd + v];
+    b.y = tile[(j + 1) * kTileLd + v];
+    *reinterpret_cast<__nv_bfloat162*>(dO + (size_t)(v0 + v) * DO + j) = b;
+  }
+  store_tile_t(tile, DO, 0, v0, rows, dOt);
   lr = warp_sum(lr);
   lc = warp_sum(lc);
-  if (lane == 0 && v < batch) {
+  if (lane == 0) {
     atomicAdd(&loss[0], lr * inv_b);
     atomicAdd(&loss[1], lc * inv_b);
   }
 }
 
-// grad[j] = sum over the batch of Mt[j][:] (rows of a transposed BF16 matrix).
-__global__ void row_sum_kernel(int N, int cols, const __nv_bfloat16* __restrict__ Mt, float* __restrict__ out) {
-  const int j = blockIdx.x;
-  if (j >= N) return;
+// Bias gradients of the three layers: the sum over the batch of each row of a
+// transposed BF16 matrix.
+struct BiasArgs {
+  const __nv_bfloat16* mt[3];  // [N][rows]
+  int N[3];
+  float* out[3];
+  int rows;
+};
+__global__ void __launch_bounds__(256) bias_grads_kernel(const __grid_constant__ BiasArgs a) {
+  const int l = blockIdx.y, j = blockIdx.x;
+  if (j >= a.N[l]) return;
   float s = 0.0f;
-  for (int c = threadIdx.x; c < cols; c += blockDim.x) s += __bfloat162float(Mt[(size_t)j * cols + c]);
+#pragma unroll 8
+  for (int c = threadIdx.x; c < a.rows; c += blockDim.x) s += __bfloat162float(a.mt[l][(size_t)j * a.rows + c]);
   __shared__ float red[32];
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = s;
@@ -522,12 +675,39 @@ __global__ void row_sum_kernel(int N, int cols, const __nv_bfloat16* __restrict_
   if (threadIdx.x < 32) {
     float t = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0f;
     t = warp_sum(t);
-    if (threadIdx.x == 0) out[j] = t;
+    if (threadIdx.x == 0) a.out[l][j] = t;
   }
 }
 
+// The BF16 copies of a weight vector: row-major and, for the backward pass,
+// transposed.
+struct PackArgs {
+  __nv_bfloat16 *W1, *W2, *W2t, *W3, *W3t;
+  size_t b1, W2o, b2, W3o, b3;  // offsets of b1, W2, b2, W3, b3
+  int DO;
+};
+__device__ __forceinline__ void pack_weight(const PackArgs& a, size_t i, float w) {
+  const __nv_bfloat16 b = __float2bfloat16(w);
+  if (i < a.b1) {
+    a.W1[i] = b;
+  } else if (i >= a.W2o && i < a.b2) {
+    const unsigned e = (unsigned)(i - a.W2o);
+    a.W2[e] = b;
+    a.W2t[(e % kH) * kH + e / kH] = b;
+  } else if (i >= a.W3o && i < a.b3) {
+    const unsigned e = (unsigned)(i - a.W3o);
+    a.W3[e] = b;
+    a.W3t[(e % kH) * a.DO + e / kH] = b;
+  }
+}
+__global__ void pack_kernel(long long count, const float* __restrict__ w, PackArgs a) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
+    pack_weight(a, (size_t)i, w[i]);
+}
+// Adam's step and the copies of the new weights (a launch for the four).
 __global__ void adam_kernel(long long count, float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
+                            float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2,
+                            PackArgs a) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
        i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -535,20 +715,9 @@ __global__ void adam_kernel(long long count, float* __restrict__ w, const float*
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  }
-}
-
-// BF16 copies of a [rows][cols] FP32 weight: W (row-major) and optionally W^T.
-__global__ void pack_kernel(int rows, int cols, const float* __restrict__ w, __nv_bfloat16* wb,
-                            __nv_bfloat16* wt) {
-  const long long total = (long long)rows * cols;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(e / cols), c = (int)(e % cols);
-    const __nv_bfloat16 b = __float2bfloat16(w[e]);
-    wb[e] = b;
-    if (wt) wt[(size_t)c * rows + r] = b;
+    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[i] = wi;
+    pack_weight(a, (size_t)i, wi);
   }
 }
 
@@ -747,11 +916,12 @@ cudaError_t mlp_alloc(MlpState** out, int n_tx, int qam, int cap) {
   return cudaSuccess;
 }
 
+PackArgs pack_args(MlpState* s) {
+  return PackArgs{s->W1, s->W2, s->W2t, s->W3, s->W3t, s->ob1(), s->oW2(), s->ob2(), s->oW3(), s->ob3(), s->DO};
+}
+
 cudaError_t mlp_pack(MlpState* s, cudaStream_t st) {
-  const int D0 = s->D0, DO = s->DO;
-  pack_kernel<<<grid_for((long long)kH * D0, 256), 256, 0, st>>>(kH, D0, s->w + s->oW1(), s->W1, nullptr);
-  pack_kernel<<<grid_for((long long)kH * kH, 256), 256, 0, st>>>(kH, kH, s->w + s->oW2(), s->W2, s->W2t);
-  pack_kernel<<<grid_for((long long)DO * kH, 256), 256, 0, st>>>(DO, kH, s->w + s->oW3(), s->W3, s->W3t);
+  pack_kernel<<<grid_for(s->count, 256), 256, 0, st>>>(s->count, s->w, pack_args(s));
   return cudaGetLastError();
 }
 
@@ -765,8 +935,12 @@ cudaError_t mlp_features(MlpState* s, int batch, int rows, const float* R32, con
         batch, rows, s->n, s->P, alpha, s->D0, R32, yb32, nv, s->X, train ? s->Xt : nullptr, F);
     return cudaGetLastError();
   }
-  mlp_features_kernel<<<grid_for((long long)rows * 32, 256), 256, 0, st>>>(
-      batch, rows, s->n, s->D0, R32, yb32, nv, s->X, train ? s->Xt : nullptr, F);
+  if (train)
+    train_features_kernel<<<dim3(rows / 32, s->D0 / 64), 256, 0, st>>>(batch, rows, s->n, s->D0, R32, yb32, nv, s->X,
+                                                                       s->Xt, F);
+  else
+    mlp_features_kernel<<<grid_for((long long)rows * 32, 256), 256, 0, st>>>(batch, rows, s->n, s->D0, R32, yb32, nv,
+                                                                             s->X, F);
   return cudaGetLastError();
 }
 
@@ -803,9 +977,11 @@ cudaError_t mlp_backward(MlpState* s, int batch, int rows, const double* ml_metr
                          const uint8_t* ml_sym, cudaStream_t st) {
   cudaError_t r = cudaMemsetAsync(s->loss, 0, 2 * sizeof(float), st);
   if (r != cudaSuccess) return r;
-  mlp_loss_kernel<<<(rows + 7) / 8, 256, 0, st>>>(batch, rows, s->n, s->P, s->n_tx, s->DO, s->O, ml_metric, nv,
-                                                  ml_sym, 0.9f, 0.2f, s->reduced ? 0 : s->n, s->dO, s->dOt,
-                                                  s->loss);
+  const int loss_smem = (int)sizeof(__nv_bfloat16) * s->DO * kTileLd;
+  r = cudaFuncSetAttribute(mlp_loss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, loss_smem);
+  if (r != cudaSuccess) return r;
+  mlp_loss_kernel<<<rows / 32, 256, loss_smem, st>>>(batch, rows, s->n, s->P, s->n_tx, s->DO, s->O, ml_metric, nv,
+                                                     ml_sym, 0.9f, 0.2f, s->reduced ? 0 : s->n, s->dO, s->dOt, s->loss);
   if ((r = cudaGetLastError()) != cudaSuccess) return r;
   TcEpi e{};
   e.err = s->err;
@@ -823,21 +999,16 @@ cudaError_t mlp_backward(MlpState* s, int batch, int rows, const double* ml_metr
   e.outb = s->dH1;
   e.outt = s->dH1t;
   if ((r = tc_gemm(s->dH2, kH, s->W2t, kH, rows, kH, kH, e, st)) != cudaSuccess) return r;
-  // weight gradients: dW3 = dO^T H2, dW2 = dH2^T H1, dW1 = dH1^T X (reductions over the batch)
-  TcEpi f{};
-  f.err = s->err;
-  f.mode = TC_F32;
-  f.outf = s->g + s->oW3();
-  f.ldf = kH;
-  if ((r = tc_gemm(s->dOt, rows, s->H2t, rows, s->DO, kH, rows, f, st)) != cudaSuccess) return r;
-  f.outf = s->g + s->oW2();
-  if ((r = tc_gemm(s->dH2t, rows, s->H1t, rows, kH, kH, rows, f, st)) != cudaSuccess) return r;
-  f.outf = s->g + s->oW1();
-  f.ldf = s->D0;
-  if ((r = tc_gemm(s->dH1t, rows, s->Xt, rows, kH, s->D0, rows, f, st)) != cudaSuccess) return r;
-  row_sum_kernel<<<s->DO, 256, 0, st>>>(s->DO, rows, s->dOt, s->g + s->ob3());
-  row_sum_kernel<<<kH, 256, 0, st>>>(kH, rows, s->dH2t, s->g + s->ob2());
-  row_sum_kernel<<<kH, 256, 0, st>>>(kH, rows, s->dH1t, s->g + s->ob1());
+  // weight gradients: dW3 = dO^T H2, dW2 = dH2^T H1, dW1 = dH1^T X (sums over the batch)
+  const Wgrad w[3] = {{s->dOt, s->H2t, s->DO, kH, s->g + s->oW3()},
+                      {s->dH2t, s->H1t, kH, kH, s->g + s->oW2()},
+                      {s->dH1t, s->Xt, kH, s->D0, s->g + s->oW1()}};
+  if ((r = tc_wgrad(w, rows, s->err, st)) != cudaSuccess) return r;
+  const BiasArgs a{{s->dOt, s->dH2t, s->dH1t},
+                   {s->DO, kH, kH},
+                   {s->g + s->ob3(), s->g + s->ob2(), s->g + s->ob1()},
+                   rows};
+  bias_grads_kernel<<<dim3(std::max(s->DO, kH), 3), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -845,10 +1016,9 @@ cudaError_t mlp_adam(MlpState* s, float lr, cudaStream_t st) {
   s->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.0f - powf(b1, (float)s->step), c2 = 1.0f - powf(b2, (float)s->step);
-  adam_kernel<<<grid_for(s->count, 256), 256, 0, st>>>(s->count, s->w, s->g, s->m, s->v, lr, b1, b2, 1e-8f, c1, c2);
-  cudaError_t r = cudaGetLastError();
-  if (r != cudaSuccess) return r;
-  return mlp_pack(s, st);
+  adam_kernel<<<grid_for(s->count, 256), 256, 0, st>>>(s->count, s->w, s->g, s->m, s->v, lr, b1, b2, 1e-8f, c1, c2,
+                                                       pack_args(s));
+  return cudaGetLastError();
 }
 
 cudaError_t mlp_radius(MlpState* s, int batch, const double* nv, bool learned, bool order, int base_mode,
