@@ -48,6 +48,8 @@ struct mdx_ctx {
   // followed by an event the QR of that chunk waits for (see run_detect)
   static constexpr int kHostChunks = 8;
   cudaStream_t copy_stream = nullptr;
+  cudaStream_t side_stream = nullptr;  // an uneven batch's second kernel
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_free = nullptr;
   cudaEvent_t ev_chunk[kHostChunks] = {};
   // uneven batches (detect_mixed): the uploaded request table and its device
@@ -161,6 +163,9 @@ void free_all(mdx_ctx* c) {
     if (ev) cudaEventDestroy(ev);
   if (c->ev_free) cudaEventDestroy(c->ev_free);
   if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
+  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->side_stream) cudaStreamDestroy(c->side_stream);
 }
 
 enum Algo { ALGO_SD = 0, ALGO_KBEST = 1, ALGO_HYBRID = 2, ALGO_LINEAR = 3 };
@@ -401,7 +406,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
     }
     m.gscratch = c->mx_scratch;
     if (ev) cudaEventRecord(ev[1], s);
-    e = launch_mixed(m, 0, c->mx_W, 0, c->num_sms, s);
+    e = launch_mixed(m, 0, c->mx_W, 0, c->num_sms, MixedFork{}, s);
   } else if (algo == ALGO_SD) {
     if (ev) cudaEventRecord(ev[1], s);
     // The antenna order is the search's own business where nothing that the
@@ -649,7 +654,8 @@ cudaError_t mixed_launches(mdx_ctx* c, int nreq, const double* dH, const double*
   a.metric_out = dmet;
   a.vstatus = dvst;
   a.stats = dstats;
-  e = launch_mixed(a, c->mx_walks, c->mx_W, c->mx_maxK, c->num_sms, s);
+  e = launch_mixed(a, c->mx_walks, c->mx_W, c->mx_maxK, c->num_sms,
+                   MixedFork{c->side_stream, c->ev_fork, c->ev_join}, s);
   if (ev && e == cudaSuccess) cudaEventRecord(ev[2], s);
   return e;
 }
@@ -976,6 +982,9 @@ mdx_status mdx_create(mdx_ctx** out, int device, int max_batch, int max_n_rx, in
   chk(alloc(c, &c->sd_order, sd_order_ints(max_batch)));
   chk(alloc(c, &c->sd_sorted, B * (1 + 2 * (size_t)std::min(max_n_tx, kReorderMaxTx))));
   chk(cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+  chk(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
+  chk(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+  chk(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
   chk(cudaEventCreateWithFlags(&c->ev_free, cudaEventDisableTiming));
   for (cudaEvent_t& ev : c->ev_chunk) chk(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
   if (e != cudaSuccess) {

@@ -906,30 +906,39 @@ int mixed_resident_warps(int W, int slice_bytes, int max_K, int num_sms) {
     cudaGetLastError();
     return 0;
   }
-  return std::max(walks, others) * W;
+  return (walks + others) * W;
 }
 
-cudaError_t launch_mixed(const MixedArgs& a, int walks, int W, int max_K, int num_sms, cudaStream_t s) {
+cudaError_t launch_mixed(const MixedArgs& a, int walks, int W, int max_K, int num_sms, const MixedFork& fork,
+                         cudaStream_t s) {
   if (W < 1 || W > 16 || a.slice_bytes < 0 || (a.slice_bytes & 15)) return cudaErrorInvalidConfiguration;
   const size_t smem = (size_t)W * a.slice_bytes;
-  for (int form = 0; form < 2; ++form) {
+  const bool both = walks > 0 && a.nreq > walks;
+  cudaError_t e = both ? cudaEventRecord(fork.begin, s) : cudaSuccess;
+  int slots = 0;
+  for (int form = 0; form < 2 && e == cudaSuccess; ++form) {
     MixedArgs g = a;
     g.nreq = form == 0 ? walks : a.nreq - walks;
     if (g.nreq <= 0) continue;
     if (form == 1) {
       if (a.order) g.order = a.order + walks;
       g.counter = a.counter + 1;
+      g.gscratch = a.gscratch + (size_t)slots * a.gslot_bytes;
     }
     int grid = 0;
-    cudaError_t e = prepare(form == 0 ? walk_fn() : mixed_fn(max_K), W, a.slice_bytes, num_sms, &grid);
+    e = prepare(form == 0 ? walk_fn() : mixed_fn(max_K), W, a.slice_bytes, num_sms, &grid);
     if (e != cudaSuccess) return e;
-    if (form == 0) walk_kernel<<<grid, W * 32, smem, s>>>(g);
-    else if (max_K > 64) mixed_kernel<8><<<grid, W * 32, smem, s>>>(g);
-    else mixed_kernel<2><<<grid, W * 32, smem, s>>>(g);
+    slots += grid * W;
+    const cudaStream_t on = form == 1 && both ? fork.side : s;
+    if (on != s && (e = cudaStreamWaitEvent(on, fork.begin, 0)) != cudaSuccess) return e;
+    if (form == 0) walk_kernel<<<grid, W * 32, smem, on>>>(g);
+    else if (max_K > 64) mixed_kernel<8><<<grid, W * 32, smem, on>>>(g);
+    else mixed_kernel<2><<<grid, W * 32, smem, on>>>(g);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess && on != s) e = cudaEventRecord(fork.end, on);
+    if (e == cudaSuccess && on != s) e = cudaStreamWaitEvent(s, fork.end, 0);
   }
-  return cudaSuccess;
+  return e;
 }
 
 }  // namespace mdx
