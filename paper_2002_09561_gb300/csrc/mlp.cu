@@ -441,30 +441,6 @@ namespace {
 
 constexpr int kH = 256;
 
-__global__ void mlp_features_kernel(int batch, int rows, int n, int D0, const float* __restrict__ R32,
-                                    const float* __restrict__ yb32, const double* __restrict__ nv,
-                                    __nv_bfloat16* X, float* F) {
-  // a warp per vector row, its lanes over the features (no index division)
-  const int T = n * (n + 1) / 2;
-  const int ts = tri_stride32(n), vs = vec_stride32(n);
-  const int lane = threadIdx.x & 31;
-  const int w0 = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)(((long long)gridDim.x * blockDim.x) >> 5);
-  for (int v = w0; v < rows; v += nw) {
-    for (int f = lane; f < D0; f += 32) {
-      float x = 0.0f;
-      if (v < batch) {
-        if (f < T) x = R32[(size_t)v * ts + f];
-        else if (f < T + n) x = yb32[(size_t)v * vs + (f - T)];
-        else if (f == T + n) x = (float)(-10.0 * log10(nv[v]) / 30.0);
-      }
-      const __nv_bfloat16 b = __float2bfloat16(x);
-      X[(size_t)v * D0 + f] = b;
-      if (F && v < batch) F[(size_t)v * D0 + f] = x;
-    }
-  }
-}
-
 // Rows [32][cols] of a bf16 tile in shared memory (element (c, v) at
 // t[c * kTileLd + v]) to a row-major matrix and its transpose: 16-byte pieces of
 // rows would need another layout, pairs of columns and whole 64-byte row pieces
@@ -480,14 +456,15 @@ __device__ __forceinline__ void store_tile_t(const __nv_bfloat16* t, int cols, i
   }
 }
 
-// The training batch's features and their transpose: 32 vectors per CTA, 64
-// features at a time (D0 is a multiple of 64).  4,096 vectors 16x16: 35 us with
-// the transpose written in place, 12 so.
-__global__ void __launch_bounds__(256) train_features_kernel(int batch, int rows, int n, int D0,
-                                                             const float* __restrict__ R32,
-                                                             const float* __restrict__ yb32,
-                                                             const double* __restrict__ nv, __nv_bfloat16* X,
-                                                             __nv_bfloat16* Xt, float* F) {
+// Features and, for training, their transpose: 32 vectors x 64 features per CTA
+// (D0 is a multiple of 64).  4,096 vectors 16x16 with the transpose 35 us written
+// in place a warp per vector, 12 so; 100,000 without it 255 us, 129 so (the FP64
+// logarithm of the SNR was a lane at a time).
+__global__ void __launch_bounds__(256) mlp_features_kernel(int batch, int rows, int n, int D0,
+                                                           const float* __restrict__ R32,
+                                                           const float* __restrict__ yb32,
+                                                           const double* __restrict__ nv, __nv_bfloat16* X,
+                                                           __nv_bfloat16* Xt, float* F) {
   __shared__ __align__(4) __nv_bfloat16 tile[64 * kTileLd];
   __shared__ float snr[32];
   const int T = n * (n + 1) / 2, ts = tri_stride32(n), vs = vec_stride32(n);
@@ -509,8 +486,9 @@ __global__ void __launch_bounds__(256) train_features_kernel(int batch, int rows
     const __nv_bfloat16 b = __float2bfloat16(x);
     X[(size_t)v * D0 + f] = b;
     if (F && v < batch) F[(size_t)v * D0 + f] = x;
-    tile[(e & 63) * kTileLd + (e >> 6)] = b;
+    if (Xt) tile[(e & 63) * kTileLd + (e >> 6)] = b;
   }
+  if (!Xt) return;
   __syncthreads();
   store_tile_t(tile, 64, f0, v0, rows, Xt);
 }
@@ -935,12 +913,8 @@ cudaError_t mlp_features(MlpState* s, int batch, int rows, const float* R32, con
         batch, rows, s->n, s->P, alpha, s->D0, R32, yb32, nv, s->X, train ? s->Xt : nullptr, F);
     return cudaGetLastError();
   }
-  if (train)
-    train_features_kernel<<<dim3(rows / 32, s->D0 / 64), 256, 0, st>>>(batch, rows, s->n, s->D0, R32, yb32, nv, s->X,
-                                                                       s->Xt, F);
-  else
-    mlp_features_kernel<<<grid_for((long long)rows * 32, 256), 256, 0, st>>>(batch, rows, s->n, s->D0, R32, yb32, nv,
-                                                                             s->X, F);
+  mlp_features_kernel<<<dim3(rows / 32, s->D0 / 64), 256, 0, st>>>(batch, rows, s->n, s->D0, R32, yb32, nv, s->X,
+                                                                   train ? s->Xt : nullptr, F);
   return cudaGetLastError();
 }
 
