@@ -87,17 +87,18 @@ METRIC = "decoded vectors/s at matched BER (16x16 16QAM, 100x100 64QAM), learned
 # reports no traffic until the kernel is captured again.
 KERNEL_SOURCES = {
     "16x16-16qam-sd-learned": ("sd_group.cu", "sd_common.cuh", "mdx_internal.cuh"),
-    "100x100-64qam-hybrid32-learned": ("kbest.cu", "warp_kbest.cuh", "mdx_internal.cuh"),
+    "100x100-64qam-hybrid32-learned": ("hybrid_warp.cu", "select_run.cuh", "warp_kbest.cuh", "mdx_internal.cuh"),
 }
 TRAFFIC_PER_VECTOR = {
-    "16x16-16qam-sd-learned": ((225.208576e6 + 6.209024e6) / 30000,
+    "16x16-16qam-sd-learned": ((225.353472e6 + 5.748992e6) / 30000,
                                "ncu capture of sd_group_kernel, 30,000 vectors of the learned 16x16 sweep "
-                               "(profiles/sd_group_kernel_16x16_16qam_sweep_30k.md), scaled by vectors",
-                               "41cf9bf6e4c91aa7"),
-    "100x100-64qam-hybrid32-learned": ((516.954880e6 + 4.081664e6) / 2000,
-                                       "ncu capture of hybrid_kernel, 2,000 vectors of the learned 100x100 "
-                                       "workload (profiles/hybrid_kernel_100x100_64qam_2k.md), scaled by vectors",
-                                       "e4500e2afb5bc28e"),
+                               "(profiles/search_and_qr_kernels.md), scaled by vectors",
+                               "7e12b2722ccb6bd4"),
+    "100x100-64qam-hybrid32-learned": ((369.485824e6 + 8.572928e6 + 30.755840e6 + 0.067840e6 + 216.549120e6
+                                        + 6.335232e6) / 2000,
+                                       "ncu capture of the hybrid's three search kernels, 2,000 vectors of the learned "
+                                       "100x100 workload (profiles/search_and_qr_kernels.md), scaled by vectors",
+                                       "c063e981d9e0b5ff"),
 }
 
 
@@ -121,11 +122,11 @@ def code_hash(files, csrc=None):
 # tied to the sources in the same way: with the live node rate this gives the
 # kernel's instruction-issue rate, the resource that bounds it.
 INSTRUCTIONS_PER_NODE = {
-    "16x16-16qam-sd-learned": (1.2128964723e10 / 297008606,
+    "16x16-16qam-sd-learned": (1.2249798059e10 / 296364808,
                                "ncu capture of sd_group_kernel, 30,000 vectors of the learned 16x16 sweep: "
                                "smsp__inst_executed.sum over the launch's branched nodes "
-                               "(profiles/sd_group_kernel_16x16_16qam_sweep_30k.md)",
-                               "41cf9bf6e4c91aa7"),
+                               "(profiles/search_and_qr_kernels.md)",
+                               "7e12b2722ccb6bd4"),
 }
 
 
@@ -573,8 +574,16 @@ def main():
     stream = torch.cuda.current_stream(dev)
     arm = Arm(torch, mdx, replicas, ctx, algo, H, y, nv, truth, qam, stream, dist, dev, local)
 
-    ms, (qr_ms, search_ms, calls), errs, sampler = arm.time(params, out, args.steps, args.warmup)
+    # the timed calls ask for the points, metrics and status; the visited-node
+    # statistics, which fix the search to the natural antenna order, come from an
+    # arm of their own, with the search's time for them (roofline)
+    ms, _, errs, sampler = arm.time(params, out[:3] + (None,), args.steps, args.warmup)
     value = B * world * args.steps / (ms / 1e3)
+    timed = [o.clone() for o in out[:3]]
+    ssteps = max(1, min(args.steps, 5))
+    sms_, (qr_ms, search_ms, calls), _, _ = arm.time(params, out, ssteps, 1)
+    with_stats = {"value": B * world * ssteps / (sms_ / 1e3), "unit": "vectors/s", "ms_per_step": sms_ / ssteps,
+                  "steps": ssteps, "identical_decisions": bool(torch.equal(timed[0], out[0]))}
     host = lambda o: (o[0].cpu().numpy(), o[2].cpu().numpy(), o[3].cpu().numpy())  # noqa: E731
     main_host = host(out)
     bits_vec = 2 * n * int(round(math.log2(int(round(qam ** 0.5)))))
@@ -584,8 +593,8 @@ def main():
         pparams = mdx.make_params(n, n, qam, radius=w["radius"], K=max(w["K"], 1), depth=w["depth"],
                                   flags=base_flags)
         pout = mdx._outputs(B, n, dev, True)
-        pms, pprof, perrs, _ = arm.time(pparams, pout, args.steps, 1)
-        plain_qr = pprof
+        pms, plain_qr, perrs, _ = arm.time(pparams, pout[:3] + (None,), args.steps, 1)
+        _, pprof, _, _ = arm.time(pparams, pout, 1, 0)  # statistics
         ph = host(pout)
         plain = {"value": B * world * args.steps / (pms / 1e3), "unit": "vectors/s", "ms_per_step": pms / args.steps,
                  "initial_radius": "r^2 = N M sigma^2", "mean_nodes": float(ph[2][:, 0].mean()),
@@ -598,7 +607,8 @@ def main():
             bsteps = max(1, min(args.steps, 5))
             bparams = mdx.make_params(n, n, qam, radius=math.inf, flags=base_flags)
             bout = mdx._outputs(B, n, dev, True)
-            bms, bprof, berrs, _ = arm.time(bparams, bout, bsteps, 1)
+            bms, _, berrs, _ = arm.time(bparams, bout[:3] + (None,), bsteps, 1)
+            _, bprof, _, _ = arm.time(bparams, bout, 1, 0)  # statistics
             bh = host(bout)
             babai = {"value": B * world * bsteps / (bms / 1e3), "unit": "vectors/s", "ms_per_step": bms / bsteps,
                      "steps": bsteps, "initial_radius": "none (the Babai point reached by the first descent sets it)",
@@ -669,7 +679,7 @@ def main():
                 "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32 search, f64 QR and re-scoring",
                 "data": "synthetic (seeded Rayleigh channels, uniform QAM symbols, AWGN)",
-                "config": cfg, "roofline": roof, "qr_roofline": qr_roof, "cpu_baseline": cpu, "e2e": e2e,
+                "config": cfg, "with_statistics": with_stats, "roofline": roof, "qr_roofline": qr_roof, "cpu_baseline": cpu, "e2e": e2e,
                 "gpu_launches": launches_per_call(algo, learned, n) * args.steps, "clocks": sampler.summary(),
                 "measured_peaks": probe, "oracle_check": check, "plain": plain, "babai": babai,
                 "quality": {"ber": bit_err / bits, "ser": sym_err / (B * world * n),
@@ -685,9 +695,10 @@ def main():
 
 
 def launches_per_call(algo, learned, n):
-    """Kernels of one timed step: the QR, the network (features, three GEMMs,
-    radius) when learned, the sphere decoder's heaviest-first ordering (three
-    kernels) for detect_sd, the search, and the error count."""
+    """Kernels of one timed step, at least: the QR, the network (features, three
+    GEMMs, radius) when learned, three kernels that order the sphere decoder's
+    work for detect_sd, the search, and the error count.  (The QR's second form
+    and the searches' follow-up kernels are not counted.)"""
     k = 3 + (5 if learned else 0)
     if algo == "sd":
         k += 3
@@ -779,10 +790,12 @@ def search_roofline(workload, algo, stats, search_ms, calls, qr_ms, sms, probe, 
 
 
 def qr_roofline(n_rx, n_tx, B, prof, sms, probe):
-    """FP64 roofline of the QR: 8 (N M^2 - M^3 / 3) real flops per complex
+    """The QR against the FP64 unit: 8 (N M^2 - M^3 / 3) real flops per complex
     Householder QR of an N x M matrix, over the QR interval's CUDA-event
-    duration, against the derived FP64 peak (SMs x 2 FP64 FMA lanes x 2 x the
-    maximum SM clock) and the probe's measured FP64 FMA and MMA rates."""
+    duration, beside the derived FP64 peak (SMs x 2 FP64 FMA lanes x 2 x the
+    maximum SM clock) and the probe's measured FP64 FMA and MMA rates.  The QR
+    itself works in 64-bit fixed point on the integer multiply-add pipe, so it
+    can pass the FP64 unit's rate: a figure above 1 says by how much."""
     qr_ms, _, calls = prof
     peaks = load_peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
@@ -792,7 +805,7 @@ def qr_roofline(n_rx, n_tx, B, prof, sms, probe):
     s = (qr_ms / max(calls, 1)) / 1e3
     achieved = flops / s / 1e12 if s > 0 else 0.0
     meas = max(probe["fp64_fma_tflops"], probe["fp64_mma_tflops"])
-    return {"bound": "fp64", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+    return {"bound": "integer multiply-add (fixed point; against the FP64 unit)", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "measured_fp64_peak": meas, "frac_of_measured": achieved / meas, "ms_per_launch": 1e3 * s,
             "flops_per_matrix": flops / B, "matrices": B,
             "peak_source": f"derived: {sms} SMs x 2 FP64 FMA lanes x 2 x {sm_max:.0f} MHz; measured = the larger "
@@ -828,7 +841,8 @@ def hybrid_record(args, rank, world, local, dev, dist, torch, mdx, replicas, pro
     for name, fl, warm in (("learned", mdx.MDX_LEARNED_RADIUS, args.warmup), ("plain", 0, 1)):
         prm = mdx.make_params(n, n, qam, radius="paper", K=w["K"], depth=w["depth"], flags=fl)
         o = mdx._outputs(B, n, dev, True)
-        ms, prof, errs, sampler = arm.time(prm, o, args.steps, warm)
+        ms, qprof, errs, sampler = arm.time(prm, o[:3] + (None,), args.steps, warm)
+        _, prof, _, _ = arm.time(prm, o, max(1, min(args.steps, 5)), 1)  # statistics, and the search's time with them
         hh = (o[0].cpu().numpy(), o[2].cpu().numpy(), o[3].cpu().numpy())
         outs[name] = (o, hh)
         r = {"value": B * world * args.steps / (ms / 1e3), "unit": "vectors/s", "ms_per_step": ms / args.steps,
@@ -837,7 +851,7 @@ def hybrid_record(args, rank, world, local, dev, dist, torch, mdx, replicas, pro
                                          sms, probe, B),
              "clocks": sampler.summary(), "per_snr": per_snr(w, hh, data["sym"])}
         if name == "plain":
-            r["qr_roofline"] = qr_roofline(n, n, B, prof, sms, probe)
+            r["qr_roofline"] = qr_roofline(n, n, B, qprof, sms, probe)
         rec[name] = r
     rec["identical_decisions"] = bool(torch.equal(outs["learned"][0][0], outs["plain"][0][0]))
     rec["speedup_learned"] = rec["learned"]["value"] / rec["plain"]["value"]

@@ -5,15 +5,16 @@
 //   FP32 FFMA  the tree searches' partial distances (Eq. 4 / Eq. inc) are
 //              FP32 FMAs; the probe runs 8 independent FFMA chains per
 //              thread on every SM.
-//   FP64 DFMA  the QR's panel (Householder reflectors, Sec. III-B) is FP64
-//              FMA work; 8 independent DFMA chains per thread.
-//   FP64 MMA   the QR's trailing updates are mma.sync m8n8k4 FP64 tiles; the
-//              probe runs 4 independent accumulator chains per warp and
-//              changes the A and B operand values before every MMA with an
-//              integer XOR of their lowest mantissa bit (an ALU-pipe op), so
-//              the hardware sees fresh operands each time, as in the QR.  A
-//              loop that feeds the same operands reads several times higher
-//              and does not describe real tiles.
+//   FP64 DFMA  the unit that the fixed-point QR (Householder reflectors, Sec.
+//              III-B) is compared with, and that of the re-scoring and the
+//              triangular solves; 8 independent DFMA chains per thread.
+//   FP64 MMA   the other route to it, mma.sync m8n8k4 FP64 tiles; the probe
+//              runs 4 independent accumulator chains per warp and changes the
+//              A and B operand values before every MMA with an integer XOR of
+//              their lowest mantissa bit (an ALU-pipe op), so the hardware
+//              sees fresh operands each time, as real tiles give it.  A loop
+//              that feeds the same operands reads several times higher and
+//              does not describe real tiles.
 // Flops count an FMA as two; an m8n8k4 MMA as 2 * 8 * 8 * 4 = 512.
 #include <cuda_runtime.h>
 
