@@ -759,9 +759,14 @@ cudaError_t launch_sd(const SearchArgs& a, const SdWorkspace& w, int num_sms, cu
   g.order = nullptr;
   cudaError_t e = cudaMemsetAsync(w.shared, 0, sizeof(SdShared), s);
   if (e != cudaSuccess) return e;
+  // Heaviest first only where vectors wait for a place: a warp holds four of up
+  // to 32 rows (some 80 an SM), or one of more rows (12 an SM).  Below, the
+  // order's four launches are the time (us a call with and without them: 500 vectors
+  // 12x9 94 and 81, 8,000 of 3x3 108 and 85, 20 of 8x8 87 and 74).
+  const int places = num_sms * (a.n <= 32 ? 64 : 8);
   if (w.ordered) {
     g.order = w.order;
-  } else if (a.noise_var && w.order && a.batch > 1) {
+  } else if (a.noise_var && w.order && a.batch > places) {
     int* order = w.order;
     unsigned int* cnt = reinterpret_cast<unsigned int*>(order + a.batch);
     e = cudaMemsetAsync(cnt, 0, sizeof(unsigned int) * kOrderBuckets, s);
