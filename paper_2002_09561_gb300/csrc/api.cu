@@ -68,9 +68,10 @@ struct mdx_ctx {
   size_t mx_gslot = 16;
   unsigned char* mx_scratch = nullptr;
   size_t mx_scratch_bytes = 0;
-  int mx_W = 8, mx_slice = 14336;
+  int mx_W = 8, mx_slice = 12288;
+  bool mx_tuned = false;
   int mx_walks = 0;     // exact SDs of the uploaded table, first in its order
-  int mx_used = 14336;  // the slice of the uploaded table (its walks' records at least)
+  int mx_used = 12288;  // the slice of the uploaded table (what its walks and selections need at least)
   std::vector<std::pair<unsigned long long, int>> mx_modes;  // class key -> MIX_* bits
   cudaGraphExec_t mx_graph = nullptr;
   std::vector<const void*> mx_graph_key;
@@ -504,7 +505,13 @@ mdx_status mixed_upload(mdx_ctx* c, int nreq, const mdx_request* reqs, cudaStrea
   if (same_table(c, nreq, reqs)) return MDX_OK;
   std::vector<MixedReq> d((size_t)nreq);
   long long roff = 0, yoff = 0;
-  int maxK = 0, slice = c->mx_slice;
+  // Walks and selections alone do better with more of the SM's memory as L1 than
+  // as slices (10,000 mixed requests with 8 / 9 / 11 / 12 / 14 KB a warp: 15.9 / 16.1 /
+  // 16.3 / 16.4 / 17.2 ms); the forms whose placement goes by the slice keep theirs
+  const bool placed = std::any_of(reqs, reqs + nreq, [](const mdx_request& q) {
+    return q.algo != MDX_ALGO_SD && (q.algo != MDX_ALGO_KBEST || q.K > 64);
+  });
+  int maxK = 0, slice = c->mx_tuned || placed ? c->mx_slice : 8192;
   size_t gslot = 16;
   std::vector<std::pair<double, int>> cost((size_t)nreq);
   for (int r = 0; r < nreq; ++r) {
@@ -800,6 +807,7 @@ mdx_status time_mixed(mdx_ctx* c, int nreq, const mdx_request* reqs, const doubl
 void set_tuning(mdx_ctx* c, int W, int slice, const std::vector<std::pair<unsigned long long, int>>& modes) {
   c->mx_W = W;
   c->mx_slice = slice;
+  c->mx_tuned = true;
   c->mx_modes = modes;
   c->mx_table.clear();  // descriptors are rebuilt with the new placement
 }
