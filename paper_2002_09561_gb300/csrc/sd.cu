@@ -11,7 +11,7 @@
 // expand) of one vector, explored depth-first by one warp.  A vector starts
 // as its root task.  Warps take work in this order: a queued task, else a
 // fresh vector (heaviest first, see launch_sd), else they wait (idle).  While any warp is idle, a busy warp
-// checks every kSplitEvery nodes and donates all untried children of its
+// checks every split_every nodes and donates all untried children of its
 // top-most open level whose next child is inside the sphere as new tasks,
 // marking that level exhausted.  The only
 // state the tasks of a vector share is its radius (an FP32 r^2 in global
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
       ++task_nodes;
 
       // periodic: radius refresh, budget, and splitting while warps are idle
-      if (++since >= kSplitEvery) {
+      if (++since >= g.split_every) {
         since = 0;
         SD_FOLD();
         const float gr2 = __uint_as_float(
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
         }
         // split only while more warps wait than tasks are queued for them
         int want = 0;
-        if (may_split && task_nodes >= kSplitMinNodes && lane == 0) {
+        if (may_split && task_nodes >= g.split_nodes && lane == 0) {
           const int idle_w = *(volatile int*)&g.sh->idle;
           const int queued = (int)(*(volatile unsigned int*)&g.sh->q_tail - *(volatile unsigned int*)&g.sh->q_head);
           want = idle_w > queued ? 1 : 0;
@@ -764,6 +764,16 @@ cudaError_t launch_sd(const SearchArgs& a, const SdWorkspace& w, int num_sms, cu
   // order's four launches are the time (us a call with and without them: 500 vectors
   // 12x9 94 and 81, 8,000 of 3x3 108 and 85, 20 of 8x8 87 and 74).
   const int places = num_sms * (a.n <= 32 ? 64 : 8);
+  // When a task splits: soon where the batch leaves workers idle from the start,
+  // later where they only fall idle at the end, and not sooner for small trees,
+  // which end by themselves (us a call with 512 / 128 nodes and with the rule's: 30
+  // and 300 vectors 16x16 16-QAM 275 -> 209 and 362 -> 292, 3,000 at 6 to 20 dB
+  // 1,721 -> 1,290, 1,000 of 24x24 905 -> 700; 20,000 of 10x10 64-QAM 753 -> 707,
+  // 8,000 of 24x24 4,178 -> 4,071; 300 of 8x8 131, 147 if split at 128).  A node
+  // budget is looked at as often, so its calls keep their cadence.
+  const bool few = a.batch <= places;
+  g.split_nodes = a.budget > 0 || a.n <= 16 ? 512 : few ? 128 : a.n <= 32 ? 256 : 384;
+  g.split_every = a.budget > 0 || a.n <= 16 || !few ? 128 : 64;
   if (w.ordered) {
     g.order = w.order;
   } else if (a.noise_var && w.order && a.batch > places) {

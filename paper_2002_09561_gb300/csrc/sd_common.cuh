@@ -27,10 +27,8 @@ struct SdShared {
 
 constexpr int kWarpsMax = 4;     // warps per CTA
 constexpr int kCand = 8;         // leaf candidates kept per vector
-constexpr int kSplitEvery = 128; // nodes between split / radius checks
 constexpr int kTaskPath = 224;   // path bytes in a task record (n <= 224)
 constexpr int kMinSplitLevel = 3; // donate only children with at least 3 rows below
-constexpr int kSplitMinNodes = 512; // a task donates only after searching this many nodes
 
 struct SdTask {
   unsigned long long seq;  // (epoch << 32) | (slot index + 1) once written
@@ -77,6 +75,8 @@ struct SdArgs {
   size_t vstride;
   unsigned long long epoch;
   const int* order;  // fresh vectors in this order (heaviest first), or null
+  int split_nodes;   // a task donates only after searching this many nodes,
+  int split_every;   // checked every so many (a multiple of 16)
 };
 
 __device__ __forceinline__ SdVec* vec_of(const SdArgs& g, int v) {

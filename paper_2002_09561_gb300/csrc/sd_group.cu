@@ -69,7 +69,7 @@
 // under a million tasks per second and left most groups idle for the last
 // half of a heavy-tailed batch) and waits until that slot is published.
 // While tickets outnumber the tasks reserved, a busy group that has searched
-// kSplitMinNodes nodes of its task donates the in-sphere children of its
+// split_nodes nodes of its task donates the in-sphere children of its
 // top-most open level (at least kMinSplitLevel rows above the leaves); from
 // then on the vector's radius is shared through atomicMin on its FP32 bits,
 // its tasks merge their candidates into the vector's list under its lock,
@@ -104,7 +104,7 @@ __host__ __device__ constexpr int group_warps() {
   return G >= 8 ? 2 : 1;
 }
 constexpr int kTri = 528;       // column-packed triangle of n = 32
-// node-step passes per vote of the slow paths (divides 16 and kSplitEvery);
+// node-step passes per vote of the slow paths (divides 16, and with it split_every);
 // a group that raised an event sits out the rest of them
 #ifndef MDX_SDG_PASSES
 #define MDX_SDG_PASSES 16
@@ -118,7 +118,6 @@ constexpr int kPassesPerVote = MDX_SDG_PASSES;
 #endif
 constexpr int kPassUnroll = MDX_SDG_UNROLL;
 static_assert(kPassesPerVote <= 16 && 16 % kPassesPerVote == 0, "the ticket check cadence");
-static_assert(kSplitEvery % kPassesPerVote == 0, "the split check cadence");
 
 // R and the residual stack in shared memory: column c (rows 0..c) starts at
 // zoff(c) = kTri - (c + 1)(c + 2) / 2, the columns in descending order.  A
@@ -291,9 +290,9 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
     const bool want = (mode == 0) || (mode == 2 && (recheck || (since & 15) == 16 - kPassesPerVote));
     // one vote per pass decides whether anything but the node step runs:
     // events of the last pass, groups that want work, the periodic check
-    if (__any_sync(full, ev_leaf || ev_done || want || since >= kSplitEvery)) {
+    if (__any_sync(full, ev_leaf || ev_done || want || since >= g.split_every)) {
       // ---------------------------------------------------- periodic check
-      if (since >= kSplitEvery) {
+      if (since >= g.split_every) {
         since = 0;
         recheck = true;
         const bool busy = mode == 1 && !ev_done;
@@ -338,7 +337,7 @@ __global__ void __launch_bounds__(group_warps<G>() * 32, MDX_SDG_MIN_BLOCKS) sd_
         }
         // donation while more groups wait than tasks are queued for them
         int wantd = 0;
-        if (busy && may_split && task_nodes >= kSplitMinNodes && gl == 0) {
+        if (busy && may_split && task_nodes >= g.split_nodes && gl == 0) {
           // tickets taken beyond the tasks reserved so far: groups waiting for work
           const int waiting = (int)(*(volatile unsigned int*)&g.sh->q_head - *(volatile unsigned int*)&g.sh->q_tail);
           wantd = waiting > 0 ? 1 : 0;

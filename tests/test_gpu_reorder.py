@@ -83,3 +83,19 @@ def test_sorted_search_with_the_network_and_host_buffers():
     mdx.detect_host("sd", ctx, p, w["H"], w["y"], w["noise_var"], sym, met, vst)
     assert np.array_equal(sym, want[0].cpu().numpy()) and np.array_equal(met, want[1].cpu().numpy())
     assert np.array_equal(vst, want[2].cpu().numpy())
+
+
+def test_vectors_that_fit_need_no_order():
+    """On both sides of the number of places (64 an SM up to 32 rows), with and without an order: the same answers."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = 64 * sms + 1
+    w = wl.generate(9477, B, 3, 3, 16, 14.0)
+    H, y, nv = (torch.from_numpy(w[k]).cuda() for k in ("H", "y", "noise_var"))
+    ctx = mdx.Context(0, B, 3, 3)
+    p = mdx.make_params(3, 3, 16, radius="paper")
+    every = mdx.detect("sd", ctx, p, H, y, nv)
+    most = mdx.detect("sd", ctx, p, H[:-1].contiguous(), y[:-1].contiguous(), nv[:-1].contiguous())
+    for a, b in zip(every[:3], most[:3]):
+        assert torch.equal(a[:-1], b)
