@@ -177,8 +177,15 @@ constexpr unsigned int kSdQueueSlots = 1u << 16;
 // Whether choosing antenna orders can pay (sd_reorder.cu chooses vector by
 // vector): a handful of vectors leaves the GPU idle, and the order's extra QR
 // takes longer than it saves (one 16x16 vector at 18 dB: 119 us a call
-// without, 155 with); trees of fewer than four antennas are small.
-bool reorder_pays(int batch, int n_tx) { return n_tx >= 4 && n_tx <= kReorderMaxTx && batch >= 32; }
+// without, 155 with); trees of fewer than four antennas are small, and those of
+// up to eight pay for the extra kernels with more vectors only (us sorted /
+// natural, 100 and 1,000 vectors: 4x4 64-QAM at 15 to 20 dB 129 / 142 and 157 /
+// 206, at 23 to 29 dB 85 / 70 and 105 / 92; 6x6 16-QAM at 10 to 16 dB 189 / 142 and
+// 244 / 287; 8x8 at 17 to 23 dB 116 / 95 and 143 / 135, at 8 to 16 dB 303 / 362 and
+// 429 / 435; 16x16 at 8 to 20 dB 424 / 447 and 593 / 722; 24x24 337 / 405, 698 / 1,401).
+bool reorder_pays(int batch, int n_tx) {
+  return n_tx >= 4 && n_tx <= kReorderMaxTx && batch >= (n_tx <= 8 ? 512 : 32);
+}
 
 mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, const double* H,
                       const double* y, const double* nv, uint8_t* sym, double* met, int32_t* vst,

@@ -28,7 +28,9 @@ def _both(ctx, p, H, y, nv):
     (4, 4, 16, 6.0, 33, "paper"), (5, 5, 64, 14.0, 700, math.inf), (9, 8, 16, 6.0, 1300, "paper"),
     (12, 9, 64, 16.0, 500, 0.5), (16, 16, 16, 8.0, 1300, "paper"), (16, 16, 4, 2.0, 1217, math.inf),
     (17, 17, 16, 16.0, 300, "paper"), (24, 24, 16, 18.0, 1900, "paper"), (25, 25, 4, 8.0, 200, 3.0),
-    (32, 32, 4, 9.0, 1900, "paper"), (36, 33, 4, 12.0, 40, "paper")])
+    (32, 32, 4, 9.0, 1900, "paper"), (36, 33, 4, 12.0, 40, "paper"),
+    (4, 4, 16, 6.0, 511, "paper"), (4, 4, 16, 6.0, 512, "paper"), (8, 8, 16, 8.0, 513, "paper"),
+    (9, 9, 16, 8.0, 32, "paper")])
 def test_sorted_search_returns_what_the_natural_one_does(N, M, qam, snr, B, radius):
     import torch
 
