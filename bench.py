@@ -90,10 +90,10 @@ KERNEL_SOURCES = {
     "100x100-64qam-hybrid32-learned": ("hybrid_warp.cu", "select_run.cuh", "warp_kbest.cuh", "mdx_internal.cuh"),
 }
 TRAFFIC_PER_VECTOR = {
-    "16x16-16qam-sd-learned": ((225.353472e6 + 5.748992e6) / 30000,
+    "16x16-16qam-sd-learned": ((225.393408e6 + 5.746176e6) / 30000,
                                "ncu capture of sd_group_kernel, 30,000 vectors of the learned 16x16 sweep "
                                "(profiles/search_and_qr_kernels.md), scaled by vectors",
-                               "7e12b2722ccb6bd4"),
+                               "155b845d7303518d"),
     "100x100-64qam-hybrid32-learned": ((369.485824e6 + 8.572928e6 + 30.755840e6 + 0.067840e6 + 216.549120e6
                                         + 6.335232e6) / 2000,
                                        "ncu capture of the hybrid's three search kernels, 2,000 vectors of the learned "
@@ -122,11 +122,11 @@ def code_hash(files, csrc=None):
 # tied to the sources in the same way: with the live node rate this gives the
 # kernel's instruction-issue rate, the resource that bounds it.
 INSTRUCTIONS_PER_NODE = {
-    "16x16-16qam-sd-learned": (1.2249798059e10 / 296364808,
+    "16x16-16qam-sd-learned": (1.2359628411e10 / 300102995,
                                "ncu capture of sd_group_kernel, 30,000 vectors of the learned 16x16 sweep: "
                                "smsp__inst_executed.sum over the launch's branched nodes "
                                "(profiles/search_and_qr_kernels.md)",
-                               "7e12b2722ccb6bd4"),
+                               "155b845d7303518d"),
 }
 
 
