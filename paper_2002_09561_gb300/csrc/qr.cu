@@ -1065,6 +1065,9 @@ __device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
     }
   }
   __syncthreads();
+  // (the barriers end here: the FP64 form takes this memory for other things)
+  for (int k = tid; k < M; k += blockDim.x)
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_at(bar + k)) : "memory");
   if (*flag) return false;
   if (out.Rdense)
     for (int t = tid; t < n * n; t += blockDim.x)
