@@ -200,6 +200,7 @@ __device__ void sd_natural(const MixedArgs& g, const MixedReq& q, int r, const f
         c = lv_c[i];
         rii = lv_rii[i];
         next = lv_k[i];
+        __syncwarp();  // the level's state is read before lane 0 writes it again
         continue;
       }
       const int k = next++;
@@ -514,6 +515,9 @@ __device__ void sd_walk(const MixedArgs& g, const MixedReq& q, int r, const floa
 #pragma unroll
       for (int t = 0; t < ROWS; ++t) z[t] = lane + 32 * t < i ? zi[lane + 32 * t] : 0.0f;
       z1 = i > 0 ? zi[i - 1] : 0.0f;
+      // a level's record and residuals, read by lanes that did not write them, are
+      // written again only after a pop: the reads so far come before
+      __syncwarp();
       reach();
     }
     if (ncand == 0 && !bh && r2_start < INFINITY && restarts < 64) {
@@ -521,6 +525,7 @@ __device__ void sd_walk(const MixedArgs& g, const MixedReq& q, int r, const floa
       r2_start *= 2.0f;
       r2 = r2_start;
       ++restarts;
+      __syncwarp();  // as after a pop
       continue;
     }
     break;
@@ -603,6 +608,7 @@ __device__ void sdc_request(const MixedArgs& g, const MixedReq& q, int r, const 
         c0 = s4.z;
         mask = (unsigned long long)__float_as_uint(s4.w) | ((unsigned long long)lv_hi[j] << 32);
         rl = lv_r[j];
+        __syncwarp();  // the level's state is read before lane 0 writes it again
         continue;
       }
       const int qk = (int)(best & 0xffffffffu);

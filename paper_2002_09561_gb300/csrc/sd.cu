@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(kWarpsMax * 32, ROWS == 1 ? MDX_SD_MIN_BLOCKS_
       lo = (lh & 0xff) - 1;
       ret = (lh >> 8) & 0xff;
       hi = lh >> 16;
+      __syncwarp();  // the level's state is read before lane 0 writes it again
       return true;
     };
     // budget left for this task's uncommitted nodes (n32 counts them)
