@@ -321,7 +321,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
     QrOut q{c->R64 + (size_t)b0 * tri_stride64(n), c->yb64 + (size_t)b0 * vec_stride64(n),
             c->R32 + (size_t)b0 * tri_stride32(n), c->yb32 + (size_t)b0 * vec_stride32(n),
             nullptr, nullptr, c->singular + b0};
-    e = launch_qr(nb, N, M, dH + (size_t)b0 * 2 * N * M, dy + (size_t)b0 * 2 * N, q, s);
+    e = launch_qr(nb, N, M, dH + (size_t)b0 * 2 * N * M, dy + (size_t)b0 * 2 * N, q, c->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "QR launch");
   }
 
@@ -643,7 +643,7 @@ cudaError_t mixed_launches(mdx_ctx* c, int nreq, const double* dH, const double*
   QrOut q{c->R64, c->yb64, c->R32, c->yb32, nullptr, nullptr, c->singular};
   for (size_t k = 0; k + 3 < c->mx_qr.size(); k += 4) {
     const cudaError_t e = launch_qr_gather(c->mx_qr[k + 3], c->mx_qr[k], c->mx_qr[k + 1], dids + c->mx_qr[k + 2],
-                                           dreqs, dH, dy, q, s);
+                                           dreqs, dH, dy, q, c->num_sms, s);
     if (e != cudaSuccess) return e;
   }
   cudaError_t e = cudaMemsetAsync(c->counter, 0, 2 * sizeof(unsigned int), s);
@@ -1045,7 +1045,7 @@ mdx_status mdx_qr(mdx_ctx* c, int batch, int n_rx, int n_tx, const double* H, co
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "earlier asynchronous error");
   QrOut q{nullptr, nullptr, nullptr, nullptr, R_out, ybar_out, nullptr};
-  e = launch_qr(batch, n_rx, n_tx, H, y, q, static_cast<cudaStream_t>(stream));
+  e = launch_qr(batch, n_rx, n_tx, H, y, q, c->num_sms, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(c, e, "QR launch");
   return MDX_OK;
 }
@@ -1234,7 +1234,7 @@ static mdx_status mlp_prepare(mdx_ctx* c, const mdx_params* p, int batch, const 
     if (!is_device_ptr(q, c->device)) return fail(c, MDX_EINVAL, "pointer %p is not device memory", q);
   const int rows = round_up(batch, 128);
   QrOut q{c->R64, c->yb64, c->R32, c->yb32, nullptr, nullptr, c->singular};
-  cudaError_t e = launch_qr(batch, p->n_rx, p->n_tx, H, y, q, s);
+  cudaError_t e = launch_qr(batch, p->n_rx, p->n_tx, H, y, q, c->num_sms, s);
   if (e == cudaSuccess) e = mlp_features(c->mlp, batch, rows, c->R32, c->yb32, nv, train, feat_out, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "features");
   *rows_out = rows;

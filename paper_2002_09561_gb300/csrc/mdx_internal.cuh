@@ -104,7 +104,7 @@ struct AugArgs {
 };
 cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s);
 
-cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out,
+cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out, int num_sms,
                       cudaStream_t s);
 
 // One request of an uneven batch as the device sees it (built by the host
@@ -133,7 +133,7 @@ enum { MIX_STAGE_R = 1, MIX_STATE_SMEM = 2 };
 enum { MIX_ALGO_SD_COMPLEX = 2, MIX_ALGO_SD_NATURAL = 3 };
 
 cudaError_t launch_qr_gather(int count, int n_rx, int n_tx, const int* ids, const MixedReq* reqs,
-                             const double* H, const double* y, QrOut out, cudaStream_t s);
+                             const double* H, const double* y, QrOut out, int num_sms, cudaStream_t s);
 
 struct MixedArgs {
   int nreq;

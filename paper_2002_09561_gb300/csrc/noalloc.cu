@@ -131,7 +131,7 @@ extern "C" mdx_status detect_kbest_noalloc(const mdx_params* p, int batch, const
   QrOut q{reinterpret_cast<double*>(base + oR64), reinterpret_cast<double*>(base + oy64),
           reinterpret_cast<float*>(base + oR32), reinterpret_cast<float*>(base + oy32), nullptr, nullptr,
           reinterpret_cast<int*>(base + osing)};
-  if (launch_qr(batch, N, M, H, y, q, s) != cudaSuccess) return MDX_ECUDA;
+  if (launch_qr(batch, N, M, H, y, q, sms, s) != cudaSuccess) return MDX_ECUDA;
 
   SearchArgs a{};
   a.batch = batch;

@@ -8,7 +8,7 @@
 // (qr_cta_kernel).  The few matrices that a fixed scale per column does not
 // suit (a residual column below 2^-26 of its norm: singular or nearly so;
 // infinities, NaN and exponents near the ends of the range) are factored by
-// the FP64 forms (qr64_one).  The complex R is written out in the real
+// the FP64 forms (qr_small64, qr_one).  The complex R is written out in the real
 // interleaved form (entry r_ab -> [[Re,-Im],[Im,Re]]) that the tree search
 // uses.
 //
@@ -158,8 +158,8 @@ __device__ void qr_one(int N, int M, const double2* __restrict__ Hb, const doubl
   for (int k = 0; k < M; ++k) {
     double2* col = A + (size_t)k * N;
     if (tid < 32) {
-      // warp 0 forms the reflector; with LPC = 16 both half-warps compute the
-      // same sums, so full-warp shuffles stay uniform
+      // warp 0 forms the reflector; with LPC < 32 its workers all compute the same
+      // sums, so full-warp shuffles stay uniform
       double s = 0.0;
       for (int i = k + lane_g; i < N; i += LPC) s += col[i].x * col[i].x + col[i].y * col[i].y;
       s = group_sum<LPC>(s);
@@ -196,8 +196,13 @@ __device__ void qr_one(int N, int M, const double2* __restrict__ Hb, const doubl
         if (act) {
           for (int i = k + lane_g; i < N; i += LPC) {
             const double2 v = col[i], a = cj[i];
-            wr += v.x * a.x + v.y * a.y;
-            wi += v.x * a.y - v.y * a.x;
+            if constexpr (LPC == 32) {
+              wr += v.x * a.x + v.y * a.y;
+              wi += v.x * a.y - v.y * a.x;
+            } else {  // eight FP64 instructions an entry instead of twelve
+              wr = fma(v.x, a.x, fma(v.y, a.y, wr));
+              wi = fma(v.x, a.y, fma(-v.y, a.x, wi));
+            }
           }
         }
         wr = group_sum<LPC>(wr) * t;
@@ -206,8 +211,13 @@ __device__ void qr_one(int N, int M, const double2* __restrict__ Hb, const doubl
           for (int i = k + lane_g; i < N; i += LPC) {
             const double2 v = col[i];
             double2 a = cj[i];
-            a.x -= v.x * wr - v.y * wi;
-            a.y -= v.x * wi + v.y * wr;
+            if constexpr (LPC == 32) {
+              a.x -= v.x * wr - v.y * wi;
+              a.y -= v.x * wi + v.y * wr;
+            } else {
+              a.x = fma(-v.x, wr, fma(v.y, wi, a.x));
+              a.y = fma(-v.x, wi, fma(-v.y, wr, a.y));
+            }
             cj[i] = a;
           }
         }
@@ -283,10 +293,11 @@ __device__ __forceinline__ void put_y(const QrDst& out, int k, u64 re, u64 im) {
 }
 
 // ---------------------------------------------------------------------------
-// The FP64 form of a small system (n_rx <= 32): one matrix by one warp, column
-// by column in the left-looking order, lane h < L holding rows L q + h of the
-// current column (the other lanes run along on zeros).  V, Tau: qs_vo(M, N)
-// reflector entries and M scalars of shared memory.
+// The FP64 form of a small system (n_rx <= 32), column by column in the
+// left-looking order, L lanes per matrix: lane h of the group holds rows L q + h
+// of the current column.  kMats matrices by the warp (32 / L, or one by its first
+// group, the other lanes running along on zeros).  V, Tau: kMats qs_vo(M, N)
+// reflector entries, the matrices innermost, and kMats M scalars of shared memory.
 __host__ __device__ inline int qs_vo(int k, int N) { return k * N - k * (k - 1) / 2; }  // first entry of v_k
 // Conversions between a positive normal double in [1e-30, 1e30] and a float
 // estimate of it, done on the integer pipe (rebias the exponent, keep the top
@@ -321,13 +332,14 @@ __device__ __forceinline__ double rcp64(double d) {
   return fma(y, fma(e, e, e), y);
 }
 
-template <int L>
-__device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, const double2* __restrict__ yv,
-                               const QrDst& out, double2* V, double* Tau) {
+template <int L, int kMats>
+__device__ void qr_small64(int N, int M, bool act, const double2* __restrict__ Hb, const double2* __restrict__ yv,
+                           const QrDst& out, double2* V, double* Tau) {
   constexpr int kQsSlots = 8;  // rows per lane (N <= 8 L)
   const int lane = threadIdx.x & 31, h = lane % L;
-  const bool act = lane < L;
   const int n = 2 * M;
+  V += lane / L % kMats;
+  Tau += lane / L % kMats;
   double2 a[kQsSlots], ph[kQsSlots];
 #pragma unroll
   for (int q = 0; q < kQsSlots; ++q) ph[q] = make_double2(1.0, 0.0);
@@ -342,14 +354,14 @@ __device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, con
     // reflectors 0 .. j-1: a <- a - v_k tau_k (v_k^H a) over rows k..N-1
     const int kend = j < M ? j : M;
     for (int k = 0; k < kend; ++k) {
-      const double2* vk = V + (size_t)(qs_vo(k, N) - k);  // entry r at vk[r]
+      const double2* vk = V + (size_t)(qs_vo(k, N) - k) * kMats;  // entry r at vk[r kMats]
       double wr = 0.0, wi = 0.0;
 #pragma unroll
       for (int q = 0; q < kQsSlots; ++q) {
         const int r = L * q + h;
         if (L * q + L - 1 < k || L * q >= N) continue;  // no lane of the group has this row
         if (r >= k && r < N) {
-          const double2 v = vk[r];
+          const double2 v = vk[r * kMats];
           wr = fma(v.x, a[q].x, fma(v.y, a[q].y, wr));
           wi = fma(v.x, a[q].y, fma(-v.y, a[q].x, wi));
         }
@@ -359,7 +371,7 @@ __device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, con
         wr += __shfl_xor_sync(0xffffffffu, wr, o);
         wi += __shfl_xor_sync(0xffffffffu, wi, o);
       }
-      const double tk = Tau[k];
+      const double tk = Tau[k * kMats];
       wr *= tk;
       wi *= tk;
 #pragma unroll
@@ -367,7 +379,7 @@ __device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, con
         const int r = L * q + h;
         if (L * q + L - 1 < k || L * q >= N) continue;
         if (r >= k && r < N) {
-          const double2 v = vk[r];
+          const double2 v = vk[r * kMats];
           a[q].x = fma(-v.x, wr, fma(v.y, wi, a[q].x));
           a[q].y = fma(-v.x, wi, fma(-v.y, wr, a[q].y));
         }
@@ -417,14 +429,14 @@ __device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, con
       } else {
         sing = 1;
       }
-      double2* vj = V + (size_t)(qs_vo(j, N) - j);
+      double2* vj = V + (size_t)(qs_vo(j, N) - j) * kMats;
 #pragma unroll
       for (int q = 0; q < kQsSlots; ++q) {
         const int r = L * q + h;
-        if (act && r >= j && r < N) vj[r] = (r == j) ? make_double2(x0.x - al.x, x0.y - al.y) : a[q];
+        if (act && r >= j && r < N) vj[r * kMats] = (r == j) ? make_double2(x0.x - al.x, x0.y - al.y) : a[q];
         if (r == j) ph[q] = phr;
       }
-      if (lane == 0) Tau[j] = tj;
+      if (act && h == 0) Tau[j * kMats] = tj;
       if (act && h == h0) put_r(out, n, j, j, (u64)__double_as_longlong(sigma), 0);
     } else {
       // ybar = Q^H y: rows k < M of the y column, phase-fixed
@@ -448,25 +460,27 @@ __device__ void qr_small64_one(int N, int M, const double2* __restrict__ Hb, con
 }
 
 
-__host__ __device__ inline size_t qr64_smem(int N, int M) {
-  return N <= 32 ? sizeof(double2) * (size_t)qs_vo(M, N) + sizeof(double) * (size_t)M
-                 : sizeof(double2) * ((size_t)(M + 1) * N + M) + sizeof(double) * M + sizeof(int) * 4;
+// Lanes per matrix (as few as hold the column in eight slots: every FP64
+// instruction then serves many rows), and shared memory of `mats` matrices.
+__host__ __device__ inline int qs64_lanes(int N) { return N <= 16 ? 2 : 4; }
+__host__ __device__ inline size_t qs64_smem(int N, int M, int mats) {
+  return (sizeof(double2) * (size_t)qs_vo(M, N) + sizeof(double) * (size_t)M) * mats;
 }
-// Factorises one [H | y] in FP64 with the calling CTA.
-__device__ __noinline__ void qr64_one(int N, int M, const double* Hb, const double* yb, const QrDst& out) {
+// Factorises one [H | y] (n_rx <= 32) in FP64 with the calling CTA's first warp.
+__device__ __noinline__ void qr_small64_one(int N, int M, const double* Hb, const double* yb, const QrDst& out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const double2* H2 = reinterpret_cast<const double2*>(Hb);
   const double2* y2 = reinterpret_cast<const double2*>(yb);
-  if (N > 32) {
-    qr_one<32>(N, M, H2, y2, out);
-  } else if (threadIdx.x < 32) {
-    double2* V = reinterpret_cast<double2*>(smem_raw);
-    double* Tau = reinterpret_cast<double*>(V + qs_vo(M, N));
-    if (N <= 16)
-      qr_small64_one<2>(N, M, H2, y2, out, V, Tau);
-    else
-      qr_small64_one<4>(N, M, H2, y2, out, V, Tau);
-  }
+  if (threadIdx.x >= 32) return;
+  double2* V = reinterpret_cast<double2*>(smem_raw);
+  double* Tau = reinterpret_cast<double*>(V + qs_vo(M, N));
+  if (qs64_lanes(N) == 2)
+    qr_small64<2, 1>(N, M, threadIdx.x < 2, H2, y2, out, V, Tau);
+  else
+    qr_small64<4, 1>(N, M, threadIdx.x < 4, H2, y2, out, V, Tau);
+}
+__host__ __device__ inline size_t qr_one_smem(int N, int M) {
+  return sizeof(double2) * ((size_t)(M + 1) * N + M) + sizeof(double) * M + sizeof(int) * 4;
 }
 
 // a conj(p) of a fixed-point entry and a phase p (limbs), as double bits.
@@ -782,7 +796,7 @@ __device__ __forceinline__ QrDst batch_dst(const QrOut& out, int b, int n) {
 // One matrix of a launch: input, output, shape.  A uniform batch has ids =
 // null; an uneven one lists its requests (all of one shape) in ids.
 struct QrBatch {
-  int count, N, M;
+  int count, N, M, num_sms;
   const int* ids;
   const MixedReq* reqs;
   const double* H;
@@ -837,21 +851,66 @@ __global__ void __launch_bounds__(32) qr_reorder_small_kernel(ReorderArgs g, int
   qr_small_pair<L, SL>(g.a.n_tx, g.a.n_tx, act, src, d, reinterpret_cast<int4*>(smem_raw));
 }
 
-// The matrices that qr_small_kernel left, in FP64.
-__global__ void qr_redo_kernel(QrBatch g) {
-  const int n = 2 * g.M;
-  for (int base = blockIdx.x * blockDim.x; base < g.count; base += gridDim.x * blockDim.x) {
-    const double *Hb, *yb;
-    const int i = base + threadIdx.x;
-    const bool mine = i < g.count && is_redo(g.get(i, Hb, yb), n);
-    if (!__syncthreads_or(mine)) continue;
-    for (int t = base; t < min(g.count, base + (int)blockDim.x); ++t) {
-      const QrDst d = g.get(t, Hb, yb);
-      if (!is_redo(d, n)) continue;
-      __syncthreads();  // every thread has read the mark that qr_one overwrites
-      qr64_one(g.N, g.M, Hb, yb, d);
-      __syncthreads();
+// The matrices that the fixed-point forms left, in FP64: n_rx <= 32, 32 / L of
+// them per warp.  A warp looks through `per` matrices of the batch and factors
+// the marked ones as it finds them, a warp full at a time: a batch of nothing but
+// such matrices (keyhole or line-of-sight channels, copied columns) keeps the GPU
+// as full as one kernel for all of them would.  Whole calls, a column twice in
+// every matrix, us (128 matrices to a CTA, one after another, before / now; in
+// brackets 1 % of them so): 10,000 of 16x16 52,117 / 726 (2,284 / 616), 100,000
+// 157,397 / 5,305, 10,000 of 32x32 185,917 / 5,518; 1,000 of 64x64 130,993 / 3,283,
+// of 100x100 346,849 / 11,686 (10,781 / 5,238).
+template <int L>
+__global__ void __launch_bounds__(32) qr_redo_small_kernel(QrBatch g, int per) {
+  constexpr int mats = 32 / L;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int list[mats + 32];
+  double2* V = reinterpret_cast<double2*>(smem_raw);
+  double* Tau = reinterpret_cast<double*>(V + (size_t)mats * qs_vo(g.M, g.N));
+  const int lane = threadIdx.x & 31, end = min(g.count, ((int)blockIdx.x + 1) * per);
+  int base = blockIdx.x * per, have = 0;
+  const double *Hb, *yb;
+  for (;;) {
+    for (; have < mats && base < end; base += 32) {
+      const int i = base + lane;
+      const bool mine = i < end && is_redo(g.get(i, Hb, yb), 2 * g.M);
+      const unsigned who = __ballot_sync(0xffffffffu, mine);
+      if (mine) list[have + __popc(who & ((1u << lane) - 1u))] = i;
+      have += __popc(who);
     }
+    if (have == 0) return;
+    __syncwarp();
+    const bool act = lane / L < have;
+    const QrDst d = g.get(list[act ? lane / L : 0], Hb, yb);
+    qr_small64<L, mats>(g.N, g.M, act, reinterpret_cast<const double2*>(Hb), reinterpret_cast<const double2*>(yb), d, V,
+                        Tau);
+    have = max(have - mats, 0);
+    const int next = lane < have ? list[mats + lane] : 0;
+    __syncwarp();
+    if (lane < have) list[lane] = next;
+    __syncwarp();
+  }
+}
+// n_rx > 32: a CTA each, CTA b the marked ones among matrices b, b + grid, ...
+// LPC lanes per column: 32 below 48 antennas; above, where a reduction over 32
+// lanes would be half of a column's FP64 instructions, 8.
+template <int LPC>
+__global__ void __launch_bounds__(256) qr_redo_kernel(QrBatch g) {
+  __shared__ unsigned marks[8];
+  const int n = 2 * g.M;
+  const double *Hb, *yb;
+  for (int base = blockIdx.x; base < g.count; base += gridDim.x * 256) {
+    const int i = base + threadIdx.x * gridDim.x;
+    const unsigned who = __ballot_sync(0xffffffffu, i < g.count && is_redo(g.get(i, Hb, yb), n));
+    if ((threadIdx.x & 31) == 0) marks[threadIdx.x >> 5] = who;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w)
+      for (unsigned left = marks[w]; left; left &= left - 1) {
+        const QrDst d = g.get(base + (32 * w + __ffs(left) - 1) * gridDim.x, Hb, yb);
+        qr_one<LPC>(g.N, g.M, reinterpret_cast<const double2*>(Hb), reinterpret_cast<const double2*>(yb), d);
+        __syncthreads();
+      }
+    __syncthreads();  // the marks are read
   }
 }
 
@@ -1076,14 +1135,14 @@ __device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
 }
 
 template <int L, int SL, int T, int B>
-__global__ void __launch_bounds__(T, B) qr_cta_kernel(QrBatch g) {
+__global__ void __launch_bounds__(T, B) qr_cta_kernel(QrBatch g, int here) {
   const double *Hb, *yb;
   const QrDst d = g.get(blockIdx.x, Hb, yb);
   const SrcH src{reinterpret_cast<const longlong2*>(Hb), reinterpret_cast<const longlong2*>(yb), g.M};
   const bool ok = qr_cta_one<L, SL>(g.N, g.M, src, d);
-  __syncthreads();  // the zeroed triangle, before the mark in it; the shared memory, before qr64_one
-  if (!ok && g.N <= 32)
-    qr64_one(g.N, g.M, Hb, yb, d);
+  __syncthreads();  // the zeroed triangle, before the mark in it; the shared memory, before the FP64 form
+  if (!ok && here)
+    qr_small64_one(g.N, g.M, Hb, yb, d);
   else if (threadIdx.x == 0)
     mark_redo(d, 2 * g.M, !ok);
 }
@@ -1133,14 +1192,32 @@ __global__ void __launch_bounds__(288, 2) qr_aug_cta_kernel(AugArgs g) {
 size_t qr_cta_smem(int n_rx, int n_tx) {
   QrCtaLayout L;
   L.init(n_rx, n_tx);
-  return n_rx <= 32 ? std::max(L.bytes, qr64_smem(n_rx, n_tx)) : L.bytes;
+  return n_rx <= 32 ? std::max(L.bytes, qs64_smem(n_rx, n_tx, 1)) : L.bytes;
 }
 
-cudaError_t launch_redo(const QrBatch& g, cudaStream_t s) {
-  const size_t sm = qr64_smem(g.N, g.M);
-  cudaFuncSetAttribute(qr_redo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  qr_redo_kernel<<<std::min((g.count + 127) / 128, 304), 128, sm, s>>>(g);
+// CTAs an SM's shared memory holds (a kilobyte each is the system's).
+int smem_ctas(size_t bytes, int most) { return std::max(1, std::min(most, (int)(228 * 1024 / (bytes + 1024)))); }
+
+template <int L>
+cudaError_t launch_redo_small(const QrBatch& g, cudaStream_t s) {
+  constexpr int mats = 32 / L;
+  const size_t sm = qs64_smem(g.N, g.M, mats);
+  const int warps = (g.count + mats - 1) / mats, most = g.num_sms * smem_ctas(sm + 256, 32);
+  const int turns = (warps + most - 1) / most;
+  cudaFuncSetAttribute(qr_redo_small_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_redo_small_kernel<L><<<(warps + turns - 1) / turns, 32, sm, s>>>(g, turns * mats);
   return cudaGetLastError();
+}
+template <int LPC>
+cudaError_t launch_redo_large(const QrBatch& g, cudaStream_t s) {
+  const size_t sm = qr_one_smem(g.N, g.M);
+  cudaFuncSetAttribute(qr_redo_kernel<LPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  qr_redo_kernel<LPC><<<std::min(g.count, g.num_sms * smem_ctas(sm + 32, 4)), 256, sm, s>>>(g);
+  return cudaGetLastError();
+}
+cudaError_t launch_redo(const QrBatch& g, cudaStream_t s) {
+  if (g.N <= 32) return qs64_lanes(g.N) == 2 ? launch_redo_small<2>(g, s) : launch_redo_small<4>(g, s);
+  return g.M < 48 ? launch_redo_large<32>(g, s) : launch_redo_large<8>(g, s);
 }
 
 template <int L, int SL>
@@ -1157,9 +1234,15 @@ template <int L, int SL, int T, int B>
 cudaError_t launch_qc(const QrBatch& g, int most, cudaStream_t s) {
   const size_t sm = qr_cta_smem(g.N, g.M);
   cudaFuncSetAttribute(qr_cta_kernel<L, SL, T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  qr_cta_kernel<L, SL, T, B><<<g.count, qc_threads(L, g.M, most), sm, s>>>(g);
+  // A small matrix left to FP64 is factored by its own CTA, which spares a launch
+  // (5 us of 90 for 1,216 of 16x16): up to a matrix per scheduler that takes no
+  // longer; for the few more of n_rx <= 16 that come here (all dependent, 1,216: 951
+  // us, 480 by the launch) the ordinary call counts, above (1,824 of 32x32: 5.1 ms,
+  // 1.7 by the launch) the others.
+  const bool here = g.N <= 16 || (g.N <= 32 && g.count <= 4 * g.num_sms);
+  qr_cta_kernel<L, SL, T, B><<<g.count, qc_threads(L, g.M, most), sm, s>>>(g, here);
   const cudaError_t e = cudaGetLastError();
-  return e != cudaSuccess || g.N <= 32 ? e : launch_redo(g, s);
+  return e != cudaSuccess || here ? e : launch_redo(g, s);
 }
 
 // Lanes per matrix of qr_small_kernel, or 0: qr_cta_kernel.  A warp of the
@@ -1280,13 +1363,13 @@ cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s) {
 }
 
 cudaError_t launch_qr_gather(int count, int n_rx, int n_tx, const int* ids, const MixedReq* reqs,
-                             const double* H, const double* y, QrOut out, cudaStream_t s) {
-  return launch(QrBatch{count, n_rx, n_tx, ids, reqs, H, y, out}, s);
+                             const double* H, const double* y, QrOut out, int num_sms, cudaStream_t s) {
+  return launch(QrBatch{count, n_rx, n_tx, num_sms, ids, reqs, H, y, out}, s);
 }
 
-cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out,
+cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out, int num_sms,
                       cudaStream_t s) {
-  return launch(QrBatch{batch, n_rx, n_tx, nullptr, nullptr, H, y, out}, s);
+  return launch(QrBatch{batch, n_rx, n_tx, num_sms, nullptr, nullptr, H, y, out}, s);
 }
 
 }  // namespace mdx
