@@ -7,8 +7,9 @@
 // search on the bits (one compare and add per child and one warp reduction a
 // step) finds the K-th smallest.  Sorting 64-bit
 // keys, the ALU work that bound the CTA kernel (kbest.cu), disappears, and so
-// do its CTA barriers.  A vector whose cut a tie straddles (about 1 in 3,000
-// at K = 64, 16x16) is marked and left to that kernel, which sorts.
+// do its CTA barriers.  Where a tie straddles a cut the parents' distances say
+// which children stay; only where those are equal as well is the vector marked
+// and left to that kernel, which sorts.
 //
 // Survivor paths are bytes 2k - (P - 1) in depth order (row n - 1 first, so
 // that the rows fixed so far are a prefix), the stride an odd number of
@@ -89,6 +90,66 @@ __device__ __forceinline__ float interference1(const float* Rc, const float* yb,
       if (b + m < d) c = fmaf(-Rc[col_off(n - 1 - b - m) + i], level_of(w, m, alpha), c);
   }
   return c;
+}
+
+// Keeps, of the children at the distance T that a cut of K straddles, those of
+// the lower parent ranks, then the lower children.  Ranks go by distance, so the
+// parents' distances tell; false where they are equal and it matters.  (A call
+// on copies: in line its registers cost every level 2 %.)
+template <int SL, int C>
+__device__ __noinline__ bool resolve_cut_at(unsigned* key, unsigned T, int K, const float* ped) {
+  int need = K;
+  uint64_t tied[SL];
+#pragma unroll
+  for (int q = 0; q < SL; ++q) tied[q] = 0;
+#pragma unroll
+  for (int j = 0; j < SL * C; ++j) {
+    need -= __popc(__ballot_sync(0xffffffffu, key[j] < T));
+    if (key[j] == T) {
+      tied[j / C] |= 1ull << (j % C);
+      key[j] = 0xffffffffu;
+    }
+  }
+  while (need > 0) {
+    unsigned low = 0xffffffffu;
+#pragma unroll
+    for (int q = 0; q < SL; ++q)
+      if (tied[q]) low = min(low, __float_as_uint(ped[q]));
+    const unsigned m = __reduce_min_sync(0xffffffffu, low);
+    int parents = 0, children = 0;
+#pragma unroll
+    for (int q = 0; q < SL; ++q)
+      if (tied[q] && __float_as_uint(ped[q]) == m) {
+        ++parents;
+        children += __popcll(tied[q]);
+      }
+    children = __reduce_add_sync(0xffffffffu, children);
+    if (children > need && __reduce_add_sync(0xffffffffu, parents) > 1) return false;
+#pragma unroll
+    for (int q = 0; q < SL; ++q)
+      if (tied[q] && __float_as_uint(ped[q]) == m) {
+        int left = need;
+#pragma unroll
+        for (int k = 0; k < C; ++k)
+          if ((tied[q] >> k) & 1ull && left-- > 0) key[q * C + k] = T;
+        tied[q] = 0;
+      }
+    need -= children;
+  }
+  return true;
+}
+template <int SL, int C>
+__device__ __forceinline__ bool resolve_cut(unsigned (&key)[SL * C], unsigned T, int K, const float (&ped)[SL]) {
+  unsigned k[SL * C];
+  float p[SL];
+#pragma unroll
+  for (int j = 0; j < SL * C; ++j) k[j] = key[j];
+#pragma unroll
+  for (int q = 0; q < SL; ++q) p[q] = ped[q];
+  if (!resolve_cut_at<SL, C>(k, T, K, p)) return false;
+#pragma unroll
+  for (int j = 0; j < SL * C; ++j) key[j] = k[j];
+  return true;
 }
 
 // SL survivors per lane (K <= 32 SL), C children per survivor: the PAM size P
@@ -185,7 +246,7 @@ __global__ void __launch_bounds__(kWarps * 32) kbest_warp_kernel(SearchArgs a, K
       flops += CPLX ? (long long)S * (4 * (n - 1 - i) + 10 * C) : (long long)S * (2 * (n - 1 - i) + 4 * C);
       unsigned T;
       int kept;
-      if (!level_cut<SL, C>(key, S, K, lane, T, kept)) {
+      if (!level_cut<SL, C>(key, S, K, lane, T, kept) && !resolve_cut<SL, C>(key, T, K, ped)) {
         tie = true;
         break;
       }
@@ -245,8 +306,8 @@ __global__ void __launch_bounds__(kWarps * 32) kbest_warp_kernel(SearchArgs a, K
 #pragma unroll
       for (int q = 0; q < SL; ++q)
         if (slot[t] == lane + 32 * q) ped[q] = __uint_as_float(0xffffffffu);  // taken
-      if (t == kCandMax - 1) {
-        bool same = false;  // another leaf at the last one's distance
+      if (t == kCandMax - 1 && __uint_as_float(m) <= prune_bound(best, E, n)) {
+        bool same = false;  // another leaf at the last one's distance, and it counts
 #pragma unroll
         for (int q = 0; q < SL; ++q) same |= lane + 32 * q < S && __float_as_uint(ped[q]) == m;
         if (__any_sync(0xffffffffu, same)) tie = true;
