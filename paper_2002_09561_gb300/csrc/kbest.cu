@@ -1249,9 +1249,9 @@ cudaError_t launch_kbest(const SearchArgs& a, int num_sms, cudaStream_t s) {
   else
     kb_geometry(L, a.n, a.K, a.P);
   if (L.bytes > 227 * 1024) return cudaErrorInvalidConfiguration;
-  // a vector per warp, and the few with a tie at a cut by the sorting kernel;
-  // where the warp form does not fit, all of them
-  const cudaError_t e = launch_kbest_warp(a, L.E > 0, s);
+  // a vector per warp, and what it leaves (ties) by the sorting kernel; where the
+  // warp form does not fit or pay, all of them
+  const cudaError_t e = launch_kbest_warp(a, L.E > 0, num_sms, s);
   if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
   return launch_generic((const void*)kbest_kernel, a, L, L.T, num_sms, s, e == cudaSuccess);
 }

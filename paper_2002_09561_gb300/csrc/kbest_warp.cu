@@ -405,15 +405,45 @@ cudaError_t launch_kw_k(const SearchArgs& a, const KwLayout& L, bool eight, cuda
   return cudaErrorNotSupported;
 }
 
+// Where a vector per warp (`warps` of them on an SM) is faster than the sorting
+// CTA.  A warp takes its lanes' children one after another, so a vector alone
+// takes longer where a lane has many survivors (large K of few children: the CTA
+// sorts those on many threads); with the SMs full, the warp's fewer instructions
+// win, except where its shared memory leaves an SM one CTA.  A cut of K <= 4 is a
+// sort of a few keys.  Measured, time of the warp form over the sorting one, whole
+// calls with the QR, 150 / 600 / 2,500 vectors:
+//   real tree    K = 4 64-QAM 16 rows 1.10 / 1.14 / 1.10, 64 rows 1.17 / 1.12 / 1.20; 4-QAM 64 rows 0.91 / 0.95 / 1.10
+//                K = 32 64 rows, 4-QAM 0.58 / 0.61 / 0.67, 64-QAM 0.60 / 0.57 / 0.51
+//                K = 256 4-QAM 32 rows 1.56 / 0.98 / 0.77, 64 rows (a CTA on an SM) 2.25 / 1.29 / 1.54;
+//                16-QAM 32 rows 1.27 / 0.50 / 0.37; 64-QAM 32 rows 0.85 / 0.27 / 0.20
+//   complex tree K = 4 16 rows, 16-QAM 1.18 / 1.19 / 1.11, 64-QAM 1.23 / 1.14 / 0.99
+//                K = 16 32 rows, 4-QAM 1.08 / 1.10 / 0.99, 16-QAM 1.06 / 0.94 / 0.61, 64-QAM 1.24 / 0.63 / 0.40
+//                K = 32 32 rows, 4-QAM 0.92 / 0.93 / 0.75, 64-QAM 0.90 / 0.37 / 0.21
+//                K = 128 32 rows, 4-QAM 1.47 / 0.96 / 0.71, 16-QAM 1.32 / 0.53 / 0.33
+//                K = 48 4-QAM 96 rows (a CTA on an SM) 1.34 / 1.13 / 1.44
+bool selection_pays(const SearchArgs& a, int warps, int num_sms) {
+  const int K = a.K, P = a.P, per_sm = (a.batch + num_sms - 1) / num_sms;
+  if (!(a.flags & MDX_COMPLEX_TREE)) {
+    if (K <= 4) return P < 8 && a.n > 32;
+    if (K > 128 && P < 8) return per_sm > 2 && !(P == 2 && warps <= 4);
+    return true;
+  }
+  if (K <= 4) return P == 8 && per_sm > 8 && warps > 8;
+  if (K <= 16 && P == 2) return per_sm > 8 && warps > 16;
+  if (K > 16 && (P == 8 || (P == 2 && K <= 32))) return true;
+  return per_sm > (P == 2 || warps <= 8 ? 2 : 1) && !(P == 2 && warps <= 4);
+}
+
 }  // namespace
 
-// Runs where a lane's children fit in registers (64 distances) and four
-// vectors in an SM's shared memory; else cudaErrorNotSupported, nothing
-// launched.
-cudaError_t launch_kbest_warp(const SearchArgs& a, bool eight, cudaStream_t s) {
+// Runs where a lane's children fit in registers (64 distances), four vectors
+// in an SM's shared memory, and where it pays; else cudaErrorNotSupported,
+// nothing launched.
+cudaError_t launch_kbest_warp(const SearchArgs& a, bool eight, int num_sms, cudaStream_t s) {
   KwLayout L;
   L.init(a.n, a.K);
-  if (L.warp_bytes * kWarps > 227 * 1024) return cudaErrorNotSupported;
+  const int ctas = (int)(228 * 1024 / (L.warp_bytes * kWarps + 1024));
+  if (L.warp_bytes * kWarps > 227 * 1024 || !selection_pays(a, ctas * kWarps, num_sms)) return cudaErrorNotSupported;
   if (a.flags & MDX_COMPLEX_TREE) {
     if (a.P == 2) return launch_kw_k<4, true>(a, L, eight, s);
     if (a.P == 4) return launch_kw_k<16, true>(a, L, eight, s);

@@ -202,7 +202,7 @@ cudaError_t launch_kbest(const SearchArgs& a, int num_sms, cudaStream_t s);
 // chains (else one).  Vectors it leaves to the sorting kernel get this mark in
 // their singular flag.
 constexpr int kKbestRedo = 2;
-cudaError_t launch_kbest_warp(const SearchArgs& a, bool eight, cudaStream_t s);
+cudaError_t launch_kbest_warp(const SearchArgs& a, bool eight, int num_sms, cudaStream_t s);
 // Shared memory of the K-best kernel for (n, K, P, key capacity).
 size_t kbest_smem_bytes(int n, int K, int P, bool complex_tree);
 // Workspace of the hybrid: vectors handed from form to form.
