@@ -1,16 +1,16 @@
 // Batched QR preprocessing (Sec. III-B): H = QR with a real positive diagonal
 // and ybar = Q^H y, by complex Householder reflections applied to the
-// augmented matrix [H | y], to better than FP64 accuracy on the integer
-// multiply-add pipe (fx64.cuh: this GPU's FP64 unit is thirty times slower per
-// multiply-add instruction).  Two forms: up to 32 receive antennas and enough
-// matrices to fill the GPU, several matrices per warp held in registers
-// (qr_small_kernel); otherwise one CTA per matrix in shared memory
-// (qr_cta_kernel).  The few matrices that a fixed scale per column does not
-// suit (a residual column below 2^-26 of its norm: singular or nearly so;
-// infinities, NaN and exponents near the ends of the range) are factored by
-// the FP64 forms (qr_small64, qr_one).  The complex R is written out in the real
-// interleaved form (entry r_ab -> [[Re,-Im],[Im,Re]]) that the tree search
-// uses.
+// augmented matrix [H | y] in 58-bit fixed point on the integer multiply-add pipe
+// (fx64.cuh: this GPU's FP64 unit is thirty times slower per multiply-add
+// instruction), with errors of a column's norm below those of FP64 arithmetic.
+// Two forms: up to 32 receive antennas and enough matrices to fill the GPU,
+// several matrices per warp held in registers (qr_small_kernel); otherwise one CTA
+// per matrix in shared memory (qr_cta_kernel).  The few matrices that a fixed scale
+// per column does not suit (a residual column below 2^-26 of its norm: singular or
+// nearly so; last rows far below the first; infinities, NaN and exponents near the
+// ends of the range) are factored by the FP64 forms (qr_small64, qr_one).  The
+// complex R is written out in the real interleaved form (entry r_ab ->
+// [[Re,-Im],[Im,Re]]) that the tree search uses.
 //
 // Measured (GB300; before: FP64 FMAs and FP64 MMA trailing updates): one 16x16
 // matrix 384 -> 25 us, 100,000 of them 4.02 -> 1.44 ms, 3,000 64x64 7.52 ->
@@ -559,6 +559,15 @@ __device__ __forceinline__ float fx_rel(u64 bits, int ex) {
 }
 // Columns outside these exponents are left to the FP64 form.
 __device__ __forceinline__ bool fx_in_range(int ex) { return ex < 1023 + 400 && ex > 1023 - 400; }
+// And so are channels whose last rows (M - 1 .. N - 1, from which R's last row
+// comes) are below 2^-kFxGraded of the largest: a column's one scale leaves an
+// entry 2^-k of its norm 58 - k bits, and Householder reflections in FP64 keep
+// small rows' relative accuracy where they come last (pre-whitened antennas,
+// strongest first).  Row-wise error of R, 8x8, rows graded evenly down to 2^-T, T =
+// 4 / 6 / 8 / 10 / 20: fixed 0.9e-16 / 3.3e-16 / 0.9e-15 / 3.1e-15 / 3.4e-12, FP64 0.7e-15 to
+// 1.4e-15 (2x2: equal at T = 6).  In any other order of the rows FP64 loses as many
+// digits and is behind (T = 10, shuffled: 3.1e-15 and 3.6e-14).
+constexpr int kFxGraded = 6;
 template <int L>
 __device__ __forceinline__ i64 lanes_sum(i64 v) {
 #pragma unroll
@@ -668,6 +677,19 @@ struct SrcAug {  // [R; sigma I] and [ybar; 0] of a factored R: the regularised 
     return make_longlong2(r <= j ? at[0] : 0, r < j ? at[1] : 0);
   }
 };
+
+// Whether the last rows are far below the first one (see kFxGraded).
+__device__ __forceinline__ int entry_ex(const SrcH& src, int r, int c) {
+  const longlong2 z = src(r, c);
+  return max(ex_of((u64)z.x), ex_of((u64)z.y));
+}
+// Largest exponent of the rows from M - 1 on (lane h's of G), or one close enough to high.
+__device__ __forceinline__ int last_rows_ex(const SrcH& src, int N, int high, int h, int G) {
+  int low = 0;
+  for (int e = h; e < (N - src.M + 1) * src.M && high - low >= kFxGraded; e += G)
+    low = max(low, entry_ex(src, src.M - 1 + e / src.M, e % src.M));
+  return low;
+}
 
 // A matrix left to the FP64 form is marked by -1 in its singular flag or,
 // without one (mdx_qr), in the entry of the dense R below its first diagonal
@@ -851,6 +873,20 @@ __global__ void __launch_bounds__(32) qr_reorder_small_kernel(ReorderArgs g, int
   qr_small_pair<L, SL>(g.a.n_tx, g.a.n_tx, act, src, d, reinterpret_cast<int4*>(smem_raw));
 }
 
+// Whether matrix i was left to FP64, or has to be: last rows far below the first
+// one.  By a lane, which looks closer where two entries of each row give reason to;
+// here so that qr_small_kernel keeps its registers.
+__device__ __forceinline__ bool left_to_fp64(const QrBatch& g, int i) {
+  const double *Hb, *yb;
+  const QrDst d = g.get(i, Hb, yb);
+  const SrcH src{reinterpret_cast<const longlong2*>(Hb), reinterpret_cast<const longlong2*>(yb), g.M};
+  const int c = g.M > 1 ? 1 : 0;
+  const int high = max(entry_ex(src, 0, 0), entry_ex(src, 0, c));
+  const int low = max(entry_ex(src, g.M - 1, 0), entry_ex(src, g.M - 1, c));
+  if (is_redo(d, 2 * g.M)) return true;
+  return high - low >= kFxGraded && high - last_rows_ex(src, g.N, high, 0, 1) >= kFxGraded;
+}
+
 // The matrices that the fixed-point forms left, in FP64: n_rx <= 32, 32 / L of
 // them per warp.  A warp looks through `per` matrices of the batch and factors
 // the marked ones as it finds them, a warp full at a time: a batch of nothing but
@@ -873,7 +909,7 @@ __global__ void __launch_bounds__(32) qr_redo_small_kernel(QrBatch g, int per) {
   for (;;) {
     for (; have < mats && base < end; base += 32) {
       const int i = base + lane;
-      const bool mine = i < end && is_redo(g.get(i, Hb, yb), 2 * g.M);
+      const bool mine = i < end && left_to_fp64(g, i);
       const unsigned who = __ballot_sync(0xffffffffu, mine);
       if (mine) list[have + __popc(who & ((1u << lane) - 1u))] = i;
       have += __popc(who);
@@ -897,11 +933,10 @@ __global__ void __launch_bounds__(32) qr_redo_small_kernel(QrBatch g, int per) {
 template <int LPC>
 __global__ void __launch_bounds__(256) qr_redo_kernel(QrBatch g) {
   __shared__ unsigned marks[8];
-  const int n = 2 * g.M;
   const double *Hb, *yb;
   for (int base = blockIdx.x; base < g.count; base += gridDim.x * 256) {
     const int i = base + threadIdx.x * gridDim.x;
-    const unsigned who = __ballot_sync(0xffffffffu, i < g.count && is_redo(g.get(i, Hb, yb), n));
+    const unsigned who = __ballot_sync(0xffffffffu, i < g.count && left_to_fp64(g, i));
     if ((threadIdx.x & 31) == 0) marks[threadIdx.x >> 5] = who;
     __syncthreads();
     for (int w = 0; w < 8; ++w)
@@ -1000,9 +1035,10 @@ struct QcApply {  // one reflector, by the piece of k
 };
 
 // Factorises the matrix with the calling CTA; false if it needs the FP64 form
-// (the outputs are then unfinished).
+// (the outputs are then unfinished).  rows: for last rows far below the first as
+// well (warp 0 looks when it is done; the last columns are with other warps).
 template <int L, int SL, typename Src>
-__device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
+__device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out, bool rows) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kCols = 32 / L;  // columns of a group
   QrCtaLayout lay;
@@ -1123,6 +1159,14 @@ __device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out) {
       if (c < M && h == 0) put_r(out, n, c, c, fx_to_bits((i64)sigma, e + sexp - 4), 0);
     }
   }
+  if constexpr (std::is_same<Src, SrcH>::value) {
+    if (rows && warp == 0) {
+      const int c = lane % M, high = __reduce_max_sync(0xffffffffu, entry_ex(src, 0, c));
+      if (high - __reduce_max_sync(0xffffffffu, entry_ex(src, M - 1, c)) >= kFxGraded &&
+          high - __reduce_max_sync(0xffffffffu, last_rows_ex(src, N, high, lane, 32)) >= kFxGraded)
+        *flag = 1;
+    }
+  }
   __syncthreads();
   // (the barriers end here: the FP64 form takes this memory for other things)
   for (int k = tid; k < M; k += blockDim.x)
@@ -1139,7 +1183,7 @@ __global__ void __launch_bounds__(T, B) qr_cta_kernel(QrBatch g, int here) {
   const double *Hb, *yb;
   const QrDst d = g.get(blockIdx.x, Hb, yb);
   const SrcH src{reinterpret_cast<const longlong2*>(Hb), reinterpret_cast<const longlong2*>(yb), g.M};
-  const bool ok = qr_cta_one<L, SL>(g.N, g.M, src, d);
+  const bool ok = qr_cta_one<L, SL>(g.N, g.M, src, d, here);
   __syncthreads();  // the zeroed triangle, before the mark in it; the shared memory, before the FP64 form
   if (!ok && here)
     qr_small64_one(g.N, g.M, Hb, yb, d);
@@ -1152,7 +1196,7 @@ __global__ void __launch_bounds__(288, 2) qr_reorder_cta_kernel(ReorderArgs g, i
   if (count > few || (int)blockIdx.x >= count) return;
   SrcR src;
   const QrDst d = reorder_at(g, blockIdx.x, src);
-  if (!qr_cta_one<L, SL>(g.a.n_tx, g.a.n_tx, src, d)) {
+  if (!qr_cta_one<L, SL>(g.a.n_tx, g.a.n_tx, src, d, false)) {
     __syncthreads();
     if (threadIdx.x == 0) *d.sorted = 0;
     src.restore(d, threadIdx.x, blockDim.x);
@@ -1185,7 +1229,7 @@ template <int L, int SL>
 __global__ void __launch_bounds__(288, 2) qr_aug_cta_kernel(AugArgs g) {
   SrcAug src;
   const QrDst d = aug_at(g, blockIdx.x, src);
-  const bool ok = qr_cta_one<L, SL>(2 * g.a.n_tx, g.a.n_tx, src, d);
+  const bool ok = qr_cta_one<L, SL>(2 * g.a.n_tx, g.a.n_tx, src, d, false);
   if (threadIdx.x == 0) *d.pk_bad = ok ? 0 : 1;
 }
 
