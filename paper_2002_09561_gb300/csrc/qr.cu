@@ -874,8 +874,9 @@ __global__ void __launch_bounds__(32) qr_reorder_small_kernel(ReorderArgs g, int
 }
 
 // Whether matrix i was left to FP64, or has to be: last rows far below the first
-// one.  By a lane, which looks closer where two entries of each row give reason to;
-// here so that qr_small_kernel keeps its registers.
+// one, or a y of subnormal numbers, whose ybar is all zeros.  By a lane, which looks
+// closer where two entries of each row or the first of ybar give reason to (all of
+// them loaded at once); here so that qr_small_kernel keeps its registers.
 __device__ __forceinline__ bool left_to_fp64(const QrBatch& g, int i) {
   const double *Hb, *yb;
   const QrDst d = g.get(i, Hb, yb);
@@ -883,8 +884,14 @@ __device__ __forceinline__ bool left_to_fp64(const QrBatch& g, int i) {
   const int c = g.M > 1 ? 1 : 0;
   const int high = max(entry_ex(src, 0, 0), entry_ex(src, 0, c));
   const int low = max(entry_ex(src, g.M - 1, 0), entry_ex(src, g.M - 1, c));
-  if (is_redo(d, 2 * g.M)) return true;
-  return high - low >= kFxGraded && high - last_rows_ex(src, g.N, high, 0, 1) >= kFxGraded;
+  const double* y0 = d.yb64 ? d.yb64 : d.ybdense;  // (aligned to a double)
+  const double yr = y0[0], yi = y0[1];
+  const bool marked = is_redo(d, 2 * g.M), none = yr == 0.0 && yi == 0.0;
+  if (!marked && !none && high - low < kFxGraded) return false;
+  if (marked || high - last_rows_ex(src, g.N, high, 0, 1) >= kFxGraded) return true;
+  bool some = false;
+  for (int r = 0; none && r < 2 * g.N; ++r) some = some || yb[r] != 0.0;
+  return some;
 }
 
 // The matrices that the fixed-point forms left, in FP64: n_rx <= 32, 32 / L of
@@ -1082,6 +1089,12 @@ __device__ bool qr_cta_one(int N, int M, const Src& src, const QrDst& out, bool 
     const bool fine = fx_in_range(ex);
     const int e = fine ? fx_scale(ex, ss) : 0;
     if (ex != 0 && !fine) *flag = 1;
+    if (c == M && ex == 0) {  // y of subnormal numbers
+      i64 bits = 0;
+#pragma unroll
+      for (int q = 0; q < SL; ++q) bits |= ar[q] << 1 | ai[q] << 1;
+      if (bits) *flag = 1;
+    }
 #pragma unroll
     for (int q = 0; q < SL; ++q) {
       ar[q] = fine ? fx_from((u64)ar[q], e) : 0;

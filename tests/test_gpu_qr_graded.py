@@ -1,6 +1,6 @@
 """The QR on receive antennas of very different scale, strongest first (pre-whitened or attenuated rows):
 row-wise accuracy of R and ybar, which FP64 Householder reflections keep for such an order of the rows and a
-fixed scale per column does not.
+fixed scale per column does not; and received vectors of subnormal numbers.
 
 Bound: every row of R and ybar goes through at most M reflectors, each with a relative error of a few u of
 that row (u = 2^-53), so the root mean square of the rows' relative errors is held to 8 M u, the constant of
@@ -68,3 +68,16 @@ def test_zero_rows_and_other_orders_are_ordinary(N, M):
     if N > M:
         H[5, M:] = 0.0
     _check(H, y, *_run(H, y))
+
+
+@pytest.mark.parametrize("N,M,B", [(4, 4, 2), (16, 16, 1300), (40, 40, 2)])
+def test_subnormal_received_vectors(N, M, B):
+    w = wl.generate(8900 + N, B, N, M, 16, 10.0)
+    H, y = w["H"], w["y"].copy()
+    _, plain = _run(H, y)
+    y[:2] *= 2.0 ** -1040
+    _, yb = _run(H, y)
+    # numbers of 2^-1040 hold 34 bits; N rounded products of them
+    np.testing.assert_allclose(yb[:2] * 2.0 ** 1000, plain[:2] * 2.0 ** -40, rtol=0,
+                               atol=2.0 ** -40 * np.abs(plain[:2]).max() * N * 2.0 ** -32)
+    assert np.array_equal(yb[2:], plain[2:])
