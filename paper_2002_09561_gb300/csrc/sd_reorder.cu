@@ -36,6 +36,7 @@ namespace {
 
 constexpr float kReorderNodes = 40.0f;
 constexpr float kNoiseRadius = 1.25f;
+constexpr float kMostNodes = 100.0f;  // log2: P^level passes FP32's range from 22 antennas of 64-QAM on
 
 // log2 of the volume of the unit ball in k dimensions
 __device__ __forceinline__ float log2_ball(int k) {
@@ -72,13 +73,15 @@ __global__ void __launch_bounds__(128) reorder_select_kernel(ReorderArgs g) {
   float nodes = 0.0f;
   if (mine) {
     const int k = 2 * (M - c);  // both rows of antenna c, then its first alone
-    nodes = exp2f(fminf(lp * (float)k, log2_ball(k) + lr * (float)k - below)) +
-            exp2f(fminf(lp * (float)(k - 1), log2_ball(k - 1) + lr * (float)(k - 1) - (below - ld)));
+    const float b1 = fminf(lp * (float)k, log2_ball(k) + lr * (float)k - below);
+    const float b0 = fminf(lp * (float)(k - 1), log2_ball(k - 1) + lr * (float)(k - 1) - (below - ld));
+    nodes = exp2f(fminf(b1, kMostNodes)) + exp2f(fminf(b0, kMostNodes));
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) nodes += __shfl_xor_sync(gmask, nodes, o, G);
-  // (NaN or a zero diagonal: left in natural order)
-  const bool pick = act && nodes > kReorderNodes && !(a.singular && a.singular[v]) && nodes < INFINITY;
+  // (a zero, infinite or NaN diagonal: left in natural order)
+  const bool sound = __all_sync(gmask, !mine || (rcc > 0.0f && rcc < INFINITY));
+  const bool pick = act && sound && nodes > kReorderNodes && !(a.singular && a.singular[v]);
   if (act && c == 0) g.sorted[v] = pick ? 1 : 0;
   // the search's order: the vectors chosen from the front, the others from the back
   const unsigned first = __ballot_sync(0xffffffffu, c == 0 && pick);
