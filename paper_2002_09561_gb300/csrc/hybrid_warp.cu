@@ -127,8 +127,9 @@ __device__ __forceinline__ void unpack_path(const uint32_t* x, int KS, int s, in
   }
 }
 // A slot for a leaf at distance p, the list locked; -1: not among the best
-// kCandMax (the list not locked).  The holder copies one path, so the wait is
-// short; it is bounded all the same (then the vector is left: budget_hit).
+// kCandMax (the list not locked).  Two equally near for the last place are noted
+// (budget_hit: the least such distance).  The holder copies one path, so the wait is
+// short; it is bounded all the same (then the vector is left: budget_hit -1).
 __device__ int take_slot(SdVec* st, float p) {
   bool got = false;
   for (int it = 0; it < (1 << 16) && !got; ++it) {
@@ -145,12 +146,19 @@ __device__ int take_slot(SdVec* st, float p) {
     *(volatile int*)&st->ncand = slot + 1;
   } else {
     float worst = -1.0f;
+    int equal = 0;
     for (int t = 0; t < kCandMax; ++t) {
       const float c = ((volatile float*)st->cand_ped)[t];
+      equal = c > worst ? 1 : equal + (c == worst ? 1 : 0);
       if (c > worst) {
         worst = c;
         slot = t;
       }
+    }
+    if (p == worst || (p < worst && equal > 1)) {
+      // (an arrival at the last one's distance, or one of several such leaves goes)
+      const int hit = *(volatile int*)&st->budget_hit, tied = __float_as_int(worst);
+      if (hit == 0 || (hit > 0 && tied < hit)) atomicCAS(&st->budget_hit, hit, tied);
     }
     if (!(p < worst)) {
       __threadfence();
@@ -284,7 +292,7 @@ __device__ void leave(const HybridWork& w, int v) {
 
 // The leaves within lim join the candidates, nc of them, of which the
 // kCandMax nearest are kept; tie: the least distance at which two were equally
-// near for the last place.
+// near for the last place (an arrival, or two kept of which one had to go).
 template <int SL>
 __device__ void add_leaves(const Survivors<SL>& w, int S, float lim, const SelectWs& ws, int n, SdVec* st, uint8_t* cx,
                            int cs, int& nc, float& tie, int lane) {
@@ -300,9 +308,11 @@ __device__ void add_leaves(const Survivors<SL>& w, int S, float lim, const Selec
         __syncwarp();
         const unsigned c = lane < kCandMax ? __float_as_uint(st->cand_ped[lane]) : 0u;
         const unsigned worst = __reduce_max_sync(0xffffffffu, c);
-        if (p == __uint_as_float(worst)) tie = fminf(tie, p);
+        const unsigned last = __ballot_sync(0xffffffffu, c == worst && lane < kCandMax);
+        if (p == __uint_as_float(worst) || (p < __uint_as_float(worst) && (last & (last - 1))))
+          tie = fminf(tie, __uint_as_float(worst));
         if (!(p < __uint_as_float(worst))) continue;
-        slot = __ffs(__ballot_sync(0xffffffffu, c == worst && lane < kCandMax)) - 1;
+        slot = __ffs(last) - 1;
       }
       if (lane == 0) st->cand_ped[slot] = p;
       unpack_path(ws.x, ws.KS, s + 32 * t, n, cx + (size_t)slot * cs, lane);

@@ -835,6 +835,15 @@ __host__ __device__ inline void hy_layout(HyLayout& L, int n, int K, int P, int 
   L.bytes = o;
 }
 
+// Whether index path x comes before y, top row first (other warps may have written them).
+__device__ bool path_before(const uint8_t* x, const uint8_t* y, int n) {
+  for (int i = n - 1; i >= 0; --i) {
+    const uint8_t a = *(const volatile uint8_t*)(x + i), b = *(const volatile uint8_t*)(y + i);
+    if (a != b) return a < b;
+  }
+  return false;
+}
+
 // redo: only the vectors listed there (*listed of them, taken from the counter next).
 __global__ void hybrid_kernel(SearchArgs a, HyLayout L, const unsigned char* redo, size_t stride, const unsigned int* listed,
                               unsigned int* next) {
@@ -1083,14 +1092,19 @@ __global__ void hybrid_kernel(SearchArgs a, HyLayout L, const unsigned char* red
                   slot = nc;
                   misc[3] = nc + 1;
                 } else {
+                  // the last by distance, then path: which leaves stay does not
+                  // depend on the order in which the warps bring them
                   float worst = -1.0f;
                   int w = -1;
-                  for (int c2 = 0; c2 < kCandMax; ++c2)
-                    if (((volatile float*)cped)[c2] > worst) {
-                      worst = ((volatile float*)cped)[c2];
+                  for (int c2 = 0; c2 < kCandMax; ++c2) {
+                    const float p2 = ((volatile float*)cped)[c2];
+                    if (p2 > worst || (p2 == worst && path_before(cx + (size_t)w * L.pp, cx + (size_t)c2 * L.pp, n))) {
+                      worst = p2;
                       w = c2;
                     }
-                  if (ps < worst) slot = w;
+                  }
+                  if (ps < worst || (ps == worst && path_before(xcur + (size_t)sidx * L.pp, cx + (size_t)w * L.pp, n)))
+                    slot = w;
                 }
                 if (slot < 0) {
                   __threadfence_block();
