@@ -424,7 +424,7 @@ mdx_status run_detect(int algo, mdx_ctx* c, const mdx_params* p, int batch, cons
       ReorderArgs r{a, c->sd_sorted, c->sd_sorted + batch, c->sd_sorted + (size_t)batch * (1 + M),
                     c->sd_order, c->counter + 1};
       e = launch_reorder_select(r, s);
-      if (e == cudaSuccess) e = launch_qr_reorder(r, s);
+      if (e == cudaSuccess) e = launch_qr_reorder(r, c->num_sms, s);
       if (e != cudaSuccess) return cuda_fail(c, e, "antenna order");
       a.sorted = r.sorted;
       a.place = r.place;

@@ -290,7 +290,7 @@ cudaError_t launch_linear(const AugArgs& g, bool mmse, int num_sms, cudaStream_t
   if (a.batch <= 0) return cudaSuccess;
   const int* only = nullptr;
   if (a.n_tx <= kAugMaxTx) {
-    cudaError_t e = mmse ? launch_qr_augmented(g, s) : cudaSuccess;
+    cudaError_t e = mmse ? launch_qr_augmented(g, num_sms, s) : cudaSuccess;
     if (e != cudaSuccess) return e;
     e = a.n_tx <= 8    ? launch_linear_group<1>(g, mmse, s)
         : a.n_tx <= 16 ? launch_linear_group<2>(g, mmse, s)

@@ -84,7 +84,7 @@ struct ReorderArgs {
 };
 cudaError_t launch_reorder_select(const ReorderArgs& r, cudaStream_t s);
 // QR of the chosen vectors' R with permuted columns (qr.cu).
-cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s);
+cudaError_t launch_qr_reorder(const ReorderArgs& r, int num_sms, cudaStream_t s);
 
 // MMSE's augmented systems [R; sigma I] x = [ybar; 0], factored into the space
 // of the FP32 R (the triangle as complex FP64 numbers: above the diagonal, then
@@ -102,7 +102,7 @@ struct AugArgs {
   __host__ __device__ double* diag(int v) const { return R(v) + (size_t)a.n_tx * (a.n_tx - 1); }
   __host__ __device__ double* y(int v) const { return reinterpret_cast<double*>(space + (size_t)v * stride); }
 };
-cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s);
+cudaError_t launch_qr_augmented(const AugArgs& g, int num_sms, cudaStream_t s);
 
 cudaError_t launch_qr(int batch, int n_rx, int n_tx, const double* H, const double* y, QrOut out, int num_sms,
                       cudaStream_t s);

@@ -1315,12 +1315,14 @@ cudaError_t launch_qc(const QrBatch& g, int most, cudaStream_t s) {
 //   24x24:  1,216: 131 / - / 314 / 234, 4,864: 515 / - / 336 / 301,
 //          38,912: 3,883 / - / 2,410 / 2,538
 //   32x32:  2,432: 445 / - / 567 / 377, 9,728: 1,667 / - / 1,655 / 1,213
-int qr_form(int count, int n_rx) {
-  if (n_rx > 32 || count <= (n_rx <= 16 ? 1216 : 1824)) return 0;
+// (The lines in matrices per SM, of which this GPU has 152.)
+int few_matrices(int n_rx, int num_sms) { return (n_rx <= 16 ? 8 : 12) * num_sms; }
+int qr_form(int count, int n_rx, int num_sms) {
+  if (n_rx > 32 || count <= few_matrices(n_rx, num_sms)) return 0;
   if (n_rx <= 4) return 2;
-  if (n_rx <= 8) return count <= 16384 ? 4 : 2;
-  if (n_rx <= 12) return count <= 9728 ? 8 : 4;
-  if (n_rx > 16 && n_rx <= 24) return count <= 4864 ? 8 : 4;
+  if (n_rx <= 8) return count <= 108 * num_sms ? 4 : 2;
+  if (n_rx <= 12) return count <= 64 * num_sms ? 8 : 4;
+  if (n_rx > 16 && n_rx <= 24) return count <= 32 * num_sms ? 8 : 4;
   return 8;
 }
 
@@ -1343,27 +1345,24 @@ cudaError_t launch_rs(const ReorderArgs& r, int few, cudaStream_t s) {
 cudaError_t launch(const QrBatch& g, cudaStream_t s) {
   if (g.count <= 0) return cudaSuccess;
   const int N = g.N;
-  switch (qr_form(g.count, N)) {
+  switch (qr_form(g.count, N, g.num_sms)) {
     case 0: {
       // Few matrices: more warps each, for the chain; many: CTAs of fewer warps.
-      const int w = g.count <= 152 ? 9 : g.count <= 1216 ? 5 : 3;
+      const int w = g.count <= g.num_sms ? 9 : g.count <= 8 * g.num_sms ? 5 : 3;
       if (N <= 16) return launch_qc<16, 1, 288, 2>(g, std::min(w, 5), s);
       if (N <= 32) return launch_qc<16, 2, 288, 2>(g, w, s);
-      if (N <= 48) return launch_qc<16, 3, 256, 3>(g, g.count <= 152 ? 8 : 4, s);
+      if (N <= 48) return launch_qc<16, 3, 256, 3>(g, g.count <= g.num_sms ? 8 : 4, s);
       if (N <= 64) return launch_qc<32, 2, 256, 3>(g, 8, s);
       if (N <= 96) return launch_qc<32, 3, 256, 3>(g, 8, s);
       return launch_qc<32, 4, 384, 2>(g, 12, s);
     }
     case 2:
       if (N <= 4) return launch_qs<2, 2>(g, s);
-      if (N <= 8) return launch_qs<2, 4>(g, s);
-      if (N <= 12) return launch_qs<2, 6>(g, s);
-      return launch_qs<2, 8>(g, s);
+      return launch_qs<2, 4>(g, s);
     case 4:
       if (N <= 8) return launch_qs<4, 2>(g, s);
-      if (N <= 16) return launch_qs<4, 4>(g, s);
-      if (N <= 24) return launch_qs<4, 6>(g, s);
-      return launch_qs<4, 8>(g, s);
+      if (N <= 12) return launch_qs<4, 4>(g, s);
+      return launch_qs<4, 6>(g, s);
     default:
       if (N <= 16) return launch_qs<8, 2>(g, s);
       return launch_qs<8, 4>(g, s);
@@ -1375,8 +1374,8 @@ cudaError_t launch(const QrBatch& g, cudaStream_t s) {
 // The number of vectors chosen is on the device: the CTA form's grid is for
 // up to `few` of them (as in qr_form), the other's for the whole batch, and
 // the one that does not apply returns at once.
-cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s) {
-  const int M = r.a.n_tx, few = M <= 16 ? 1216 : 1824;
+cudaError_t launch_qr_reorder(const ReorderArgs& r, int num_sms, cudaStream_t s) {
+  const int M = r.a.n_tx, few = few_matrices(M, num_sms);
   const size_t sm = qr_cta_smem(M, M);
   const int grid = std::min(r.a.batch, few), threads = qc_threads(8, M, 9);
   if (M <= 16) {
@@ -1392,9 +1391,9 @@ cudaError_t launch_qr_reorder(const ReorderArgs& r, cudaStream_t s) {
   return launch_rs<8, 4>(r, few, s);
 }
 
-cudaError_t launch_qr_augmented(const AugArgs& g, cudaStream_t s) {
+cudaError_t launch_qr_augmented(const AugArgs& g, int num_sms, cudaStream_t s) {
   const int M = g.a.n_tx;
-  switch (qr_form(g.a.batch, 2 * M)) {
+  switch (qr_form(g.a.batch, 2 * M, num_sms)) {
     case 0: {
       const size_t sm = qr_cta_smem(2 * M, M);
       if (M <= 8) {
