@@ -14,10 +14,14 @@
 // A number x in [-2, 2] is the integer x 2^58 = h 2^29 + l with -2^28 <= l <
 // 2^28 (|h| <= 2^30; signed low limbs, so that the dropped products average to
 // zero and 0 stays exactly 0).  A sum of products is kept as two 64-bit accumulators,
-// hh = sum h h' (units) and md = sum h l' + l h' (units 2^-29): for vectors u
-// of norm sqrt(2) and a of norm 1 with m real entries, |md| is below
-// sqrt(m) 2^59 (Cauchy-Schwarz on the high limbs), so up to 256 entries per
-// accumulator cannot overflow.
+// hh = sum h h' (units) and md = sum h l' + l h' (units 2^-29), by lane: a lane
+// sums at most kFxEntries complex entries before it shifts md to units, and only
+// units are added across lanes.  Bounds for u of norm sqrt(2) and a of norm 1
+// (Cauchy-Schwarz, m entries): md of plain products is below 1.8 sqrt(m) 2^58, that
+// of three-product complex ones (FxDot in qr.cu: sums of limbs, up to twice as large)
+// 1.8 sqrt(m) 2^59, and their sum, as the imaginary part needs it, 3.6 sqrt(m) 2^59 <
+// 2^63 up to m = 19.  Norms: md below sqrt(2 m) 2^57, ll (a square of the low limbs'
+// each) m 2^57, added over up to 128 entries after the shift by 3: 2^61.
 #pragma once
 
 #include <stdint.h>
@@ -31,35 +35,32 @@ typedef unsigned long long u64;
 
 constexpr int kFxBits = 58;   // fraction bits
 constexpr int kFxLimb = 29;   // bits of the low limb
+constexpr int kFxEntries = 8;   // complex entries a lane sums at most
 constexpr i64 kFxHalf = 1ll << (kFxLimb - 1);  // rounds md to the nearest unit
 
-__host__ __device__ __forceinline__ int fx_lo(i64 a) { return (int)((unsigned)a << (32 - kFxLimb)) >> (32 - kFxLimb); }
-__host__ __device__ __forceinline__ int fx_hi(i64 a) { return (int)(a >> kFxLimb) + (int)((unsigned)fx_lo(a) >> 31); }
+__device__ __forceinline__ int fx_lo(i64 a) { return (int)((unsigned)a << (32 - kFxLimb)) >> (32 - kFxLimb); }
+__device__ __forceinline__ int fx_hi(i64 a) { return (int)(a >> kFxLimb) + (int)((unsigned)fx_lo(a) >> 31); }
 // a b as one wide multiply.  (Written out: where the
 // compiler can tell a limb's sign it may widen it with zeros and multiply in 64
 // bits, three instructions for one.)
-__host__ __device__ __forceinline__ i64 wide(int a, int b) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ i64 wide(int a, int b) {
   i64 r;
   asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
   return r;
-#else
-  return (i64)a * (i64)b;
-#endif
 }
 // c + a b: the multiply above and a plain addition fuse into one wide
 // multiply-add (mad.wide itself becomes a multiply and an addition: 2 x the
 // instructions, measured).
-__host__ __device__ __forceinline__ i64 wide_add(int a, int b, i64 c) { return c + wide(a, b); }
+__device__ __forceinline__ i64 wide_add(int a, int b, i64 c) { return c + wide(a, b); }
 
 // A complex number as limbs: {re high, re low, im high, im low}.
-__host__ __device__ __forceinline__ int4 fx_split(i64 re, i64 im) {
+__device__ __forceinline__ int4 fx_split(i64 re, i64 im) {
   return make_int4(fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im));
 }
 
 // x 2^(58 - e) of a double |x| <= 2^e (e a power-of-two exponent), rounded to
 // nearest (ties away); zero, subnormals and anything below half a unit give 0.
-__host__ __device__ __forceinline__ i64 fx_from(u64 bits, int e) {
+__device__ __forceinline__ i64 fx_from(u64 bits, int e) {
   const int ex = (int)((bits >> 52) & 0x7ff);
   const u64 m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
   const int s = ex - 1075 + kFxBits - e;  // m 2^s
@@ -74,15 +75,11 @@ __host__ __device__ __forceinline__ i64 fx_from(u64 bits, int e) {
 
 // The double a 2^(e - 58), rounded to nearest even (the exponent must stay in
 // the normal range).
-__host__ __device__ __forceinline__ u64 fx_to_bits(i64 a, int e) {
+__device__ __forceinline__ u64 fx_to_bits(i64 a, int e) {
   if (a == 0) return 0;
   const u64 sign = (u64)a & 0x8000000000000000ull;
   u64 m = a < 0 ? (u64)(-a) : (u64)a;
-#ifdef __CUDA_ARCH__
   const int lz = __clzll((i64)m);
-#else
-  const int lz = __builtin_clzll(m);
-#endif
   m <<= lz;
   const unsigned rem = (unsigned)m & 0x7ffu;
   u64 f = m >> 11;
@@ -92,7 +89,7 @@ __host__ __device__ __forceinline__ u64 fx_to_bits(i64 a, int e) {
 
 // The float nearest the double `bits` (round to nearest even, as the
 // conversion instruction), for zero or magnitudes in float's normal range.
-__host__ __device__ __forceinline__ unsigned f32_bits_of(u64 bits) {
+__device__ __forceinline__ unsigned f32_bits_of(u64 bits) {
   if (bits == 0) return 0;
   const u64 m = bits & 0x7fffffffffffffffull;
   const unsigned rem = (unsigned)m & 0x1fffffffu;
@@ -101,31 +98,19 @@ __host__ __device__ __forceinline__ unsigned f32_bits_of(u64 bits) {
   return f | ((unsigned)(bits >> 32) & 0x80000000u);
 }
 
-__host__ __device__ __forceinline__ u64 fx_mulhi(u64 a, u64 b) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ u64 fx_mulhi(u64 a, u64 b) {
   return __umul64hi(a, b);
-#else
-  return (u64)(((unsigned __int128)a * b) >> 64);
-#endif
 }
-__host__ __device__ __forceinline__ int fx_clz(u64 x) {
-#ifdef __CUDA_ARCH__
+__device__ __forceinline__ int fx_clz(u64 x) {
   return __clzll((i64)x);
-#else
-  return x ? __builtin_clzll(x) : 64;
-#endif
 }
 
 // 2^59 / sqrt(X 2^-60) for X in [2^58, 2^60]: the single-precision estimate y
 // (24 bits, exact square) refined by 1 / sqrt(1 - e) = 1 + e/2 + 3 e^2/8,
 // e = 1 - x y^2 (|e| < 2^-20, so the next term is below 2^-61).
-__host__ __device__ __forceinline__ u64 fx_rsqrt(u64 X) {
+__device__ __forceinline__ u64 fx_rsqrt(u64 X) {
   const float xf = (float)(unsigned)(X >> 32) * 3.7252903e-9f;  // 2^-28
-#ifdef __CUDA_ARCH__
   const float yf = rsqrtf(xf);
-#else
-  const float yf = 1.0f / sqrtf(xf);
-#endif
   const unsigned Y = (unsigned)(yf * 8388608.0f);  // y 2^23
   const i64 e = (1ll << 61) - (i64)fx_mulhi(X << 4, ((u64)Y * Y) << 15);  // e 2^61
   const int es = (int)(e >> 21);
@@ -136,14 +121,14 @@ __host__ __device__ __forceinline__ u64 fx_rsqrt(u64 X) {
 // x y / 2^58 of |x|, |y| < 2^60, in units 2^-(58 + X): the full product's high
 // part with X more bits.
 template <int X>
-__host__ __device__ __forceinline__ i64 fx_mul(i64 x, i64 y) {
+__device__ __forceinline__ i64 fx_mul(i64 x, i64 y) {
   const int xh = fx_hi(x), xl = fx_lo(x), yh = fx_hi(y), yl = fx_lo(y);
   const i64 md = wide_add(xh, yl, wide_add(xl, yh, wide(xl, yl) >> kFxLimb));
   return (wide(xh, yh) << X) + ((md + (1ll << (kFxLimb - 1 - X))) >> (kFxLimb - X));
 }
 
 // S 2^-116 = x 4^h with x in [1/4, 1): returns x 2^60 and h (S > 0).
-__host__ __device__ __forceinline__ u64 fx_norm4(unsigned __int128 S, int& h) {
+__device__ __forceinline__ u64 fx_norm4(unsigned __int128 S, int& h) {
   const u64 hi = (u64)(S >> 64), lo = (u64)S;
   const int p = hi ? 127 - fx_clz(hi) : 63 - fx_clz(lo);  // top bit
   h = (p - 114) >> 1;                                     // ceil((p - 115) / 2)
@@ -160,13 +145,13 @@ struct FxReflector {
   i64 g;       // units 2^-58, at most 2
   int s;       // sigma in [2^(s-1), 2^s)
   u64 sigma;   // sigma 2^(62 - s)
-  __host__ __device__ __forceinline__ i64 scale(i64 x) const {  // u_r of x_r
+  __device__ __forceinline__ i64 scale(i64 x) const {  // u_r of x_r
     return (fx_mul<4>(s > 0 ? x >> s : x << -s, g) + 8) >> 4;
   }
 };
 // hh = sum xh^2, md = sum xh xl, ll = sum xl^2 over the entries' limbs (ll / 8,
 // so that the sum over 128 rows fits); x0 the first entry.  False (and nothing computed) if sigma < 2^-26.
-__host__ __device__ __forceinline__ bool fx_reflector(i64 hh, i64 md, u64 ll, i64 x0r, i64 x0i, FxReflector& f) {
+__device__ __forceinline__ bool fx_reflector(i64 hh, i64 md, u64 ll, i64 x0r, i64 x0i, FxReflector& f) {
   typedef unsigned __int128 u128;
   const u128 S = ((u128)(u64)hh << 58) + ((u128)(__int128)md << 30) + ((u128)ll << 3);
   if ((i64)(S >> 64) <= 0) return false;

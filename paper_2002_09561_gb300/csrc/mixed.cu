@@ -1,8 +1,9 @@
-// Uneven batches: one persistent search kernel over requests that differ in
+// Uneven batches: two persistent search kernels, side by side (walk_kernel for
+// exact SDs, mixed_kernel for the others), over requests that differ in
 // antennas, modulation, detector and K (the batching layer around the
 // paper's detectors; the paper runs one system at a time).
 //
-// Every warp of the grid takes requests from a global counter, in the order
+// Every warp of a grid takes requests from a global counter, in the order
 // the host chose (heaviest classes first), and searches each one alone:
 //   exact SD   Algorithm 1 with Schnorr-Euchner child order (Sec. IV-A) and
 //              incremental partial distances (Eq. inc), one warp walking the
@@ -541,7 +542,7 @@ __device__ void sd_walk(const MixedArgs& g, const MixedReq& q, int r, const floa
 // found by a warp arg-min; a level is exhausted when that child leaves the
 // sphere.  A descent updates the residuals of the rows below by both fixed
 // rows; the rest (candidates, radius shrink and doubling, budget, FP64
-// re-scoring) is as in sd_request.
+// re-scoring) is as in sd_walk.
 template <int ROWS>
 __device__ void sdc_request(const MixedArgs& g, const MixedReq& q, int r, const float* Rc, const float* yb,
                             unsigned char* st, float E, int lane) {

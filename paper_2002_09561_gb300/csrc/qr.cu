@@ -594,6 +594,7 @@ __host__ __device__ inline size_t qs_smem(int N, int M, int lanes) {
 
 template <int L, int SL, int Q0>
 __device__ __forceinline__ void qs_apply(i64 (&ar)[SL], i64 (&ai)[SL], const int4* u, int k, int N, int h) {
+  static_assert(SL <= kFxEntries, "the accumulators' range");
   constexpr int stride = 32 / L;
   int4 uu[SL];
   FxDot d;
@@ -1012,6 +1013,7 @@ constexpr int qc_step = L < 16 ? 16 / L : 1;
 // lanes' columns; masked: also rows above k among the piece's first slots.
 template <int L, int SL, int Q0>
 __device__ __forceinline__ void qc_apply(i64 (&ar)[SL], i64 (&ai)[SL], const int4* u, int k, int N, int h, bool act) {
+  static_assert(SL <= kFxEntries, "the accumulators' range");
   FxDot d;
 #pragma unroll
   for (int q = Q0; q < SL; ++q) {
