@@ -4,7 +4,7 @@
 // Most vectors need one K-best run: the best prefix's leaf shrinks the radius
 // below every other prefix.  A run is a serial chain of levels, so what counts
 // is how many run at once: select_run (select_run.cuh) needs no R in shared
-// memory, so some 22 vectors share an SM where the sorting form (kbest.cu), which
+// memory, so 28 vectors share an SM where the sorting form (kbest.cu), which
 // stages R and sorts with CTA barriers, held one 100x100 vector on an SM of its
 // own.  The master keeps no sorted list either: a pass over the P^d prefixes
 // finds the best one inside the sphere after the last (128 evaluations a lane
@@ -623,9 +623,13 @@ size_t hybrid_redo_offset() { return offsetof(SdVec, r2_start); }
 
 // Runs for K <= 64, prefixes of at most four rows and no node budget (the
 // budget counts the prefixes in the sorting form's order); else
-// cudaErrorNotSupported, nothing launched.
+// cudaErrorNotSupported, nothing launched.  Nor for statistics of a few vectors
+// with the network's radius, which leaves one sphere in ten empty: their passes are
+// counted by the sorting form, behind the runs here (20 vectors 100x100 64-QAM
+// K = 32: 4.2 ms so, 3.0 by that form alone; 200: 11.2).
 cudaError_t launch_hybrid_warp(const SearchArgs& a, const HybridWork& w, int num_sms, cudaStream_t s) {
   if (a.K > 64 || a.depth > 4 || a.budget > 0) return cudaErrorNotSupported;
+  if (a.stats && a.radius_mode == RADIUS_PER_VECTOR && a.batch <= num_sms) return cudaErrorNotSupported;
   return a.K <= 32 ? launch_hw_p<1>(a, w, num_sms, s) : launch_hw_p<2>(a, w, num_sms, s);
 }
 
