@@ -2,7 +2,8 @@
 """Throughput benchmark of the batched MIMO tree-search detectors.
 
 One step = one pass of the detection path over one batch of synthetic
-received vectors resident in device memory: FP64 QR, (for the learned
+received vectors resident in device memory: the QR (58-bit fixed point,
+FP64 in and out), (for the learned
 workloads) the network's features and tensor-core forward pass giving each
 vector's initial radius, the tree search (FP32 partial distances), FP64
 re-scoring of the final leaves, and the Gray-coded bit/symbol error count of
@@ -90,15 +91,15 @@ KERNEL_SOURCES = {
     "100x100-64qam-hybrid32-learned": ("hybrid_warp.cu", "select_run.cuh", "warp_kbest.cuh", "mdx_internal.cuh"),
 }
 TRAFFIC_PER_VECTOR = {
-    "16x16-16qam-sd-learned": ((225.393408e6 + 5.746176e6) / 30000,
+    "16x16-16qam-sd-learned": ((225.374464e6 + 5.276928e6) / 30000,
                                "ncu capture of sd_group_kernel, 30,000 vectors of the learned 16x16 sweep "
                                "(profiles/search_and_qr_kernels.md), scaled by vectors",
-                               "155b845d7303518d"),
-    "100x100-64qam-hybrid32-learned": ((369.485824e6 + 8.572928e6 + 30.755840e6 + 0.067840e6 + 216.549120e6
-                                        + 6.335232e6) / 2000,
+                               "cba0117a9c3272b3"),
+    "100x100-64qam-hybrid32-learned": ((369.188096e6 + 7.888128e6 + 30.787072e6 + 0.073728e6 + 216.514560e6
+                                        + 6.273280e6) / 2000,
                                        "ncu capture of the hybrid's three search kernels, 2,000 vectors of the learned "
                                        "100x100 workload (profiles/search_and_qr_kernels.md), scaled by vectors",
-                                       "c063e981d9e0b5ff"),
+                                       "19a14dec70fdfaed"),
 }
 
 
@@ -122,11 +123,11 @@ def code_hash(files, csrc=None):
 # tied to the sources in the same way: with the live node rate this gives the
 # kernel's instruction-issue rate, the resource that bounds it.
 INSTRUCTIONS_PER_NODE = {
-    "16x16-16qam-sd-learned": (1.2359628411e10 / 300102995,
+    "16x16-16qam-sd-learned": (1.2145479546e10 / 295521813,
                                "ncu capture of sd_group_kernel, 30,000 vectors of the learned 16x16 sweep: "
                                "smsp__inst_executed.sum over the launch's branched nodes "
                                "(profiles/search_and_qr_kernels.md)",
-                               "155b845d7303518d"),
+                               "cba0117a9c3272b3"),
 }
 
 
@@ -577,7 +578,7 @@ def main():
     # the timed calls ask for the points, metrics and status; the visited-node
     # statistics, which fix the search to the natural antenna order, come from an
     # arm of their own, with the search's time for them (roofline)
-    ms, _, errs, sampler = arm.time(params, out[:3] + (None,), args.steps, args.warmup)
+    ms, (_, timed_search, timed_calls), errs, sampler = arm.time(params, out[:3] + (None,), args.steps, args.warmup)
     value = B * world * args.steps / (ms / 1e3)
     timed = [o.clone() for o in out[:3]]
     ssteps = max(1, min(args.steps, 5))
@@ -629,7 +630,12 @@ def main():
     # kernel's own count, sum over branched nodes at row i of 2(n-1-i) + 4P
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     roof = search_roofline(args.workload, algo, stats, search_ms, calls, qr_ms, sms, probe, B)
-    # the FP64 QR (timed in the arm without the network, whose QR interval is
+    if algo == "sd":
+        # two searches: the timed calls' takes the antennas in sorted order where that pays
+        # (with what chooses and factors it), the one that counts nodes in natural order
+        roof["of"] = "the search of the calls with statistics (natural antenna order)"
+        roof["search_ms_per_timed_call"] = timed_search / max(timed_calls, 1)
+    # the QR (timed in the arm without the network, whose QR interval is
     # the QR kernel and a 4-byte counter reset)
     qprof = plain_qr if plain_qr is not None else ((qr_ms, search_ms, calls) if not learned else None)
     qr_roof = qr_roofline(n, n, B, qprof, sms, probe) if qprof else None
@@ -677,7 +683,7 @@ def main():
             cfg["model"] = {k: model_meta.get(k) for k in ("traces", "snr_db", "epochs", "seed")} if model_meta else None
         line = {"metric": METRIC, "value": value, "unit": "vectors/s", "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
-                "scaling": "weak", "vs_baseline": None, "dtype": "f32 search, f64 QR and re-scoring",
+                "scaling": "weak", "vs_baseline": None, "dtype": "f32 search, 58-bit fixed-point QR, f64 re-scoring",
                 "data": "synthetic (seeded Rayleigh channels, uniform QAM symbols, AWGN)",
                 "config": cfg, "with_statistics": with_stats, "roofline": roof, "qr_roofline": qr_roof, "cpu_baseline": cpu, "e2e": e2e,
                 "gpu_launches": launches_per_call(algo, learned, n) * args.steps, "clocks": sampler.summary(),
@@ -953,7 +959,7 @@ def main_mixed(args, w, rank, world, local, dev, dist, torch, mdx):
         sd = reqs["algo"] == 0
         line = {"metric": METRIC, "value": value, "unit": "requests/s", "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
-                "scaling": "weak", "vs_baseline": None, "dtype": "f32 search, f64 QR and re-scoring",
+                "scaling": "weak", "vs_baseline": None, "dtype": "f32 search, 58-bit fixed-point QR, f64 re-scoring",
                 "data": "synthetic (seeded Rayleigh channels, uniform QAM symbols, AWGN)",
                 "config": config_of(args, w, world), "roofline": roof, "cpu_baseline": cpu, "e2e": e2e,
                 "gpu_launches": (n_runs + 1) * args.steps, "clocks": sampler.summary(), "autotune": tune,
