@@ -43,7 +43,11 @@
  *                                              node budget or MDX_SEQUENTIAL_SEARCH /
  *                                              MDX_NO_RESCORE may search the antennas of a
  *                                              vector in another order, with the same
- *                                              symbols, metrics and status
+ *                                              metrics and status and, unless more
+ *                                              than eight points are within FP32
+ *                                              error of the nearest (which eight are
+ *                                              then compared in FP64 depends on the
+ *                                              order), the same symbols
  *
  * Streams.  `stream` is a cudaStream_t passed as void* (NULL = the legacy
  * default stream).  Device-pointer calls only enqueue work and return; a
@@ -161,7 +165,9 @@ size_t mdx_workspace_bytes(const mdx_ctx* ctx);
  * ybar = Q^H y, both returned in the real interleaved form of size n = 2 n_tx.
  *   R_out    double [batch][n][n], row-major, zero below the diagonal
  *   ybar_out double [batch][n]
- * Complex Householder reflections, to FP64 accuracy or better. */
+ * Complex Householder reflections, with errors of a column's norm at most those of
+ * FP64 arithmetic; channels whose last rows are far below the first are factored in
+ * FP64, which keeps the relative accuracy of such rows. */
 mdx_status mdx_qr(mdx_ctx* ctx, int batch, int n_rx, int n_tx, const double* H, const double* y,
                   double* R_out, double* ybar_out, int flags, void* stream);
 

@@ -8,9 +8,9 @@
 // stages R and sorts with CTA barriers, held one 100x100 vector on an SM of its
 // own.  The master keeps no sorted list either: a pass over the P^d prefixes
 // finds the best one inside the sphere after the last (128 evaluations a lane
-// for 4,096 prefixes, 3 % of a run).  What is left (a sixth of the
-// vectors) goes on in CTAs whose warps take a vector's prefixes in order under a
-// shared radius.
+// for 4,096 prefixes, 3 % of a run).  Four vectors in five have prefixes left after
+// their first runs, one in eight more than 256; they go on in CTAs whose warps take a
+// vector's prefixes in order under a shared radius.
 // Vectors whose candidates tie for the last place kept go to the sorting form.
 //
 // Measured, whole calls with the QR (before: the CTA form for every vector):

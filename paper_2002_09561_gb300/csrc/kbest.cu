@@ -17,7 +17,8 @@
 // too large for register runs, kbest_levels_complex).
 //
 // Hybrid, for what the faster forms (hybrid_warp.cu) leave: K above 64, prefixes
-// of more than four rows, node budgets, ties among the candidates.  The master
+// of more than four rows, node budgets, ties among the candidates, empty spheres and
+// few vectors with statistics.  The master
 // part enumerates every depth-d prefix (rows n-1..n-d), keeps those inside the
 // initial sphere and sorts them by partial distance; the CTA then finishes them
 // best-first, each by a K-best run over the remaining rows under the current

@@ -17,8 +17,8 @@
 // the CTA kernel's operations in the same order: the same bits.
 //
 // Measured (whole calls with the QR, CTA kernel before): 16x16 16-QAM K = 64,
-// 100,000 vectors 19.7 -> 5.5 ms; complex tree 16x16 64-QAM K = 32, 20,000
-// vectors 14.8 -> 2.3 ms; 8x8 64-QAM K = 16 from host memory, 50,000 vectors
+// 100,000 vectors 19.7 -> 5.2 ms; complex tree 16x16 64-QAM K = 32, 20,000
+// vectors 14.8 -> 2.2 ms; 8x8 64-QAM K = 16 from host memory, 50,000 vectors
 // 2.29 -> 1.2 ms.
 #include "select_run.cuh"
 

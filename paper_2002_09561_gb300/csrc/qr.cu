@@ -13,8 +13,8 @@
 // [[Re,-Im],[Im,Re]]) that the tree search uses.
 //
 // Measured (GB300; before: FP64 FMAs and FP64 MMA trailing updates): one 16x16
-// matrix 384 -> 25 us, 100,000 of them 4.02 -> 1.44 ms, 3,000 64x64 7.52 ->
-// 2.15 ms, 4,000 100x100 31.5 -> 10.5 ms; error of R against 64 bits 2.5e-15
+// matrix 384 -> 28 us, 100,000 of them 4.02 -> 1.42 ms, 3,000 64x64 7.52 ->
+// 2.0 ms, 4,000 100x100 31.5 -> 9.9 ms; error of R against 64 bits 2.5e-15
 // -> 1.9e-15 (64x64, of which the reference's own is most).
 #include <algorithm>
 #include <type_traits>
